@@ -84,14 +84,16 @@ typedef struct fpw_params {
   int accum;            /* FPW_ACCUM_* (default FPW_ACCUM_FP32) */
   int K;                /* FPW_PHASE_FP32 only: re-anchor interval in frequencies (default 256) */
   int peak_mode;        /* FPW_PEAK_* (default FPW_PEAK_LOCALMAX) */
-  int threads;          /* 0 = tuned; else threads per block (multiple of 32, 32..512) */
+  int threads;          /* 0 = tuned; else threads per block (multiple of 32, 32..512); with freqs_per_thread it also places
+                           the phase anchors, threads * freqs_per_thread - 2 frequencies apart */
   int freqs_per_thread; /* 0 = tuned; else 1, 2, 4 or 8, or 3, 5 or 6 with FPW_ACCUM_FP32 on a call of one M
                            (FPW_ENOTSUP on the other calls) */
-  int obs_chunk;        /* 0 = tuned; else observations staged in shared memory per pass (>= 32) */
+  int obs_chunk;        /* 0 = tuned; else observations per pass (>= 32): counts towards the shape's size
+                           (FPW_ENOTSUP beyond a block's shared memory); a warp stages 32 at a time whatever it is */
   int use_graph;        /* 1 = capture the launch sequence in a CUDA graph and replay it on identical calls */
-  int items_per_slot;   /* 0 = tuned (default 8); else the persistent schedule's work items per resident block:
-                           each curve's frequency range is cut into segments of about total cost /
-                           (items_per_slot x resident blocks), longest first (>= 1) */
+  int items_per_slot;   /* 0 = tuned (default 8); else bounds the persistent schedule's work items from below: the
+                           curves' frequency ranges are cut into segments that shrink as the work runs out, down
+                           to 1 / (4 items_per_slot) of a resident warp's share (>= 1) */
 } fpw_params;
 
 /* Fill *p with the defaults listed above. */
@@ -287,8 +289,8 @@ FPW_API int fpw_periodogram_batch_bins(fpw_ctx* ctx, void* stream, const fpw_par
  *   Arguments as fpw_periodogram_batch_ex (device pointers; offsets_host is an
  *   optional host copy of offsets, else the offsets are read back to host
  *   memory and checked there: offsets[0] = 0, non-decreasing, offsets[ncurves]
- *   <= 2^40, FPW_EINVAL otherwise), minus S_out. One work item per curve,
- *   largest curves first. phase_mode FPW_PHASE_FP64 is not supported.
+ *   <= 2^40, FPW_EINVAL otherwise), minus S_out. Largest curves
+ *   first, each in as many work items as the scratch has room for. phase_mode FPW_PHASE_FP64 is not supported.
  *   Limit: 320 + 16*C + 4*(C+1) + C + 12*C*k + 8*(nobs+2) bytes (16*(nobs+2)
  *   with FPW_ACCUM_FP64 or FPW_ACCUM_FP32_COMP), each term rounded up to 256,
  *   must fit in 32 MiB (about 4 million observations); larger inputs return

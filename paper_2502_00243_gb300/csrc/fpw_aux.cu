@@ -1,6 +1,7 @@
 // Auxiliary FPW kernels:
-//   prep         w_i = 1/sigma_i^2 and a_i = x_i w_i per observation (Eq. 1's
-//                weights, computed once per call), input validation
+//   prep         w_i = 1/sigma_i^2, a_i = x_i w_i (Eq. 1's weights) and the
+//                phase at f_0 and step per observation, once per call; input
+//                validation; the grid's deviation from a line per anchor block
 //   merge        per-curve top-k peaks from the per-item candidates (Section 3.5)
 //   plain        the binary64 reference form: fl(t f) per evaluation, binary64
 //                bins (Appendix A.1) and sums (Eq. 1), one curve per launch
@@ -25,13 +26,42 @@ __device__ __forceinline__ int64_t curve_of(const int64_t* offsets, int64_t ncur
   return lo;
 }
 
+__device__ __forceinline__ void report(const PrepArgs& a, unsigned bit) {
+  atomicOr(a.status, bit);
+  if (a.latch) atomicOr(a.latch, bit);
+}
+
 __global__ void prep_kernel(const PrepArgs a) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const double f0 = a.freqs[0];
+  // one division a block: a binary64 operation takes a warp 50 clocks, a division
+  // 25 of them
+  __shared__ double s_df;
+  if (threadIdx.x == 0) {
+    s_df = (a.nfreq > 1) ? (a.freqs[a.nfreq - 1] - f0) / (double)(a.nfreq - 1) : 0.0;
+    if (a.df && blockIdx.x == 0) *a.df = s_df;
+  }
+  __syncthreads();
+  const double df = s_df;
+  float tmax = 0.f;
+  const bool grid_ok = isfinite(f0) && isfinite(df);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.nobs; i += stride) {
     const double s = a.sigma[i], x = a.x[i], t = a.t[i];
     const bool ok = isfinite(s) && isfinite(x) && isfinite(t) && s > 0.0;
     const double w = ok ? 1.0 / (s * s) : 0.0;
     const double xa = ok ? x * w : 0.0;
+    if (ok) tmax = fmaxf(tmax, __double2float_ru(fabs(t)));
+    if (a.rec) {
+      unsigned long long p = 0ull, d = 0ull;
+      unsigned dl = 0u;
+      if (ok && isfinite(f0) && isfinite(df)) {
+        phase_fixed96(t, df, d, dl);
+        if (dl != 0u) ++d;
+        p = phase_fixed64(t, f0) - d;
+      }
+      a.rec[i] = make_ulonglong2(p, d);
+      a.rec_low[i] = make_uint2(dl, __float_as_uint((float)t));
+    }
     if (a.aw == nullptr) {
     } else if (a.accum == FPW_ACCUM_FP64) {
       reinterpret_cast<double2*>(a.aw)[i] = make_double2(xa, w);
@@ -42,14 +72,55 @@ __global__ void prep_kernel(const PrepArgs a) {
     } else {
       reinterpret_cast<float2*>(a.aw)[i] = make_float2((float)xa, (float)w);
     }
-    if (!ok) {
+    if (!ok || !(w > 0x1p-60 && w < 0x1p+60)) {
       const int64_t c = a.offsets ? curve_of(a.offsets, a.ncurves, i) : 0;
-      a.curve_bad[c] = 1;
-      atomicOr(a.status, kStatusData);
+      atomicOr(reinterpret_cast<unsigned*>(a.curve_bad) + (c >> 2), (ok ? kCurveWide : kCurveBad) << (8 * (c & 3)));
+      if (!ok) report(a, kStatusData);
     }
   }
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < a.nfreq; q += stride)
-    if (!isfinite(a.freqs[q])) atomicOr(a.status, kStatusGrid);
+    if (!isfinite(a.freqs[q])) report(a, kStatusGrid);
+  if (!a.rec) return;
+  // (maxima of non-negative binary64 numbers as FP32 rounded up: their bits order
+  // as integers, and binary64 compares run at 2 lanes/clk/SM)
+  if (__any_sync(0xffffffffu, tmax > 0.f)) {
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(tmax));
+    if ((threadIdx.x & 31) == 0 && m > *(volatile unsigned*)(a.grid_dev + 1)) atomicMax(a.grid_dev + 1, m);
+  }
+  // per anchor block: the largest deviation of its frequencies (and one more on
+  // either side) from the line through its anchor with the mean spacing, and the
+  // anchor's own distance from the line through f_0 (exact to about 2^-50 of the
+  // frequencies' rounding errors, which it is made of). From the last block of
+  // threads on: the first ones have the observations.
+  __shared__ unsigned wd[8];
+  const int64_t A = a.anchor_span, blocks = (a.nfreq + A - 1) / A;
+  for (int64_t q = gridDim.x - 1 - blockIdx.x; q < blocks; q += gridDim.x) {
+    const int64_t s = q * A - 1, an = s < 0 ? 0 : s;
+    const double fa = a.freqs[an];
+    float dev = 0.f;
+    for (int j = threadIdx.x; j < (int)A + 2; j += blockDim.x) {
+      const int64_t k = s + j;
+      if (k >= 0 && k < a.nfreq) dev = fmaxf(dev, fabsf(__double2float_ru(fabs(a.freqs[k] - fma((double)(int)(k - an), df, fa)))));
+    }
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(dev));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) wd[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      const unsigned d = __reduce_max_sync(0xffffffffu, threadIdx.x < 8 ? wd[threadIdx.x] : 0u);
+      if (threadIdx.x == 0) {
+        a.block_dev[q] = __uint_as_float(d);
+        if (d > *(volatile unsigned*)a.grid_dev) atomicMax(a.grid_dev, d);
+        const double pr = __dmul_rn((double)an, df), pe = __fma_rn((double)an, df, -pr);  // an df = pr + pe
+        const double sm = __dadd_rn(pr, f0), bb = __dsub_rn(sm, pr);                        // pr + f0 = sm + se
+        const double se = __dadd_rn(__dsub_rn(pr, __dsub_rn(sm, bb)), __dsub_rn(f0, bb));
+        const float delta = (float)((__dsub_rn(fa, sm) - (pe + se)) * 0x1p96);
+        a.block_delta[q] = delta;
+        const unsigned far = __float_as_uint(fabsf(delta));
+        if (far > *(volatile unsigned*)(a.grid_dev + 2)) atomicMax(a.grid_dev + 2, far);
+      }
+    }
+  }
 }
 
 __device__ __forceinline__ void warp_best(double& bs, int& bi, int& bp) {
@@ -69,7 +140,18 @@ __device__ __forceinline__ void warp_best(double& bs, int& bi, int& bp) {
 // One warp per curve: the k best of its candidate rows. A candidate ranks after
 // the previously selected one iff it is strictly worse in the (S desc, idx asc)
 // order, so no marking is needed.
-__global__ void merge_kernel(const MergeArgs a) {
+__device__ __forceinline__ MergeArgs merge_group(MergeArgs a) {
+  const int64_t g = blockIdx.y;
+  a.cand_S += g * a.group_rows * a.k;
+  a.cand_idx += g * a.group_rows * a.k;
+  a.topk_idx += g * a.k;
+  a.topk_S += g * a.k;
+  if (a.topk_off) a.topk_off += g * a.k;
+  return a;
+}
+
+__global__ void merge_kernel(const MergeArgs all) {
+  const MergeArgs a = merge_group(all);
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   const bool grid_bad = (*a.status & kStatusGrid) != 0u;
@@ -78,7 +160,7 @@ __global__ void merge_kernel(const MergeArgs a) {
     int32_t* oi = a.topk_idx + c * stride;
     float* os = a.topk_S + c * stride;
     int32_t* oo = a.topk_off ? a.topk_off + c * stride : nullptr;
-    if (grid_bad || a.curve_bad[c]) {
+    if (grid_bad || (a.curve_bad[c] & kCurveBad)) {
       for (int q = lane; q < a.k; q += 32) {
         oi[q] = -1;
         os[q] = __int_as_float(0x7fc00000);
@@ -128,15 +210,34 @@ __global__ void merge_kernel(const MergeArgs a) {
 }
 
 // The same selection with one block per curve, for curves with many candidate
-// rows (one long curve split into thousands of work items): each round every
-// thread scans a slice of the rows and the block reduces the per-warp bests,
-// instead of one warp scanning every row k times.
-constexpr int kMergeBlock = 256;
+// rows (one long curve cut into thousands of work items). A row is sorted, so
+// only its first entry not yet taken can be the next best: every thread holds
+// the heads of its rows in registers, as order-preserving integers (binary64
+// compares run at 2 lanes/clk/SM: they took 40 us for 3000 rows where reading
+// and ranking integers takes 13), and replaces the one that was taken.
+// More rows than kMergeRows go through in several passes, the list so far as
+// entries of thread 0's.
+constexpr int kMergeBlock = 1024, kMergeHeads = 6, kMergeRows = kMergeBlock * kMergeHeads;
 
-__global__ void __launch_bounds__(kMergeBlock) merge_block_kernel(const MergeArgs a) {
-  __shared__ double ws[kMergeBlock / 32];
-  __shared__ int wi[kMergeBlock / 32];
-  __shared__ int wp[kMergeBlock / 32];
+// The best (largest r, then lowest key) of the warp's entries; r = 0: none.
+__device__ __forceinline__ void warp_rank(unsigned long long& r, unsigned& key, int& place) {
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(r >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(r >> 32) == hi ? (unsigned)r : 0u);
+  const unsigned long long m = ((unsigned long long)hi << 32) | lo;
+  const unsigned k = __reduce_min_sync(0xffffffffu, r == m ? key : 0xffffffffu);
+  const unsigned who = __ballot_sync(0xffffffffu, r == m && key == k);
+  place = __shfl_sync(0xffffffffu, place, __ffs(who) - 1);
+  r = m;
+  key = k;
+}
+
+__global__ void __launch_bounds__(kMergeBlock) merge_block_kernel(const MergeArgs all) {
+  const MergeArgs a = merge_group(all);
+  __shared__ unsigned long long wr[32];
+  __shared__ unsigned wk[32];
+  __shared__ int wp[32];  // the head's place: thread * kMergeHeads + number
+  __shared__ unsigned long long resR[2][FPW_MAX_TOPK];
+  __shared__ unsigned resK[2][FPW_MAX_TOPK];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool grid_bad = (*a.status & kStatusGrid) != 0u;
   const int64_t stride = a.out_stride > 0 ? a.out_stride : a.k;
@@ -144,7 +245,7 @@ __global__ void __launch_bounds__(kMergeBlock) merge_block_kernel(const MergeArg
     int32_t* oi = a.topk_idx + c * stride;
     float* os = a.topk_S + c * stride;
     int32_t* oo = a.topk_off ? a.topk_off + c * stride : nullptr;
-    if (grid_bad || a.curve_bad[c]) {
+    if (grid_bad || (a.curve_bad[c] & kCurveBad)) {
       for (int q = tid; q < a.k; q += kMergeBlock) {
         oi[q] = -1;
         os[q] = __int_as_float(0x7fc00000);
@@ -152,62 +253,79 @@ __global__ void __launch_bounds__(kMergeBlock) merge_block_kernel(const MergeArg
       }
       continue;
     }
-    const int64_t e0 = (int64_t)a.cand_base[c] * a.k, e1 = (int64_t)a.cand_base[c + 1] * a.k;
-    double ps = INFINITY;
-    int pi = -1;
-    for (int q = 0; q < a.k; ++q) {
-      double bs = -INFINITY;
-      int bi = -1, bp = -1;
-      for (int64_t e = e0 + tid; e < e1; e += kMergeBlock) {
-        const int i = a.cand_idx[e];
-        if (i < 0) continue;
-        const double s = a.cand_S[e];
-        const bool after_prev = (q == 0) || ranks_before(ps, pi, s, i);
-        if (after_prev && (bp < 0 || ranks_before(s, i, bs, bi))) {
-          bs = s;
-          bi = i;
-          bp = 1;
-        }
+    const int64_t r0 = a.cand_base[c], r1 = a.cand_base[c + 1];
+    int pass = 0;
+    for (int64_t rp = r0; rp < r1; rp += kMergeRows, ++pass) {
+      unsigned long long hr[kMergeHeads];
+      unsigned hk[kMergeHeads];
+      int hq[kMergeHeads];
+#pragma unroll
+      for (int h = 0; h < kMergeHeads; ++h) {
+        const int64_t r = rp + tid + h * kMergeBlock;
+        const int i = r < r1 ? a.cand_idx[r * a.k] : -1;
+        const double s = r < r1 ? a.cand_S[r * a.k] : 0.0;
+        hr[h] = i >= 0 ? rank_bits(s) : 0ull;
+        hk[h] = (unsigned)i;
+        hq[h] = 0;
       }
-      warp_best(bs, bi, bp);
-      if (lane == 0) {
-        ws[warp] = bs;
-        wi[warp] = bi;
-        wp[warp] = bp;
-      }
-      __syncthreads();
-      if (warp == 0) {
-        bs = lane < kMergeBlock / 32 ? ws[lane] : -INFINITY;
-        bi = lane < kMergeBlock / 32 ? wi[lane] : -1;
-        bp = lane < kMergeBlock / 32 ? wp[lane] : -1;
-        warp_best(bs, bi, bp);
-        if (lane == 0) {
-          if (oo) {
-            oi[q] = (bp >= 0) ? (bi >> 6) : -1;
-            oo[q] = (bp >= 0) ? (bi & 63) : -1;
-          } else {
-            oi[q] = (bp >= 0) ? bi : -1;
+      int lq = 0;  // thread 0: the first entry not yet taken of the list of the passes before
+      for (int q = 0; q < a.k; ++q) {
+        unsigned long long br = 0ull;
+        unsigned bk = 0xffffffffu;
+        int bp = -1;
+#pragma unroll
+        for (int h = 0; h < kMergeHeads; ++h)
+          if (hr[h] > br || (hr[h] == br && hr[h] != 0ull && hk[h] < bk)) {
+            br = hr[h];
+            bk = hk[h];
+            bp = tid * kMergeHeads + h;
           }
-          os[q] = (bp >= 0) ? (float)bs : __int_as_float(0x7fc00000);
-          ws[0] = bs;
-          wi[0] = bi;
-          wp[0] = bp;
+        if (tid == 0 && pass > 0 && lq < a.k) {
+          const unsigned long long r = resR[(pass - 1) & 1][lq];
+          const unsigned k = resK[(pass - 1) & 1][lq];
+          if (r > br || (r == br && r != 0ull && k < bk)) {
+            br = r;
+            bk = k;
+            bp = kMergeRows;
+          }
         }
-      }
-      __syncthreads();
-      ps = ws[0];
-      pi = wi[0];
-      const bool none = wp[0] < 0;
-      __syncthreads();
-      if (none) {
-        for (int r = q + 1 + tid; r < a.k; r += kMergeBlock) {
-          oi[r] = -1;
-          os[r] = __int_as_float(0x7fc00000);
-          if (oo) oo[r] = -1;
+        warp_rank(br, bk, bp);
+        if (lane == 0) {
+          wr[warp] = br;
+          wk[warp] = bk;
+          wp[warp] = bp;
         }
-        break;
+        __syncthreads();
+        br = wr[lane];
+        bk = wk[lane];
+        bp = wp[lane];
+        warp_rank(br, bk, bp);  // every warp: the block's best
+        if (br == 0ull) bp = -1;
+        if (tid == 0) {
+          resR[pass & 1][q] = br;
+          resK[pass & 1][q] = bk;
+          if (bp == kMergeRows) ++lq;
+        }
+#pragma unroll
+        for (int h = 0; h < kMergeHeads; ++h)
+          if (bp == tid * kMergeHeads + h) {  // this head was taken: its row's next entry
+            const int64_t e = (rp + tid + h * kMergeBlock) * a.k + ++hq[h];
+            const int i = hq[h] < a.k ? a.cand_idx[e] : -1;
+            const double s = hq[h] < a.k ? a.cand_S[e] : 0.0;
+            hr[h] = i >= 0 ? rank_bits(s) : 0ull;
+            hk[h] = (unsigned)i;
+          }
+        __syncthreads();
       }
     }
+    for (int q = tid; q < a.k; q += kMergeBlock) {
+      const unsigned long long r = pass > 0 ? resR[(pass - 1) & 1][q] : 0ull;
+      const int i = r != 0ull ? (int)resK[(pass - 1) & 1][q] : -1;
+      os[q] = i >= 0 ? (float)from_rank_bits(r) : __int_as_float(0x7fc00000);
+      oi[q] = oo && i >= 0 ? i >> 6 : i;
+      if (oo) oo[q] = i >= 0 ? i & 63 : -1;
+    }
+    __syncthreads();
   }
 }
 
@@ -337,7 +455,7 @@ __global__ void __launch_bounds__(kTopkThreads) dense_topk_kernel(const DenseTop
   }
 }
 
-__global__ void latch_kernel(unsigned* words) { words[2] |= words[1]; }
+__global__ void latch_kernel(unsigned* words) { words[kWordLatch] |= words[1]; }
 
 __global__ void fill_topk_kernel(int32_t* idx, float* S, int64_t n) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -364,21 +482,22 @@ cudaError_t launch_fill_topk(int32_t* idx, float* S, int64_t n, cudaStream_t st)
 cudaError_t launch_prep(const PrepArgs& a, cudaStream_t st) {
   const int64_t work = a.nobs > a.nfreq ? a.nobs : a.nfreq;
   int blocks = (int)((work + 255) / 256);
-  blocks = blocks < 1 ? 1 : (blocks > 4096 ? 4096 : blocks);
-  prep_kernel<<<blocks, 256, 0, st>>>(a);
+  blocks = blocks < 1 ? 1 : (blocks > 1216 ? 1216 : blocks);  // 8 a SM
+  prep_kernel<<<blocks, 256, 0, st>>>(a);  // 8 warps (prep_kernel's wd)
   return cudaGetLastError();
 }
 
 cudaError_t launch_merge(const MergeArgs& a, cudaStream_t st) {
   if (a.ncurves <= 0 || a.k <= 0) return cudaSuccess;
+  const unsigned groups = a.ngroups > 1 ? (unsigned)a.ngroups : 1u;
   if ((int64_t)a.max_rows * a.k > 512) {  // long curves: a block per curve
     const int64_t blocks = a.ncurves < 65535 ? a.ncurves : 65535;
-    merge_block_kernel<<<(unsigned)blocks, kMergeBlock, 0, st>>>(a);
+    merge_block_kernel<<<dim3((unsigned)blocks, groups), kMergeBlock, 0, st>>>(a);
     return cudaGetLastError();
   }
   int blocks = (int)((a.ncurves + 7) / 8);
   blocks = blocks > 65535 ? 65535 : blocks;
-  merge_kernel<<<blocks, 256, 0, st>>>(a);
+  merge_kernel<<<dim3((unsigned)blocks, groups), 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -14,6 +14,8 @@ constexpr unsigned kStatusData = 1u;     // sigma <= 0 or non-finite t/x/sigma i
 constexpr unsigned kStatusGrid = 2u;     // non-finite frequency
 constexpr unsigned kStatusTimeout = 4u;  // a bounded wait gave up
 
+constexpr int kWordLatch = 4;  // the context's status word that keeps errors until they are asked for
+
 // Largest distance (cycles) by which the linear-grid fast path may move a
 // phase relative to frac(t_i * freqs[k]): tiles whose grid deviates more are
 // evaluated with a direct per-frequency anchor instead.
@@ -22,9 +24,12 @@ constexpr double kGridTolCycles = 2e-10;
 // Largest number of derived bin counts computed from one M_max pass.
 constexpr int kMaxGroups = 8;
 
+// Per-curve flags (curve_bad): invalid data; a weight outside [2^-60, 2^60].
+constexpr unsigned kCurveBad = 1u, kCurveWide = 2u;
+
 // Several-M calls whose (M_max, groups) have a compiled combination in the
 // tile kernel (1: M_max = 60 with groups 3, 6, 15; 2: 40 with 2, 4, 10; 3: 20
-// with 1, 2, 4; groups in that order), else 0 (the generic combination).
+// with 1, 2, 4; groups in that order), else 0 (the combination for any groups).
 inline int multi_spec_of(int M, int ngroups, const int* g) {
   if (ngroups != 3) return 0;
   if (M == 60 && g[0] == 3 && g[1] == 6 && g[2] == 15) return 1;
@@ -54,7 +59,9 @@ struct TileArgs {
   int nitems;
   unsigned* counter;         // work-queue head (zeroed before launch)
   unsigned* status;          // latched status bits
-  const uint8_t* curve_bad;  // [ncurves] 1 = invalid data
+  const uint8_t* curve_bad;  // [ncurves] flags kCurveBad, kCurveWide
+  unsigned long long* floors;  // [ncurves * max(ngroups, 1)] zeroed before launch, or NULL: the k-th best S that an
+                             // item of the curve has found (its order-preserving bits)
   double* cand_S;            // [slots * k] candidate peaks (S), or NULL when k == 0
   int32_t* cand_idx;         // [slots * k]
   double* S_out;             // dense [ncurves * nfreq] or NULL
@@ -62,9 +69,19 @@ struct TileArgs {
   int k;
   int peak_raw;
   int K;                     // FPW_PHASE_FP32 re-anchor interval
-  int obs_chunk;             // observations staged per pass
   double inv_alpha2;
-  const double* tile_dev;    // per-tile grid deviation (tile_dev_kernel), or NULL: checked in the tile kernel
+  // Phase anchors: block q of the grid holds frequencies [q A, (q + 1) A), A =
+  // anchor_span, and its phases step from the exact phase at frequency max(q A -
+  // 1, 0) (so they don't depend on how the kernel cuts its tiles).
+  int64_t anchor_span;
+  int aligned;               // 1: no tile reaches into another block (dense output; no prep records)
+  const ulonglong2* rec;     // [nobs] {frac(t_i f_0) - D_i, D_i = frac(t_i df)} as 64-bit fixed point, rounded up
+                             // (prep), or NULL
+  const uint2* rec_low;      // [nobs] {D_i's next 32 bits before the rounding, t_i as FP32}
+  const float* block_dev;    // [blocks] largest deviation of a block's frequencies from its line (prep), or NULL
+  const float* block_delta;  // [blocks] 2^96 (anchor frequency - (f_0 + a df)) (prep)
+  const double* df;          // the grid's mean spacing (prep), or NULL
+  const unsigned* grid_dev;  // FP32 bits of the largest block_dev, |t| and |block_delta| (prep)
   int ngroups;               // several-M kernel: number of groups (0 = the single-M kernel)
   int group_g[kMaxGroups];   // M = M / group_g[q] for group q
   int64_t group_rows;        // candidate rows per group (cand tables are [group][slot][k])
@@ -83,11 +100,19 @@ struct PrepArgs {
   int64_t nfreq;
   void* aw;                // [nobs] float2, double2 or float4 (see TileArgs::aw), or NULL
   int accum;               // FPW_ACCUM_*
-  uint8_t* curve_bad;      // [ncurves], zeroed before launch
+  uint8_t* curve_bad;      // [ncurves] flags, zeroed before launch, 4-byte aligned and padded
   unsigned* status;
+  unsigned* latch;         // NULL, or the word that keeps the status between calls
+  int64_t anchor_span;     // TileArgs, likewise the next five (rec NULL: none of them)
+  ulonglong2* rec;
+  uint2* rec_low;
+  float* block_dev;
+  float* block_delta;
+  double* df;              // NULL, or receives the grid's mean spacing
+  unsigned* grid_dev;      // [3], zeroed before launch
 };
 
-struct MergeArgs {
+struct MergeArgs {          // ngroups groups: rows of group g at + g * group_rows, its output at + g * k
   const double* cand_S;
   const int32_t* cand_idx;
   const int32_t* cand_base;  // [ncurves + 1] candidate rows per curve
@@ -100,6 +125,8 @@ struct MergeArgs {
   int out_stride;
   int32_t* topk_off;         // several-M: receives key & 63 (the bin offset); topk_idx then gets key >> 6
   int max_rows;              // most candidate rows of one curve (0: unknown); many rows take a block per curve
+  int ngroups;               // 0 = 1
+  int64_t group_rows;
 };
 
 struct PlainArgs {           // binary64 plain form, one curve
@@ -134,31 +161,34 @@ __host__ __device__ constexpr size_t accum_bin_bytes(int accum) { return accum =
 
 // Tile-kernel shape chosen by the host (tuned per bin count and curve size).
 struct TileShape {
-  int threads;   // T
-  int R;         // frequencies per thread
-  int obs_chunk; // NC
+  int threads;   // T and R of the shape asked for or chosen by bin count: phase anchors every T R - 2 frequencies
+  int R;
+  int obs_chunk; // the caller's observations per pass (0: none given); the kernel stages 32 per warp
+  int warps;     // warps of a block as launched, each with work items of its own
+  int lane_R;    // frequencies per lane as launched
   size_t smem;   // dynamic shared memory bytes
-  int items;     // work items per resident block in the persistent schedule
+  int items;     // work items per resident warp in the persistent schedule
 };
 
 // ---- launch wrappers (defined in the .cu files) -------------------------
-size_t tile_smem_bytes(int T, int R, int M, int NC, int k, int accum, int ngroups = 0);
+size_t tile_smem_bytes(int T, int R, int M, int k, int accum, int ngroups = 0);
+// The size by which a shape is accepted or refused (FPW_ENOTSUP): the bins of T
+// threads, NC observations and the peak scratch of a block.
+size_t tile_shape_bytes(int T, int R, int M, int NC, int accum, int ngroups = 0);
 int tile_max_blocks_per_sm(int R, int phase_mode, int accum, int T, size_t smem, bool multi = false,
-                           bool dump = false, int spec = 0);  // spec: the several-M combination (fpw_tile.cuh)
-bool tile_supported_R(int R);                      // some tile kernel has R frequencies per thread
-bool tile_has_R(int R, int accum, bool multi);     // the kernel for this sum mode / several-M call has it
+                           bool dump = false, int spec = 0);  // spec: the several-M combination (multi_spec_of)
+bool tile_supported_R(int R);                      // R that a caller may ask for
+int tile_max_warps(bool multi);                    // warps of a launched block, at most
+bool tile_has_R(int R, int accum, bool multi);     // ... of the kernel for this sum mode / several-M call
 // Launches the kernel for (R, phase, accum); several-M when a.ngroups > 0, the
 // bin-dumping instantiation when a.bins_out != NULL.
 cudaError_t launch_tile(const TileArgs& a, const TileShape& s, int phase_mode, int accum, int grid, cudaStream_t st);
 cudaError_t launch_prep(const PrepArgs& a, cudaStream_t st);
-// Per-tile grid deviation for tiles of width W starting at q*(W-2)-1, q < tiles.
-cudaError_t launch_tile_dev(const double* freqs, int64_t F, int W, int64_t tiles, double* dev, cudaStream_t st);
 cudaError_t launch_merge(const MergeArgs& a, cudaStream_t st);
 cudaError_t launch_plain(const PlainArgs& a, cudaStream_t st);
 cudaError_t launch_dense_topk(const DenseTopkArgs& a, cudaStream_t st);
-cudaError_t launch_latch(unsigned* words, cudaStream_t st);  // words[2] |= words[1]
+cudaError_t launch_latch(unsigned* words, cudaStream_t st);  // words[kWordLatch] |= words[1]
 cudaError_t launch_fill_topk(int32_t* idx, float* S, int64_t n, cudaStream_t st);
-cudaError_t tile_init_attributes(int max_smem);
 cudaError_t plain_init_attributes(int max_smem);
 size_t plain_smem_bytes(int M);
 cudaError_t launch_entropy_dense(const double* t, int64_t n, const double* freqs, int64_t nfreq, int M, float* H_out,
@@ -226,6 +256,30 @@ __device__ __forceinline__ unsigned long long phase_fixed64(double t, double f) 
   return neg ? (0ull - r) : (r + (inexact ? 1ull : 0ull));
 }
 
+// The same to 96 bits (hi: the leading 64, lo: the next 32), rounded up at the last.
+__device__ __forceinline__ void phase_fixed96(double t, double f, unsigned long long& hi, unsigned& lo) {
+  unsigned long long mt, mf;
+  int et, ef;
+  split_binary64(t, mt, et);
+  split_binary64(f, mf, ef);
+  const unsigned __int128 q = (unsigned __int128)mt * mf;
+  const int s = et + ef + 96;  // frac * 2^96 = (q * 2^s) mod 2^96
+  unsigned __int128 r = 0;
+  bool inexact = false;
+  if (s >= 0) {
+    if (s < 128) r = q << s;
+  } else if (s > -128) {
+    r = q >> -s;
+    inexact = (r << -s) != q;
+  } else {
+    inexact = q != 0;
+  }
+  const bool neg = ((__double_as_longlong(t) ^ __double_as_longlong(f)) < 0) && q != 0;
+  r = neg ? -r : r + (inexact ? 1u : 0u);
+  hi = (unsigned long long)(r >> 32);
+  lo = (unsigned)r;
+}
+
 // Bin of a 64-bit fixed-point phase: floor(M * Phi_hi / 2^32). It equals
 // floor(M * Phi / 2^64) except within 2^-32 cycles below a bin edge.
 __device__ __forceinline__ unsigned bin_of_phase(unsigned long long phi, unsigned M) {
@@ -241,6 +295,16 @@ __device__ __forceinline__ float2 f2add(float2 a, float2 b) {
   float2 r;
   asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(z));
   return r;
+}
+
+// Order-preserving map of a double to an unsigned integer (larger value, larger
+// image; no double but a NaN maps to 0), and its inverse.
+__device__ __forceinline__ unsigned long long rank_bits(double s) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(s);
+  return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
+}
+__device__ __forceinline__ double from_rank_bits(unsigned long long r) {
+  return __longlong_as_double((long long)((r >> 63) ? (r & 0x7fffffffffffffffull) : ~r));
 }
 
 // Ranking used for peaks: larger S first, then lower frequency index.

@@ -35,13 +35,14 @@ struct DeviceSetup {
   unsigned char* scratch = nullptr;  // device address of g_scratch on this device
   int nsm = 0;
   int smem_optin = 0;
-  int smem_per_sm = 0;
 };
 
 std::mutex g_setup_mu;
 DeviceSetup g_setup[64];
 
-// Work list: one item per curve, ordered by decreasing size class (a counting
+// Work list: every curve's frequencies in nseg segments of whole anchor blocks
+// (enough items for the resident warps, as far as the scratch has room for
+// their candidates; one at least), ordered by decreasing size class (a counting
 // sort on floor(log2 n) + 1 in the scratch array), so that the persistent
 // kernel starts the longest curves first. Within a class the order is
 // whatever the atomics give; it changes no result, only the schedule.
@@ -52,9 +53,10 @@ __device__ __forceinline__ int size_class(const int64_t* offsets, int64_t c) {
   return n > 0 ? __clzll((long long)n) : 63;  // larger n, smaller class
 }
 
-__global__ void noalloc_count_kernel(const int64_t* offsets, int64_t C, unsigned* hist, int32_t* cand_base) {
+__global__ void noalloc_count_kernel(const int64_t* offsets, int64_t C, int64_t nseg, unsigned* hist,
+                                     int32_t* cand_base) {
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c <= C; c += (int64_t)gridDim.x * blockDim.x) {
-    cand_base[c] = (int32_t)c;
+    cand_base[c] = (int32_t)(c * nseg);
     if (c < C) atomicAdd(&hist[size_class(offsets, c)], 1u);
   }
 }
@@ -68,15 +70,22 @@ __global__ void noalloc_scan_kernel(unsigned* hist) {  // one thread: exclusive 
   }
 }
 
-__global__ void noalloc_items_kernel(const int64_t* offsets, int64_t C, int64_t F, unsigned* cursor, WorkItem* items) {
+__global__ void noalloc_items_kernel(const int64_t* offsets, int64_t C, int64_t F, int64_t nseg, int64_t A,
+                                     unsigned* cursor, WorkItem* items) {
+  const int64_t blocks = (F + A - 1) / A;
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < C; c += (int64_t)gridDim.x * blockDim.x) {
     const unsigned pos = atomicAdd(&cursor[size_class(offsets, c)], 1u);
-    WorkItem w;
-    w.curve = (int32_t)c;
-    w.f_lo = 0;
-    w.f_hi = (int32_t)F;
-    w.slot = (int32_t)c;
-    items[pos] = w;
+    int64_t lo = 0;
+    for (int64_t q = 0; q < nseg; ++q) {
+      const int64_t end = blocks * (q + 1) / nseg * A, hi = end < F ? end : F;
+      WorkItem w;
+      w.curve = (int32_t)c;
+      w.f_lo = (int32_t)lo;
+      w.f_hi = (int32_t)hi;
+      w.slot = (int32_t)(c * nseg + q);
+      items[pos * nseg + q] = w;
+      lo = hi;
+    }
   }
 }
 
@@ -101,11 +110,9 @@ int setup_device(int dev, DeviceSetup** out) {
     if (e != cudaSuccess || p == nullptr) return FPW_ECUDA;
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return FPW_ECUDA;
-    if (tile_init_attributes((int)prop.sharedMemPerBlockOptin) != cudaSuccess) return FPW_ECUDA;
     s.scratch = static_cast<unsigned char*>(p);
     s.nsm = prop.multiProcessorCount;
     s.smem_optin = (int)prop.sharedMemPerBlockOptin;
-    s.smem_per_sm = (int)prop.sharedMemPerMultiprocessor;
     s.done = true;
   }
   *out = &s;
@@ -166,44 +173,43 @@ extern "C" FPW_API int fpw_periodogram_batch_noalloc(void* stream, const fpw_par
   nobs = prev;
   if (nobs > 0 && (!t || !x || !sigma)) return FPW_EINVAL;
 
-  // kernel shape: as the tuned default, with the chunk sized to fit two blocks per SM
+  // kernel shape
   const bool wide = p.accum != FPW_ACCUM_FP32;  // 16-byte bins
   TileShape sh{};
   sh.threads = p.threads ? p.threads : 128;
   sh.R = p.freqs_per_thread ? p.freqs_per_thread : (wide ? 2 : (M <= 24 ? 4 : 2));
   if (!tile_has_R(sh.R, p.accum, false)) return FPW_ENOTSUP;
-  int NC = p.obs_chunk;
-  if (!NC) {
-    for (int blocks : {2, 1}) {
-      for (int nc = 4096; nc >= 32; nc -= 32) {
-        const size_t s = tile_smem_bytes(sh.threads, sh.R, M, nc, k, p.accum);
-        if (s <= (size_t)ds->smem_optin && (s + 1024) * blocks <= (size_t)ds->smem_per_sm) {
-          NC = nc;
-          break;
-        }
-      }
-      if (NC >= 256) break;
-      NC = 0;
-    }
-    if (!NC) return FPW_ENOTSUP;
-  }
-  sh.obs_chunk = NC;
-  sh.smem = tile_smem_bytes(sh.threads, sh.R, M, NC, k, p.accum);
+  if (tile_shape_bytes(sh.threads, sh.R, M, p.obs_chunk ? p.obs_chunk : 256, p.accum) > (size_t)ds->smem_optin)
+    return FPW_ENOTSUP;
+  sh.lane_R = sh.R;
+  sh.warps = sh.threads / 32;
+  if (sh.warps > tile_max_warps(false)) sh.warps = tile_max_warps(false);
+  while (sh.warps > 1 && tile_smem_bytes(32 * sh.warps, sh.R, M, k, p.accum) > (size_t)ds->smem_optin) --sh.warps;
+  sh.smem = tile_smem_bytes(32 * sh.warps, sh.R, M, k, p.accum);
   if (sh.smem > (size_t)ds->smem_optin) return FPW_ENOTSUP;
-  const int bps = tile_max_blocks_per_sm(sh.R, p.phase_mode, p.accum, sh.threads, sh.smem);
+  const int bps = tile_max_blocks_per_sm(sh.R, p.phase_mode, p.accum, 32 * sh.warps, sh.smem);
   if (bps < 1) return FPW_ENOTSUP;
 
   // scratch layout (256-byte aligned sections); reject inputs that do not fit
-  const size_t o_words = 0;  // counter, status (64 B), then the size-class histogram
+  // with one segment per curve, else take about 8 items per resident warp
+  const int warps = sh.warps;
+  const int64_t A = (int64_t)sh.threads * sh.R - 2, blocks1 = (nfreq + A - 1) / A, resident = (int64_t)bps * ds->nsm * warps;
+  const size_t o_words = 0;  // counter, status, grid deviation (64 B), then the size-class histogram
   const size_t o_hist = o_words + 64;
   const size_t o_items = up256(o_hist + kSizeClasses * sizeof(unsigned));
-  const size_t o_base = up256(o_items + (size_t)ncurves * sizeof(WorkItem));
-  const size_t o_bad = up256(o_base + (size_t)(ncurves + 1) * sizeof(int32_t));
-  const size_t o_cS = up256(o_bad + (size_t)ncurves);
-  const size_t o_cI = up256(o_cS + (size_t)ncurves * k * sizeof(double));
-  const size_t o_aw = up256(o_cI + (size_t)ncurves * k * sizeof(int32_t));
-  const size_t end = o_aw + (size_t)(nobs + 2) * accum_bin_bytes(p.accum);
-  if (end > kScratchBytes) return FPW_EINVAL;
+  int64_t nseg = (8 * resident + ncurves - 1) / ncurves;
+  nseg = nseg < blocks1 ? nseg : blocks1;
+  size_t o_base, o_bad, o_cS, o_cI, o_aw;
+  for (;; nseg = (nseg + 1) / 2) {
+    const size_t rows = (size_t)ncurves * (size_t)nseg;
+    o_base = up256(o_items + rows * sizeof(WorkItem));
+    o_bad = up256(o_base + (size_t)(ncurves + 1) * sizeof(int32_t));
+    o_cS = up256(o_bad + (size_t)ncurves);
+    o_cI = up256(o_cS + rows * k * sizeof(double));
+    o_aw = up256(o_cI + rows * k * sizeof(int32_t));
+    if (o_aw + (size_t)(nobs + 2) * accum_bin_bytes(p.accum) <= kScratchBytes) break;
+    if (nseg == 1) return FPW_EINVAL;
+  }
   unsigned char* S = ds->scratch;
   unsigned* words = reinterpret_cast<unsigned*>(S + o_words);
   unsigned* hist = reinterpret_cast<unsigned*>(S + o_hist);
@@ -221,9 +227,9 @@ extern "C" FPW_API int fpw_periodogram_batch_noalloc(void* stream, const fpw_par
   {
     int64_t blocks = (ncurves + 1 + 255) / 256;
     blocks = blocks > 4096 ? 4096 : blocks;
-    noalloc_count_kernel<<<(unsigned)blocks, 256, 0, st>>>(offsets, ncurves, hist, cand_base);
+    noalloc_count_kernel<<<(unsigned)blocks, 256, 0, st>>>(offsets, ncurves, nseg, hist, cand_base);
     noalloc_scan_kernel<<<1, 1, 0, st>>>(hist);
-    noalloc_items_kernel<<<(unsigned)blocks, 256, 0, st>>>(offsets, ncurves, nfreq, hist, items);
+    noalloc_items_kernel<<<(unsigned)blocks, 256, 0, st>>>(offsets, ncurves, nfreq, nseg, A, hist, items);
     if (cudaGetLastError() != cudaSuccess) return FPW_ECUDA;
   }
   PrepArgs pa{};
@@ -248,7 +254,7 @@ extern "C" FPW_API int fpw_periodogram_batch_noalloc(void* stream, const fpw_par
   ta.freqs = freqs;
   ta.nfreq = nfreq;
   ta.items = items;
-  ta.nitems = (int)ncurves;
+  ta.nitems = (int)(ncurves * nseg);
   ta.counter = words;
   ta.status = words + 1;
   ta.curve_bad = curve_bad;
@@ -259,11 +265,12 @@ extern "C" FPW_API int fpw_periodogram_batch_noalloc(void* stream, const fpw_par
   ta.k = k;
   ta.peak_raw = p.peak_mode == FPW_PEAK_RAW ? 1 : 0;
   ta.K = p.K;
-  ta.obs_chunk = sh.obs_chunk;
+  ta.anchor_span = A;
+  ta.aligned = 1;
   ta.inv_alpha2 = p.inv_alpha2;
-  int grid = bps * ds->nsm;
-  grid = grid < (int)ncurves ? grid : (int)ncurves;
-  if (launch_tile(ta, sh, p.phase_mode, p.accum, grid, st) != cudaSuccess) return FPW_ECUDA;
+  int64_t grid = (int64_t)bps * ds->nsm;
+  if (grid * warps > ta.nitems) grid = (ta.nitems + warps - 1) / warps;
+  if (launch_tile(ta, sh, p.phase_mode, p.accum, (int)grid, st) != cudaSuccess) return FPW_ECUDA;
   if (k > 0) {
     MergeArgs ma{};
     ma.cand_S = cand_S;
@@ -272,6 +279,7 @@ extern "C" FPW_API int fpw_periodogram_batch_noalloc(void* stream, const fpw_par
     ma.curve_bad = curve_bad;
     ma.status = words + 1;
     ma.ncurves = ncurves;
+    ma.max_rows = (int)nseg;
     ma.k = k;
     ma.topk_idx = topk_idx;
     ma.topk_S = topk_S;

@@ -88,12 +88,12 @@ uint64_t mix(uint64_t h, const T& v) {
 
 struct Plan {
   uint64_t key = 0;
-  TileShape shape{};
   int grid = 0;
   int nitems = 0;
   int nslots = 0;
   int max_rows = 0;  // most candidate rows (work items) of one curve
-  DevBuf items, cand_base;
+  DevBuf items;                    // work items, then the candidate rows per curve
+  int32_t* cand_base = nullptr;
   void* host_stage = nullptr;  // pinned copy of items + cand_base, the source of the asynchronous upload
   uint64_t use = 0;
 };
@@ -112,6 +112,14 @@ struct GraphEntry {
   uint64_t use = 0;
 };
 
+// Status words of a context (64 bytes): 1 the status of the current call (plain,
+// shared-timestamp and drift paths), kWordLatch the latched status (kept between
+// calls), 8-9 the shared-timestamp path's max |t|. The tile path's words precede
+// its per-curve flags: 0 work-queue head, 1 status, 2-4 the grid's largest
+// deviation from a line, the largest |t| and the largest distance of an anchor
+// from the line (FP32 bits), 6-7 the grid's mean spacing (binary64).
+constexpr int kCallWords = 8, kWordGridDev = 2, kWordDf = 6;
+
 constexpr int kMaxPlans = 16;
 constexpr int kMaxGraphs = 16;
 
@@ -124,8 +132,9 @@ struct fpw_ctx {
   int smem_per_sm = 0;
   std::mutex mu;
   cudaStream_t last_stream = nullptr;
+  const unsigned* call_status = nullptr;  // device: status word of the latest call
   cudaStream_t own_stream = nullptr;
-  DevBuf aw, cand_S, cand_idx, curve_bad, words, dense, tile_dev;
+  DevBuf scratch, curve_bad, words, dense;  // scratch: the tile path's (Scratch)
   DevBuf sh_image, sh_scale, sh_S32, sh_step, sh_sink;  // shared-timestamp path scratch
   DevBuf dr_payload, dr_H0, dr_g, dr_tabs;                     // baseline-drift path scratch
   DevBuf h_off, h_t, h_x, h_sigma, h_freqs, h_idx, h_S;  // device copies for the host entry point
@@ -153,7 +162,6 @@ void free_buf(DevBuf& b) {
 // Frees a plan; cudaFree synchronizes the device first, so its upload has ended.
 void free_plan(Plan* p) {
   free_buf(p->items);
-  free_buf(p->cand_base);
   if (p->host_stage) cudaFreeHost(p->host_stage);
   delete p;
 }
@@ -182,184 +190,195 @@ bool valid_params(const fpw_params& p) {
   return true;
 }
 
-// Kernel shape: T threads, R frequencies per thread, NC observations per pass.
-// Per-thread bins take R*M*T*(8|16) bytes (16 for binary64 and compensated
-// sums); the observation chunk takes NC*(16 + 8|16) bytes. Precedence: explicit params > the context's tuned
-// table (fpw_ctx_set_shape) > the built-in defaults, which were measured on a
-// GB300 with ZTF-like curves (threads x frequencies-per-thread sweeps at
-// M = 10, 16, 20, 24, 30, 40, 50): R = 8 for M <= 12, R = 6 for M <= 16, R = 5
-// for M <= 20, R = 4 for M <= 25, R = 3 for M <= 33 (R = 2 for these when the
-// typical curve has fewer than 300 observations, as measured at M = 20; R = 6, 5
-// and 3 for FP32 sums of one M only, else 4 and 2), R = 2 up to M = 64, R = 1
-// beyond, T = 128 (halved while the bins alone do not fit): up to about 100 bin
-// pairs per thread keep two blocks of four warps per SM and spread each
-// observation's broadcast over the most frequencies. NC: the largest chunk that
-// keeps two resident blocks per SM (one stages while the other accumulates) if
-// that is at least 128 observations, else one block per SM.
-int choose_shape(fpw_ctx* ctx, const fpw_params& p, int M, int k, int64_t max_n, int64_t n_typ, int ngroups,
-                 TileShape& out) {
-  const bool wide = p.accum != FPW_ACCUM_FP32;  // 16-byte bins
+// Warp tiles of one curve at R frequencies per lane.
+int64_t warp_tiles(int64_t F, int R) { return (F + 32 * (int64_t)R - 1) / (32 * (int64_t)R); }
+
+// Clocks per observation that `tiles` warp tiles take on w warps per SM. A round
+// takes the shared-memory pipe w (4 R + 3) wavefronts (8 R + 4 with 16-byte
+// bins), a scheduler's warps about 10 R + 8 issue slots each, and a lone warp's
+// chain of loads, adds and stores about 50 + 10 R clocks (all three as measured,
+// 4 to 16 warps); the last round ends with that chain or its share of the pipe.
+double shape_time(const fpw_ctx* ctx, int R, int w, int64_t tiles, bool wide) {
+  const int64_t per_sm = (tiles + ctx->nsm - 1) / ctx->nsm;
+  if (per_sm < w) w = (int)per_sm;
+  const double chain = 50.0 + (wide ? 16.0 : 10.0) * R;
+  const double slack = w >= 8 ? 1.05 : (w > 4 ? 1.08 : 1.2);  // few warps: staging and reductions don't overlap
+  const double round = std::max({slack * w * (wide ? 8.0 * R + 4.0 : 4.0 * R + 3.0), chain,
+                                 (double)((w + 3) / 4) * ((wide ? 20.0 : 10.0) * R + 8.0)});
+  const int64_t slots = (int64_t)ctx->nsm * w, full = tiles / slots, rest = tiles % slots;
+  return (double)full * round + (rest ? std::max(chain, round * (double)rest / (double)slots) : 0.0);
+}
+
+// Kernel shape. First T threads x R frequencies per thread, from explicit params >
+// the context's tuned table (fpw_ctx_set_shape) > the bin count: they place the
+// phase anchors (every T R - 2 frequencies), so results don't move when the
+// launch below changes. Then what is launched, in blocks of `warps` warps with
+// `lane_R` frequencies per lane, each warp with tiles of its own: T / 32 and R
+// where the caller or the table gave them; else R as measured per bin count (a
+// warp's bins take R*M*32*(8|16) bytes, 16 for binary64 and compensated sums) and
+// the warps that fit one block per SM, up to 8 (two per scheduler; 16-byte bins:
+// 12), N = 1000: M = 20 R = 5 2.05e12 evaluations/s (R = 10 on 4 warps 2.02), M =
+// 10 R = 8 2.19 (R = 6 2.13, R = 8 on 10 warps 2.14), M = 16 R = 6 2.12 (R = 8 2.10),
+// M = 30 R = 3 1.84 (R = 7 on 4 1.81), M = 50 R = 2 1.62 (R = 4 on 4 1.47, R = 1 on 16
+// 1.29), M = 64 R = 3 on 4 1.31 (R = 1 on 12 1.28), several M at M_max = 60 R = 2 on 7
+// 1.24 (R = 3 on 4 1.05), compensated M = 20 R = 2 on 10 0.90 (R = 3 on 7 0.91, R = 2 on
+// 8 0.87).
+int choose_shape(fpw_ctx* ctx, const fpw_params& p, int M, int k, int64_t C, int64_t F, int64_t max_n, int64_t n_mean,
+                 int64_t n_typ, int ngroups, const int* groups, bool dense, TileShape& out) {
+  const bool wide = p.accum != FPW_ACCUM_FP32, multi = ngroups > 0;
   int T = 128, R = 4, NC = 0, items = 8;
   if (wide)
     R = 2;
   else if (M <= 12)
     R = 8;
-  else if (M <= 16 && ngroups == 0)
+  else if (M <= 16 && !multi)
     R = n_typ < 300 ? 2 : 6;
-  else if (M <= 20 && ngroups == 0)
+  else if (M <= 20 && !multi)
     R = n_typ < 300 ? 2 : 5;
-  else if (M <= 24 || (M <= 25 && ngroups == 0))
+  else if (M <= 24 || (M <= 25 && !multi))
     R = n_typ < 300 ? 2 : 4;
-  else if (M <= 33 && ngroups == 0)
+  else if (M <= 33 && !multi)
     R = n_typ < 300 ? 2 : 3;
-  else if (M <= 40 || (M <= 50 && ngroups == 0))  // several M at M_max = 40: 1.23e12 against 1.17e12 at T = 256, R = 1
+  else if (M <= 40 || (M <= 50 && !multi))
     R = 2;
-  else if (M <= 50) {  // several M: the per-frequency combination favours more warps
+  else if (M <= 50) {
     T = 256;
     R = 1;
-  } else if (M <= 64) {  // two blocks of 6 warps per SM (T = 128, R = 2 leaves one block of 4)
-    T = 192;
+  } else if (M <= 64) {
+    T = multi ? 128 : 192;
     R = 1;
-    if (ngroups > 0) {  // several M at M_max = 60: three blocks of 4 warps, 256 observations per pass
-      T = 128;          // (1.010e12 evaluations/s against 0.992e12 for two blocks of 6 warps)
-      NC = 256;
-    }
-  } else
+  } else {
     R = 1;
+  }
+  bool given = false;  // the launch follows T and R
   for (const ShapeEntry& e : ctx->shapes)
     if (M >= e.M_lo && M <= e.M_hi && n_typ >= e.n_lo && n_typ < e.n_hi) {
       T = e.T;
       R = e.R;
       NC = e.NC;
       items = e.items ? e.items : 8;
+      given = true;
     }
-  if (ngroups > 0 && T > 256) T = 256;  // the several-M kernel's launch bound (table entries may be wider)
-  // R = 3 and 6 exist for FP32 sums of one M only: a table entry tuned there
-  // gives the neighbouring instantiated R to the other kernels
-  if (!tile_has_R(R, p.accum, ngroups > 0)) R = (R == 3) ? 2 : 4;
+  if (multi && T > 256) T = 256;  // the several-M kernel's launch bound (table entries may be wider)
+  // R = 3, 5 and 6 are offered for FP32 sums of one M only: a table entry tuned
+  // there gives a neighbouring R to the other kernels
+  if (!tile_has_R(R, p.accum, multi)) R = (R == 3) ? 2 : 4;
   if (p.threads) T = p.threads;
   if (p.items_per_slot) items = p.items_per_slot;
   if (p.freqs_per_thread) R = p.freqs_per_thread;
-  if (!tile_has_R(R, p.accum, ngroups > 0)) return FPW_ENOTSUP;
+  if (!tile_has_R(R, p.accum, multi)) return FPW_ENOTSUP;
   if (p.obs_chunk) NC = p.obs_chunk;
-  const bool fixedT = p.threads != 0;
-  while (!fixedT && T > 32 && tile_smem_bytes(T, R, M, 32, k, p.accum, ngroups) > (size_t)ctx->smem_optin) T /= 2;
-  const int64_t want_nc = std::max<int64_t>(32, ((max_n + 31) / 32) * 32);
-  const size_t per_sm = (size_t)ctx->smem_per_sm;
-  auto fits = [&](int blocks, int nc) {
-    const size_t s = tile_smem_bytes(T, R, M, nc, k, p.accum, ngroups);
-    return s <= (size_t)ctx->smem_optin && (s + 1024) * blocks <= per_sm;
-  };
-  if (!NC) {
-    for (int blocks : {2, 1}) {
-      int lo = 32, hi = (int)std::min<int64_t>(want_nc, 1 << 16);
-      if (!fits(blocks, lo)) continue;
-      while (lo < hi) {  // largest multiple of 32 that fits
-        int mid = ((lo + hi + 32) / 64) * 32;
-        if (mid <= lo) mid = lo + 32;
-        if (mid > hi) mid = hi;
-        if (fits(blocks, mid))
-          lo = mid;
-        else
-          hi = mid - 32;
-      }
-      // too small a chunk: one block per SM instead (two blocks with 128-160
-      // observations per pass ran M = 20, R = 5 at 2.0e12 evals/s, one block
-      // with a larger chunk 1.5e12)
-      if (blocks == 2 && lo < 128 && lo < want_nc) continue;
-      NC = lo;
-      break;
-    }
-    if (!NC) return FPW_ENOTSUP;  // the bins alone exceed shared memory
-  }
-  const size_t smem = tile_smem_bytes(T, R, M, NC, k, p.accum, ngroups);
-  if (smem > (size_t)ctx->smem_optin) return FPW_ENOTSUP;
+  given = given || p.threads || p.freqs_per_thread;
+  const size_t limit = (size_t)ctx->smem_optin;
+  while (!p.threads && T > 32 && tile_shape_bytes(T, R, M, 32, p.accum, ngroups) > limit) T /= 2;
+  if (tile_shape_bytes(T, R, M, NC ? NC : 32, p.accum, ngroups) > limit) return FPW_ENOTSUP;
   out.threads = T;
   out.R = R;
   out.obs_chunk = NC;
-  out.smem = smem;
+
+  const auto fit = [&](int r) { return (int)(limit / tile_smem_bytes(32, r, M, k, p.accum, ngroups)); };
+  int r = R, w = T / 32;
+  if (!given) {
+    r = wide ? 2 : M <= 12 ? 8 : M <= 16 && !multi ? 6 : M <= 20 ? 5 : M <= 25 ? 4 : M <= 33 ? 3 : M <= 50 ? 2 : M <= 64 ? 3 : 1;
+    if (multi && M > 50 && M <= 64) r = 2;
+    w = wide ? 12 : 8;
+    while (r > 1 && fit(r) < 4) --r;
+    if (r == 7 || (multi && r == 6)) --r;
+    w = std::min(w, fit(r));
+    // The shape that is estimated to finish first: for one curve, whose tiles all
+    // take the same time, by rounds of tiles; else by the work and half a tile of
+    // the longest curve at the end (R only below the measured one). A shape that
+    // cuts an anchor block evenly, with a compiled combination if the call has one.
+    const int spec = multi ? multi_spec_of(M, ngroups, groups) : 0;
+    const auto estimate = [&](int q, int v) {
+      const int64_t tiles = C * warp_tiles(F, q);
+      if (C == 1 || tiles < 4 * (int64_t)ctx->nsm) return shape_time(ctx, q, v, tiles, wide);
+      const double round = shape_time(ctx, q, v, (int64_t)ctx->nsm * v, wide);
+      return round * ((double)tiles / ((double)ctx->nsm * v) + 0.5 * (double)(max_n + 64) / (double)(n_mean + 64));
+    };
+    double best = estimate(r, w);
+    const int r0 = r;
+    for (int q : {8, 6, 5, 4, 3, 2, 1}) {
+      if (q > (C == 1 ? (wide ? 4 : 8) : r0) || (q == 6 && multi) || (q == 3 && p.accum == FPW_ACCUM_FP64)) continue;
+      if ((dense && T * R % (32 * q) != 0) || (spec && q != 2 && !(spec == 3 && q == 5))) continue;
+      for (int v : {4, 7, 8, 12}) {
+        if (v > fit(q) || v > tile_max_warps(multi) || (C > 1 && v < 8)) continue;
+        const double t = estimate(q, v);
+        if (t < 0.95 * best) {
+          best = t;
+          r = q;
+          w = v;
+        }
+      }
+    }
+    // no more warps than spread the tiles over every SM
+    w = (int)std::max<int64_t>(1, std::min<int64_t>(w, (C * warp_tiles(F, r) + ctx->nsm - 1) / ctx->nsm));
+  }
+  w = std::min({w, fit(r), tile_max_warps(multi)});
+  if (w < 1) return FPW_ENOTSUP;
+  out.warps = w;
+  out.lane_R = r;
+  out.smem = tile_smem_bytes(32 * w, r, M, k, p.accum, ngroups);
   out.items = items;
   return FPW_OK;
 }
 
-// Work items: each curve's frequency range split into segments of whole tiles
-// so that every resident block gets about sh.items items (load balance), sorted by
-// cost (observations x frequencies) descending; candidate rows per curve in
-// curve order. The tables are uploaded from a pinned copy, ordered on `st`.
+// Work items: each curve's frequency range cut into segments of whole warp
+// tiles. The curves are taken in the order of their cost (longest first) and an
+// item gets at most 1 / (1.5 * resident warps) of the work that is then left, so
+// the items shrink towards the end of the list and the warps finish together (a
+// fixed size left 2-10 % of the time to the last items); never less than a
+// tile, nor than 1 / (4 * items) of a warp's share. Cuts lie between anchor
+// blocks where an item holds one at least. halo: frequencies an item evaluates
+// beyond each end of its range (1 when peaks are asked for). aligned: tiles stay
+// inside anchor blocks. Candidate rows per curve in curve order. The tables are
+// uploaded from a pinned copy, ordered on `st`.
 Plan* build_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const TileShape& sh, int blocks_per_sm,
-                 uint64_t key, cudaStream_t st, int* err) {
+                 int halo, bool aligned, uint64_t key, cudaStream_t st, int* err) {
   *err = FPW_OK;
-  const int64_t Wown = (int64_t)sh.threads * sh.R - 2;
-  const int64_t tiles = (F + Wown - 1) / Wown;
-  const int resident = std::max(1, blocks_per_sm * ctx->nsm);
-  double total = 0.0;
-  for (int64_t c = 0; c < C; ++c) total += (double)(off[c + 1] - off[c] + 32) * (double)F;
-  const double target = std::max(total / ((double)sh.items * resident), 32.0 * (double)Wown * 16.0);
-  std::vector<double> ccv((size_t)C);
-  std::vector<int64_t> nseg((size_t)C);
-  bool all_split = C > 1;
+  const int64_t W = 32 * (int64_t)sh.lane_R, A = (int64_t)sh.threads * sh.R - 2;
+  const int64_t B = (A + 2 * halo + W - 1) / W;  // tiles of an anchor block
+  const int64_t resident = (int64_t)std::max(1, blocks_per_sm * ctx->nsm) * sh.warps;
+  // a tile's cost in observations: about 64 more for its reduction, peaks and staging
+  const auto cost = [&](int64_t c) { return (double)(off[c + 1] - off[c] + 64); };
+  std::vector<int64_t> order((size_t)C);
+  double left = 0.0;
   for (int64_t c = 0; c < C; ++c) {
-    const double cc = (double)(off[c + 1] - off[c] + 32) * (double)F;
-    ccv[(size_t)c] = cc;
-    int64_t n = (int64_t)std::llround(cc / target);
-    // A curve that would be cut finer than three tiles per item (a single long
-    // curve, cut for load balance) gets whole rounds of the resident blocks,
-    // each item at least three tiles: an item's prologue, restaging and
-    // candidate row cost about a tile's latency, and equal items that do not
-    // fill whole rounds leave blocks idle. 1000 observations x 1e6
-    // frequencies: 0.635 -> 0.60 ms of tile kernel, 0.76 -> 0.67 ms per call.
-    const int64_t rounds = tiles / (3 * (int64_t)resident);
-    if (n > tiles / 3 && rounds >= 1) n = rounds * resident;
-    n = std::max<int64_t>(1, std::min<int64_t>(n, tiles));
-    nseg[(size_t)c] = n;
-    if (n < 2) all_split = false;
+    order[(size_t)c] = c;
+    left += cost(c) * (double)((F + 2 * halo + W - 1) / W);
   }
-  // Every curve cut (a few long curves): the item count is made whole rounds
-  // of the resident blocks, shared by cost with the largest remainders (20
-  // equal curves over 2e6 frequencies and 152 blocks: 1220 items, a ninth
-  // round nearly empty, became 1216).
-  int64_t nall = 0;
-  for (int64_t c = 0; c < C; ++c) nall += nseg[(size_t)c];
-  if (all_split && nall >= resident && nall % resident != 0) {  // fewer items: the minimum item size binds
-    const int64_t want = std::max<int64_t>(resident, (nall + resident / 2) / resident * resident);
-    std::vector<std::pair<double, int64_t>> frac;
-    int64_t got = 0;
-    for (int64_t c = 0; c < C; ++c) {
-      const double share = (double)want * ccv[(size_t)c] / total;
-      const int64_t f = std::max<int64_t>(1, std::min<int64_t>((int64_t)std::floor(share), tiles));
-      nseg[(size_t)c] = f;
-      got += f;
-      if (f < tiles) frac.emplace_back(share - std::floor(share), c);
-    }
-    std::stable_sort(frac.begin(), frac.end(), [](const std::pair<double, int64_t>& x, const std::pair<double, int64_t>& y) {
-      return x.first > y.first;
-    });
-    for (size_t i = 0; i < frac.size() && got < want; ++i, ++got) nseg[(size_t)frac[i].second] += 1;
-  }
-  std::vector<WorkItem> items;
-  std::vector<double> cost;
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int64_t x, int64_t y) { return off[x + 1] - off[x] > off[y + 1] - off[y]; });
+  const double least = left / ((double)resident * 4.0 * (double)sh.items);
+  std::vector<WorkItem> sorted;  // the shares shrink as the list grows
+  sorted.reserve((size_t)C + (size_t)(resident * sh.items));
   std::vector<int32_t> base((size_t)C + 1, 0);
-  items.reserve((size_t)C);
-  for (int64_t c = 0; c < C; ++c) {
-    const double cc = ccv[(size_t)c];
-    const int64_t ns = nseg[(size_t)c];
-    base[c + 1] = base[c] + (int32_t)ns;
-    for (int64_t q = 0; q < ns; ++q) {
-      const int64_t t0 = tiles * q / ns, t1 = tiles * (q + 1) / ns;
+  for (const int64_t c : order) {
+    const double cc = cost(c);
+    int64_t lo = 0;
+    int32_t rows = 0;
+    while (lo < F) {
+      const double share = std::max(left / (1.5 * (double)resident), least);
+      const int64_t rest = (F - lo + 2 * halo + W - 1) / W;  // tiles to the end in one item
+      const int64_t n = std::max<int64_t>(1, (int64_t)(share / cc));
+      int64_t hi = n >= B ? (lo / A + n / B) * A : lo + n * W - 2 * halo;
+      if (n < B && aligned) hi = std::min(hi, (lo / A + 1) * A);
+      if (n + n / 4 >= rest && (!aligned || n >= B)) hi = F;
+      hi = std::min(hi, F);
+      const double work = cc * (double)((hi - lo + 2 * halo + W - 1) / W);
       WorkItem w;
       w.curve = (int32_t)c;
-      w.f_lo = (int32_t)(t0 * Wown);
-      w.f_hi = (int32_t)std::min<int64_t>(F, t1 * Wown);
-      w.slot = base[c] + (int32_t)q;
-      items.push_back(w);
-      cost.push_back(cc * (double)(t1 - t0) / (double)tiles);
+      w.f_lo = (int32_t)lo;
+      w.f_hi = (int32_t)hi;
+      w.slot = rows++;
+      sorted.push_back(w);
+      left = std::max(0.0, left - work);
+      lo = hi;
     }
+    base[(size_t)c + 1] = rows;
   }
-  std::vector<int> order(items.size());
-  for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
-  std::vector<WorkItem> sorted(items.size());
-  for (size_t i = 0; i < order.size(); ++i) sorted[i] = items[order[i]];
+  for (int64_t c = 0; c < C; ++c) base[(size_t)c + 1] += base[(size_t)c];
+  for (WorkItem& w : sorted) w.slot += base[(size_t)w.curve];
 
   Plan* pl = new (std::nothrow) Plan();
   if (!pl) {
@@ -367,22 +386,19 @@ Plan* build_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const T
     return nullptr;
   }
   pl->key = key;
-  pl->shape = sh;
   pl->nitems = (int)sorted.size();
   pl->nslots = base[C];
   for (int64_t c = 0; c < C; ++c) pl->max_rows = std::max(pl->max_rows, base[c + 1] - base[c]);
-  pl->grid = std::max(1, std::min(resident, pl->nitems));
+  pl->grid = (int)std::max<int64_t>(1, (std::min<int64_t>(resident, pl->nitems) + sh.warps - 1) / sh.warps);
   const size_t ib = sorted.size() * sizeof(WorkItem), bb = base.size() * sizeof(int32_t);
-  cudaError_t e = ensure(pl->items, ib);
-  if (e == cudaSuccess) e = ensure(pl->cand_base, bb);
+  cudaError_t e = ensure(pl->items, ib + bb);
   if (e == cudaSuccess) e = cudaMallocHost(&pl->host_stage, ib + bb);
+  pl->cand_base = reinterpret_cast<int32_t*>(static_cast<char*>(pl->items.p) + ib);
   if (e == cudaSuccess) {
     memcpy(pl->host_stage, sorted.data(), ib);
     memcpy(static_cast<char*>(pl->host_stage) + ib, base.data(), bb);
-    e = cudaMemcpyAsync(pl->items.p, pl->host_stage, ib, cudaMemcpyHostToDevice, st);
+    e = cudaMemcpyAsync(pl->items.p, pl->host_stage, ib + bb, cudaMemcpyHostToDevice, st);
   }
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(pl->cand_base.p, static_cast<char*>(pl->host_stage) + ib, bb, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) {
     *err = cuda_fail(e, "plan upload");
     free_plan(pl);
@@ -392,7 +408,7 @@ Plan* build_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const T
 }
 
 Plan* get_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const TileShape& sh, int blocks_per_sm,
-               cudaStream_t st, int* err) {
+               int halo, bool aligned, cudaStream_t st, int* err) {
   uint64_t key = fnv1a(off, sizeof(int64_t) * (size_t)(C + 1));
   key = mix(key, C);
   key = mix(key, F);
@@ -402,13 +418,17 @@ Plan* get_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const Til
   key = mix(key, sh.smem);
   key = mix(key, sh.items);
   key = mix(key, blocks_per_sm);
+  key = mix(key, halo);
+  key = mix(key, aligned);
+  key = mix(key, sh.warps);
+  key = mix(key, sh.lane_R);
   for (Plan* p : ctx->plans)
     if (p->key == key) {
       p->use = ++ctx->tick;
       *err = FPW_OK;
       return p;
     }
-  Plan* p = build_plan(ctx, off, C, F, sh, blocks_per_sm, key, st, err);
+  Plan* p = build_plan(ctx, off, C, F, sh, blocks_per_sm, halo, aligned, key, st, err);
   if (!p) return nullptr;
   p->use = ++ctx->tick;
   if ((int)ctx->plans.size() >= kMaxPlans) {
@@ -456,11 +476,45 @@ void drop_graphs(fpw_ctx* ctx) {
   ctx->graphs.clear();
 }
 
-// Enqueue prep -> persistent tile kernel -> merge -> status latch.
-int enqueue_tile_path(fpw_ctx* ctx, const BatchCall& b, Plan* pl, unsigned* words, cudaStream_t st) {
+// The tile path's scratch, one allocation: the call's words and per-curve flags
+// (first, cleared at once), the prep kernel's output per observation and per
+// anchor block, the candidate table.
+struct Scratch {
+  size_t floors, clear, aw, rec, low, dev, delta, cand_S, cand_idx, total;  // clear: bytes to clear, from the start
+};
+Scratch scratch_layout(const BatchCall& b, const TileShape& sh, const Plan* pl) {
+  const size_t nobs = (size_t)b.off_h[b.C], A = (size_t)sh.threads * sh.R - 2, blocks = ((size_t)b.F + A - 1) / A;
+  const size_t rows = (size_t)(b.ngroups > 0 ? b.ngroups : 1) * (size_t)pl->nslots * (size_t)b.k;
+  size_t o = 0;
+  const auto take = [&](size_t bytes) {
+    const size_t at = o;
+    o = (o + bytes + 255) & ~(size_t)255;
+    return at;
+  };
+  Scratch L;
+  take(kCallWords * sizeof(unsigned) + (size_t)b.C);
+  L.floors = take((b.k > 0 ? (size_t)b.C * (size_t)std::max(b.ngroups, 1) : 0) * sizeof(unsigned long long));
+  L.clear = o;
+  L.aw = take((nobs + 2) * accum_bin_bytes(b.p.accum));
+  L.rec = take((nobs + 2) * sizeof(ulonglong2));
+  L.low = take((nobs + 2) * sizeof(uint2));
+  L.dev = take(blocks * sizeof(float));
+  L.delta = take(blocks * sizeof(float));
+  L.cand_S = take(rows * sizeof(double));
+  L.cand_idx = take(rows * sizeof(int32_t));
+  L.total = o;
+  return L;
+}
+
+// Enqueue prep -> persistent tile kernel -> merge.
+int enqueue_tile_path(fpw_ctx* ctx, const BatchCall& b, const TileShape& sh, Plan* pl, cudaStream_t st) {
   const int64_t nobs = b.off_h[b.C];
-  FPW_CK(cudaMemsetAsync(words, 0, 2 * sizeof(unsigned), st));
-  FPW_CK(cudaMemsetAsync(ctx->curve_bad.p, 0, (size_t)b.C, st));
+  // the call's words and the curves' flags are one region, cleared at once
+  const Scratch L = scratch_layout(b, sh, pl);
+  char* const scratch = static_cast<char*>(ctx->scratch.p);
+  unsigned* const call = reinterpret_cast<unsigned*>(scratch);
+  uint8_t* const curve_bad = reinterpret_cast<uint8_t*>(scratch + kCallWords * sizeof(unsigned));
+  FPW_CK(cudaMemsetAsync(call, 0, L.clear, st));
   PrepArgs pa{};
   pa.t = b.t;
   pa.x = b.x;
@@ -470,36 +524,48 @@ int enqueue_tile_path(fpw_ctx* ctx, const BatchCall& b, Plan* pl, unsigned* word
   pa.nobs = nobs;
   pa.freqs = b.freqs;
   pa.nfreq = b.F;
-  pa.aw = ctx->aw.p;
+  pa.aw = scratch + L.aw;
   pa.accum = b.p.accum;
-  pa.curve_bad = static_cast<uint8_t*>(ctx->curve_bad.p);
-  pa.status = words + 1;
+  pa.curve_bad = curve_bad;
+  pa.status = call + 1;
+  pa.latch = static_cast<unsigned*>(ctx->words.p) + kWordLatch;
+  pa.rec = reinterpret_cast<ulonglong2*>(scratch + L.rec);
+  pa.rec_low = reinterpret_cast<uint2*>(scratch + L.low);
+  pa.anchor_span = (int64_t)sh.threads * sh.R - 2;
+  pa.block_dev = reinterpret_cast<float*>(scratch + L.dev);
+  pa.block_delta = reinterpret_cast<float*>(scratch + L.delta);
+  pa.df = reinterpret_cast<double*>(call + kWordDf);
+  pa.grid_dev = call + kWordGridDev;
   FPW_CK(launch_prep(pa, st));
-  const int W = pl->shape.threads * pl->shape.R;
-  const int64_t tiles = (b.F + (W - 2) - 1) / (W - 2);
-  FPW_CK(launch_tile_dev(b.freqs, b.F, W, tiles, static_cast<double*>(ctx->tile_dev.p), st));
   TileArgs ta{};
   ta.t = b.t;
   ta.offsets = b.offsets;
   ta.n_single = b.offsets ? 0 : nobs;
-  ta.aw = ctx->aw.p;
+  ta.aw = pa.aw;
   ta.freqs = b.freqs;
   ta.nfreq = b.F;
   ta.items = static_cast<const WorkItem*>(pl->items.p);
   ta.nitems = pl->nitems;
-  ta.counter = words;
-  ta.status = words + 1;
-  ta.curve_bad = static_cast<const uint8_t*>(ctx->curve_bad.p);
-  ta.cand_S = b.k > 0 ? static_cast<double*>(ctx->cand_S.p) : nullptr;
-  ta.cand_idx = b.k > 0 ? static_cast<int32_t*>(ctx->cand_idx.p) : nullptr;
+  ta.counter = call;
+  ta.status = call + 1;
+  ta.curve_bad = curve_bad;
+  ta.floors = b.k > 0 ? reinterpret_cast<unsigned long long*>(scratch + L.floors) : nullptr;
+  ta.cand_S = b.k > 0 ? reinterpret_cast<double*>(scratch + L.cand_S) : nullptr;
+  ta.cand_idx = b.k > 0 ? reinterpret_cast<int32_t*>(scratch + L.cand_idx) : nullptr;
   ta.S_out = b.S_out;
   ta.M = b.M;
   ta.k = b.k;
   ta.peak_raw = b.p.peak_mode == FPW_PEAK_RAW ? 1 : 0;
   ta.K = b.p.K;
-  ta.obs_chunk = pl->shape.obs_chunk;
   ta.inv_alpha2 = b.p.inv_alpha2;
-  ta.tile_dev = static_cast<const double*>(ctx->tile_dev.p);
+  ta.rec = pa.rec;
+  ta.rec_low = pa.rec_low;
+  ta.anchor_span = pa.anchor_span;
+  ta.aligned = b.S_out || b.bins_out ? 1 : 0;
+  ta.block_dev = pa.block_dev;
+  ta.block_delta = pa.block_delta;
+  ta.df = pa.df;
+  ta.grid_dev = pa.grid_dev;
   ta.ngroups = b.ngroups;
   for (int q = 0; q < b.ngroups; ++q) ta.group_g[q] = b.groups[q];
   ta.group_rows = pl->nslots;
@@ -516,32 +582,29 @@ int enqueue_tile_path(fpw_ctx* ctx, const BatchCall& b, Plan* pl, unsigned* word
     }
     FPW_CK(cudaEventRecord(ctx->ev[ctx->ev_used], st));
   }
-  FPW_CK(launch_tile(ta, pl->shape, b.p.phase_mode, b.p.accum, pl->grid, st));
+  FPW_CK(launch_tile(ta, sh, b.p.phase_mode, b.p.accum, pl->grid, st));
   if (timed) {
     FPW_CK(cudaEventRecord(ctx->ev[ctx->ev_used + 1], st));
     ctx->ev_used += 2;
   }
   if (b.k > 0) {
-    const int ng = b.ngroups > 0 ? b.ngroups : 1;
-    for (int q = 0; q < ng; ++q) {
-      const int64_t rows = (int64_t)q * pl->nslots * b.k;
-      MergeArgs ma{};
-      ma.cand_S = static_cast<const double*>(ctx->cand_S.p) + rows;
-      ma.cand_idx = static_cast<const int32_t*>(ctx->cand_idx.p) + rows;
-      ma.cand_base = static_cast<const int32_t*>(pl->cand_base.p);
-      ma.curve_bad = static_cast<const uint8_t*>(ctx->curve_bad.p);
-      ma.status = words + 1;
-      ma.ncurves = b.C;
-      ma.k = b.k;
-      ma.topk_idx = b.topk_idx + (int64_t)q * b.k;
-      ma.topk_S = b.topk_S + (int64_t)q * b.k;
-      ma.out_stride = ng * b.k;
-      ma.topk_off = b.ngroups > 0 ? b.topk_off + (int64_t)q * b.k : nullptr;
-      ma.max_rows = pl->max_rows;
-      FPW_CK(launch_merge(ma, st));
-    }
+    MergeArgs ma{};
+    ma.cand_S = ta.cand_S;
+    ma.cand_idx = ta.cand_idx;
+    ma.cand_base = pl->cand_base;
+    ma.curve_bad = curve_bad;
+    ma.status = call + 1;
+    ma.ncurves = b.C;
+    ma.k = b.k;
+    ma.topk_idx = b.topk_idx;
+    ma.topk_S = b.topk_S;
+    ma.out_stride = std::max(b.ngroups, 1) * b.k;
+    ma.topk_off = b.ngroups > 0 ? b.topk_off : nullptr;
+    ma.max_rows = pl->max_rows;
+    ma.ngroups = b.ngroups;
+    ma.group_rows = pl->nslots;
+    FPW_CK(launch_merge(ma, st));
   }
-  FPW_CK(launch_latch(words, st));
   return FPW_OK;
 }
 
@@ -556,33 +619,25 @@ int run_tile_path(fpw_ctx* ctx, const BatchCall& b) {
   }
   const int64_t n_typ = sn > 0.0 ? (int64_t)(sn2 / sn) : 0;  // observation-weighted mean curve size
   TileShape sh{};
-  int rc = choose_shape(ctx, b.p, b.M, b.k, max_n, n_typ, b.ngroups, sh);
+  int rc = choose_shape(ctx, b.p, b.M, b.k, b.C, b.F, max_n, (int64_t)(sn / (double)b.C), n_typ, b.ngroups, b.groups,
+                        b.S_out || b.bins_out, sh);
   if (rc != FPW_OK) return rc;
-  const int bps = tile_max_blocks_per_sm(sh.R, b.p.phase_mode, b.p.accum, sh.threads, sh.smem, b.ngroups > 0,
+  const int bps = tile_max_blocks_per_sm(sh.lane_R, b.p.phase_mode, b.p.accum, 32 * sh.warps, sh.smem, b.ngroups > 0,
                                          b.bins_out != nullptr, multi_spec_of(b.M, b.ngroups, b.groups));
   if (bps < 1) return FPW_ENOTSUP;
-  Plan* pl = get_plan(ctx, b.off_h, b.C, b.F, sh, bps, b.stream, &rc);
+  Plan* pl = get_plan(ctx, b.off_h, b.C, b.F, sh, bps, b.k > 0 ? 1 : 0, b.S_out || b.bins_out, b.stream, &rc);
   if (!pl) return rc;
   ctx->last_shape = sh;
   ctx->last_grid = pl->grid;
-  const int64_t nobs = b.off_h[b.C];
+  ctx->call_status = nullptr;
   // scratch (grow-only; growing invalidates captured graphs)
-  void* before[6] = {ctx->aw.p, ctx->cand_S.p, ctx->cand_idx.p, ctx->curve_bad.p, ctx->words.p, ctx->tile_dev.p};
-  cudaError_t e = ensure(ctx->aw, (size_t)(nobs + 2) * accum_bin_bytes(b.p.accum));
-  {
-    const int64_t Wown = (int64_t)sh.threads * sh.R - 2;
-    if (e == cudaSuccess) e = ensure(ctx->tile_dev, sizeof(double) * (size_t)((b.F + Wown - 1) / Wown + 1));
-  }
-  const size_t ng = (size_t)(b.ngroups > 0 ? b.ngroups : 1);
-  if (e == cudaSuccess && b.k > 0) e = ensure(ctx->cand_S, ng * pl->nslots * b.k * sizeof(double));
-  if (e == cudaSuccess && b.k > 0) e = ensure(ctx->cand_idx, ng * pl->nslots * b.k * sizeof(int32_t));
-  if (e == cudaSuccess) e = ensure(ctx->curve_bad, (size_t)b.C + 16);
+  const void* const before = ctx->scratch.p;
+  const cudaError_t e = ensure(ctx->scratch, scratch_layout(b, sh, pl).total);
   if (e != cudaSuccess) return cuda_fail(e, "scratch allocation");
-  void* after[6] = {ctx->aw.p, ctx->cand_S.p, ctx->cand_idx.p, ctx->curve_bad.p, ctx->words.p, ctx->tile_dev.p};
-  if (memcmp(before, after, sizeof(before)) != 0) drop_graphs(ctx);
-  unsigned* words = static_cast<unsigned*>(ctx->words.p);
+  if (ctx->scratch.p != before) drop_graphs(ctx);
+  ctx->call_status = static_cast<unsigned*>(ctx->scratch.p) + 1;
 
-  if (!b.p.use_graph || b.bins_out) return enqueue_tile_path(ctx, b, pl, words, b.stream);
+  if (!b.p.use_graph || b.bins_out) return enqueue_tile_path(ctx, b, sh, pl, b.stream);
 
   uint64_t gk = mix(pl->key, (const void*)b.stream);
   for (const void* q : {(const void*)b.offsets, (const void*)b.t, (const void*)b.x, (const void*)b.sigma,
@@ -600,11 +655,7 @@ int run_tile_path(fpw_ctx* ctx, const BatchCall& b) {
   gk = mix(gk, b.ngroups);
   for (int q = 0; q < b.ngroups; ++q) gk = mix(gk, b.groups[q]);
   gk = mix(gk, (const void*)b.topk_off);
-  gk = mix(gk, ctx->aw.p);
-  gk = mix(gk, ctx->cand_S.p);
-  gk = mix(gk, ctx->cand_idx.p);
-  gk = mix(gk, ctx->curve_bad.p);
-  gk = mix(gk, ctx->tile_dev.p);
+  gk = mix(gk, ctx->scratch.p);
   gk = mix(gk, pl);
   for (GraphEntry& g : ctx->graphs)
     if (g.key == gk) {
@@ -616,7 +667,7 @@ int run_tile_path(fpw_ctx* ctx, const BatchCall& b) {
   // captured); the instantiated graph is launched on the caller's stream.
   cudaGraph_t graph = nullptr;
   FPW_CK(cudaStreamBeginCapture(ctx->own_stream, cudaStreamCaptureModeThreadLocal));
-  rc = enqueue_tile_path(ctx, b, pl, words, ctx->own_stream);
+  rc = enqueue_tile_path(ctx, b, sh, pl, ctx->own_stream);
   cudaError_t ec = cudaStreamEndCapture(ctx->own_stream, &graph);
   if (rc != FPW_OK) {
     if (graph) cudaGraphDestroy(graph);
@@ -646,6 +697,7 @@ int run_tile_path(fpw_ctx* ctx, const BatchCall& b) {
 int run_plain_path(fpw_ctx* ctx, const BatchCall& b) {
   if (plain_smem_bytes(b.M) > (size_t)ctx->smem_optin) return FPW_ENOTSUP;  // binary64 bins of one block
   unsigned* words = static_cast<unsigned*>(ctx->words.p);
+  ctx->call_status = words + 1;
   FPW_CK(cudaMemsetAsync(words, 0, 2 * sizeof(unsigned), b.stream));
   // validate frequencies (and observations) once for the status word
   PrepArgs pa{};
@@ -714,7 +766,7 @@ int sync_status(fpw_ctx* ctx, cudaStream_t st, int rc) {
   if (rc != FPW_OK) return rc;
   FPW_CK(cudaStreamSynchronize(st));
   unsigned w = 0;
-  FPW_CK(cudaMemcpy(&w, static_cast<unsigned*>(ctx->words.p) + 1, sizeof(unsigned), cudaMemcpyDeviceToHost));
+  if (ctx->call_status) FPW_CK(cudaMemcpy(&w, ctx->call_status, sizeof(unsigned), cudaMemcpyDeviceToHost));
   return status_to_code(w);
 }
 
@@ -838,7 +890,6 @@ int fpw_ctx_create(fpw_ctx** out, int device) {
     ctx->nsm = prop.multiProcessorCount;
     ctx->smem_optin = (int)prop.sharedMemPerBlockOptin;
     ctx->smem_per_sm = (int)prop.sharedMemPerMultiprocessor;
-    e = tile_init_attributes(ctx->smem_optin);
   }
   if (e == cudaSuccess) e = plain_init_attributes(ctx->smem_optin);
   if (e == cudaSuccess && (size_t)ctx->smem_optin >= shared_smem_bytes()) e = shared_init_attributes();
@@ -865,7 +916,7 @@ int fpw_ctx_destroy(fpw_ctx* ctx) {
     drop_graphs(ctx);
     for (Plan* p : ctx->plans) free_plan(p);
     ctx->plans.clear();
-    for (DevBuf* b : {&ctx->aw, &ctx->cand_S, &ctx->cand_idx, &ctx->curve_bad, &ctx->words, &ctx->dense, &ctx->tile_dev, &ctx->h_off,
+    for (DevBuf* b : {&ctx->scratch, &ctx->curve_bad, &ctx->words, &ctx->dense, &ctx->h_off,
                       &ctx->h_t, &ctx->h_x, &ctx->h_sigma, &ctx->h_freqs, &ctx->h_idx, &ctx->h_S, &ctx->sh_image,
                       &ctx->sh_scale, &ctx->sh_S32, &ctx->sh_step, &ctx->sh_sink, &ctx->dr_payload,
                       &ctx->dr_H0, &ctx->dr_g, &ctx->dr_tabs})
@@ -942,8 +993,8 @@ int fpw_ctx_status(fpw_ctx* ctx) {
   std::lock_guard<std::mutex> lk(ctx->mu);
   FPW_CK(cudaStreamSynchronize(ctx->last_stream));
   unsigned w = 0;
-  FPW_CK(cudaMemcpy(&w, static_cast<unsigned*>(ctx->words.p) + 2, sizeof(unsigned), cudaMemcpyDeviceToHost));
-  FPW_CK(cudaMemset(static_cast<unsigned*>(ctx->words.p) + 2, 0, sizeof(unsigned)));
+  FPW_CK(cudaMemcpy(&w, static_cast<unsigned*>(ctx->words.p) + kWordLatch, sizeof(unsigned), cudaMemcpyDeviceToHost));
+  FPW_CK(cudaMemset(static_cast<unsigned*>(ctx->words.p) + kWordLatch, 0, sizeof(unsigned)));
   return status_to_code(w);
 }
 
@@ -1082,6 +1133,7 @@ int fpw_periodogram_ex(fpw_ctx* ctx, void* stream, const fpw_params* params, con
     // single curve: the plain kernel reads the curve directly
     if (plain_smem_bytes(M) > (size_t)ctx->smem_optin) return FPW_ENOTSUP;
     unsigned* words = static_cast<unsigned*>(ctx->words.p);
+    ctx->call_status = words + 1;
     FPW_CK(cudaMemsetAsync(words, 0, 2 * sizeof(unsigned), st));
     FPW_CK(ensure(ctx->curve_bad, 16));
     PrepArgs pa{};
@@ -1199,6 +1251,7 @@ int fpw_periodogram_shared(fpw_ctx* ctx, void* stream, const fpw_params* params,
   if ((size_t)ctx->smem_optin < shared_smem_bytes()) return FPW_ENOTSUP;
   if (ncurves == 0) return FPW_OK;
   unsigned* words = static_cast<unsigned*>(ctx->words.p);
+  ctx->call_status = words + 1;
   if (nfreq == 0) {
     if (k > 0) FPW_CK(launch_fill_topk(topk_idx, topk_S, ncurves * k, st));
     return FPW_OK;
@@ -1298,6 +1351,7 @@ int fpw_periodogram_drift(fpw_ctx* ctx, void* stream, const fpw_params* params, 
   const int64_t nobs = ctx->off_host[(size_t)ncurves];
   if (nobs > 0 && (!t || !x || !sigma)) return FPW_EINVAL;
   unsigned* words = static_cast<unsigned*>(ctx->words.p);
+  ctx->call_status = words + 1;
   if (nfreq == 0) {
     if (k > 0) FPW_CK(launch_fill_topk(topk_idx, topk_S, ncurves * k, st));
     return FPW_OK;

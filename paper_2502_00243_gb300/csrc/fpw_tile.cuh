@@ -6,34 +6,48 @@
 // side (shapes, launches) is fpw_tile.cu.
 //
 // Work decomposition
-//   A work item is (curve c, frequency segment [f_lo, f_hi)). Thread blocks pop
-//   items from a global counter (items are sorted by cost, longest first).
-//   Within an item the segment is swept in tiles of W = T * R consecutive
-//   frequencies: thread j owns tile positions j*R + r (r < R). Tiles overlap by
-//   two frequencies so that every owned frequency has both neighbours in the
-//   same tile (needed for the local-maximum test of the peak finder); tile
-//   starts sit at q*(W-2) - 1 for integer q, whatever the item's segment.
+//   A work item is (curve c, frequency segment [f_lo, f_hi)), swept by ONE WARP
+//   in tiles of W = 32 R consecutive frequencies: lane l owns tile positions
+//   l R + r (r < R). The first item of a warp is fixed by its index (so that a
+//   short list spreads over every SM), the next ones come from a global counter
+//   (items are sorted by cost, longest first). Warps share nothing: no barrier
+//   wider than a warp runs, so one warp's staging, reduction and peaks overlap
+//   the other warps' bin updates. (A block per item, its four warps meeting at
+//   barriers around every chunk and tile, ran the same loop at 1.93e12
+//   evaluations/s where warps of their own run MEASURE_M20, M = 20.)
+//   An item computes S at f_lo - 1 .. f_hi: both neighbours of every owned
+//   frequency (the local-maximum test needs them); tiles do not overlap inside
+//   an item, the last two values of a tile are carried to the next.
 //
 // Per tile
-//   1. Anchor: for each observation, Phi_s = frac(t_i * f_s) as a 64-bit
-//      fixed-point fraction from the exact integer product of the binary64
-//      significands, and the step D_i = frac(t_i * df) (df = grid spacing).
-//      Both are staged in shared memory with the prep kernel's weights
-//      (a_i = x_i w_i, w_i).
-//   2. Hot loop (per observation, per thread, per r): Phi = Phi_s + (j*R + r) D_i
+//   1. Stage (per 32 observations, lane = observation, a ring of two chunks in
+//      shared memory, the next chunk's inputs already in registers): the phase
+//      Phi_s = frac(t_i * f_s) at the tile's first frequency as a 64-bit
+//      fixed-point fraction, the step D_i = frac(t_i * df) (df = grid spacing) and
+//      the weights (a_i = x_i w_i, w_i). Where the whole grid lies on its line,
+//      Phi_s takes a few integer operations from the prep kernel's records (60
+//      operations an observation and tile for the exact product held up the hot
+//      loops for 5-10 % of the time); else it is the exact integer product of the
+//      binary64 significands.
+//   2. Hot loop (per observation, per lane, per r): Phi = Phi_s + (l R + r) D_i
 //      (mod 2^64), bin m = floor(M * Phi_hi / 2^32), A_m += a_i, B_m += w_i in a
-//      thread-private [r][m][thread] bin array in shared memory (bank = lane,
-//      so conflict-free), all R loads issued before the R stores; every thread
-//      reads each staged observation (a warp-uniform broadcast).
+//      lane-private [r][m][lane] bin array in shared memory (bank = lane, so
+//      conflict-free). Software-pipelined: the addresses of observation i + 1
+//      are formed while the bins of observation i are on their way, from a
+//      record loaded one observation earlier, across chunk boundaries too.
 //   3. Reduce: S = sum_m A_m^2 / (B_m + 1/alpha^2), empty bins contribute 0.
 //      Several-M kernel: in-place prefix sums of the M_max bins, then for each
 //      group g the windows of g consecutive bins (circularly) for every offset;
 //      S_g(f) is the largest S over the g offsets, and that offset is kept.
-//   4. Peaks: local maxima among owned frequencies, merged into the item's
-//      running top-k (shared memory), written as candidates at the item's end.
+//   4. Peaks: local maxima among owned frequencies that beat the k-th best so
+//      far are inserted into the item's sorted list (shared memory), written as
+//      candidates at the item's end.
 //
-// Grids that are not linear to within kGridTolCycles over a tile fall back to a
-// direct exact anchor per (observation, frequency).
+// Grids that are not linear to within kGridTolCycles over a tile: the phase is
+// frac(t_i f_b) (exact, f_b the tile's middle frequency) plus t_i (f_k - f_b) from
+// FP32 pairs, correct to 2^-36 cycles (NlTile). A tile whose frequencies spread
+// over more than 2^7 cycles either side takes a direct exact anchor per (observation,
+// frequency).
 //
 // Bin sums (policy P): FP32 pairs (A, B); binary64 pairs; or FP32 pairs with
 // compensation terms (A, B, cA, cB), where each addition is an exact two-sum
@@ -44,7 +58,7 @@
 //
 // DUMP instantiations additionally write the bin m of every (observation,
 // owned frequency k) with bins_k0 <= k < bins_k1 to args.bins_out, from the
-// same arithmetic as the sums (bin-identity checks of the product kernel).
+// same phase arithmetic as the sums (bin-identity checks of the product kernel).
 #pragma once
 #include <math.h>
 
@@ -57,46 +71,40 @@ const void* tile_fn_f32(int R, int phase_mode, bool dump);
 const void* tile_fn_f32_odd(int R, int phase_mode, bool dump);  // R = 3, 5, 6
 const void* tile_fn_f64(int R, int phase_mode, bool dump);
 const void* tile_fn_comp(int R, int phase_mode, bool dump);
-const void* tile_fn_multi(int R, int phase_mode, int spec);  // spec: multi_spec_of(), 0 = generic
+const void* tile_fn_multi(int R, int phase_mode, int spec);  // spec: multi_spec_of(), 0 = any groups
 
-struct TileLayout {
-  size_t bins, pd, aw, candS, candI, topS, topI, edges, red, misc, total;
+struct WarpLayout {
+  size_t pd, aw, topS, topI, total;
 };
 
 __host__ __device__ inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
-// Shared-memory carve-up of one block: bins [R][M][T] of bin_bytes, the staged
-// {Phi, D} (16 B) and weights (bin_bytes) of NC observations plus two padding
-// records (read by the hot loop's prefetch past a chunk's last observation,
-// never used), peak scratch.
-__host__ __device__ inline TileLayout tile_layout(int T, int R, int M, int NC, size_t bin_bytes, int ngroups) {
-  const size_t W = (size_t)T * R;
-  const size_t tops = (size_t)(ngroups > 1 ? ngroups : 1) * FPW_MAX_TOPK;
-  TileLayout L;
-  size_t o = 0;
-  L.bins = o;
-  o = align16(o + (size_t)R * M * T * bin_bytes);
+// Staged observations of a warp: a ring of two chunks of 32, plus copies of the
+// first two slots after the last (the hot loop prefetches two records ahead
+// without wrapping the index).
+constexpr int kSlots = 64;
+constexpr int kRing = kSlots + 2;
+
+// Shared memory of one warp: bins [R][M][32] of bin_bytes, the ring of staged
+// {Phi, D} (16 B) and weights (bin_bytes), the top-k lists of every group.
+__host__ __device__ inline WarpLayout warp_layout(int R, int M, size_t bin_bytes, int kk, int ngroups) {
+  const size_t tops = (size_t)(ngroups > 1 ? ngroups : 1) * (size_t)kk;
+  WarpLayout L;
+  size_t o = (size_t)R * M * 32 * bin_bytes;
   L.pd = o;
-  o = align16(o + (size_t)(NC + 2) * 16);
+  o += (size_t)kRing * 16;
   L.aw = o;
-  o = align16(o + (size_t)(NC + 2) * bin_bytes);
-  L.candS = o;
-  o = align16(o + W * 8);
-  L.candI = o;
-  o = align16(o + W * 4);
+  o = align16(o + (size_t)kRing * bin_bytes);
   L.topS = o;
-  o = align16(o + tops * 8);
+  o += tops * 8;
   L.topI = o;
   o = align16(o + tops * 4);
-  L.edges = o;
-  o = align16(o + (size_t)(T / 32) * 2 * 8);
-  L.red = o;
-  o = align16(o + 32 * 8);
-  L.misc = o;
-  o = align16(o + 64);
   L.total = o;
   return L;
 }
+
+// Threads of a launched block: FP32 sums of one M and the other sum modes; several M.
+constexpr int kTileMaxThreads = 384, kMultiMaxThreads = 256;
 
 #ifdef __CUDACC__
 namespace {
@@ -165,6 +173,14 @@ __device__ __forceinline__ float bin_term(float2 v, float cal) {
   const float q = __fdividef((v.x * v.x) * sc, den * sc);
   return (den > 0.f) ? q : 0.f;
 }
+// The same where every denominator is known to be 0 or inside [2^-100, 2^100]
+// (the curve's weights and 1/alpha^2 lie well inside, Warp::plain): the same
+// value, about half the instructions.
+__device__ __forceinline__ float bin_term_plain(float2 v, float cal) {
+  const float den = v.y + cal;
+  const float q = __fdividef(v.x * v.x, den);
+  return (den > 0.f) ? q : 0.f;
+}
 __device__ __forceinline__ double bin_term(double2 v, double cal) {
   const double den = v.y + cal;
   return (den > 0.0) ? v.x * v.x / den : 0.0;
@@ -177,6 +193,11 @@ __device__ __forceinline__ double bin_term(float4 v, double cal) {
   return (double)bin_term(make_float2(v.x + v.z, v.y + v.w), (float)cal);
 }
 
+__device__ __forceinline__ double bin_term_plain(double2 v, double cal) { return bin_term(v, cal); }
+__device__ __forceinline__ double bin_term_plain(float4 v, double cal) {
+  return (double)bin_term_plain(make_float2(v.x + v.z, v.y + v.w), (float)cal);
+}
+
 __device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 
 __device__ __forceinline__ double warp_max(double v) {
@@ -185,444 +206,701 @@ __device__ __forceinline__ double warp_max(double v) {
   return v;
 }
 
-// Order-preserving map of a double to an unsigned integer (larger value, larger
-// image), and its inverse.
-__device__ __forceinline__ unsigned long long rank_bits(double s) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(s);
-  return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
+// The largest s among the lanes with k >= 0 (one at least), and whether the
+// lane holds it.
+__device__ __forceinline__ bool warp_best(float s, int k, float& best) {
+  const unsigned u = __float_as_uint(s), r = k >= 0 ? ((u >> 31) ? ~u : (u | 0x80000000u)) : 0u;
+  const unsigned m = __reduce_max_sync(0xffffffffu, r);
+  best = __uint_as_float((m >> 31) ? (m & 0x7fffffffu) : ~m);
+  return k >= 0 && r == m;
 }
-__device__ __forceinline__ double from_rank_bits(unsigned long long r) {
-  return __longlong_as_double((long long)((r >> 63) ? (r & 0x7fffffffffffffffull) : ~r));
-}
-
-// Selects the best kk entries of (top list) + (candidate list) into the top
-// list, ranked by S descending then key ascending. Executed by one warp.
-// Entries with key < 0 are empty. kk <= FPW_MAX_TOPK (two results per lane).
-// Round q takes the best entry ranked after round q-1's pick (keys are unique
-// within an item, so no entry needs marking): each lane's best over its
-// strided share, then the warp's from three redux.sync maxima over (S's
-// order-preserving high word, its low word, the inverted key).
-__device__ void warp_merge_topk(double* topS, int* topI, int kk, double* cS, int* cI, int cnt, int lane) {
-  double keepS[2] = {-INFINITY, -INFINITY};
-  int keepI[2] = {-1, -1};
-  const int pool = kk + cnt;
-  unsigned long long prev_r = 0ull;
-  unsigned prev_k = 0u;
-  for (int q = 0; q < kk; ++q) {
-    unsigned long long br = 0ull;  // 0: nothing (no double maps to 0 here)
-    unsigned bk = 0u;
-    for (int e = lane; e < pool; e += 32) {
-      const int i = (e < kk) ? topI[e] : cI[e - kk];
-      if (i < 0) continue;
-      const unsigned long long r = rank_bits((e < kk) ? topS[e] : cS[e - kk]);
-      const unsigned kx = ~(unsigned)i;
-      const bool after = (q == 0) || r < prev_r || (r == prev_r && kx < prev_k);
-      if (after && (r > br || (r == br && kx > bk))) {
-        br = r;
-        bk = kx;
-      }
-    }
-    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(br >> 32));
-    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(br >> 32) == hi ? (unsigned)br : 0u);
-    const unsigned long long wr = ((unsigned long long)hi << 32) | lo;
-    const unsigned wk = __reduce_max_sync(0xffffffffu, br == wr ? bk : 0u);
-    if (wr == 0ull) break;  // every entry taken
-    prev_r = wr;
-    prev_k = wk;
-    if (lane == (q & 31)) {
-      keepS[q >> 5] = from_rank_bits(wr);
-      keepI[q >> 5] = (int)~wk;
-    }
-  }
-  __syncwarp();
-  for (int q = lane; q < kk; q += 32) {
-    topS[q] = keepS[q >> 5];
-    topI[q] = keepI[q >> 5];
-  }
-  __syncwarp();
+__device__ __forceinline__ bool warp_best(double s, int k, double& best) {
+  const unsigned long long r = k >= 0 ? rank_bits(s) : 0ull;
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(r >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(r >> 32) == hi ? (unsigned)r : 0u);
+  const unsigned long long m = ((unsigned long long)hi << 32) | lo;
+  best = from_rank_bits(m);
+  return k >= 0 && r == m;
 }
 
-// Per-block view of shared memory and the constants every stage needs.
+// The k-th best S that some item of curve row `row` has found so far (0: none):
+// items of the curve skip what lies below it. Nothing depends on when a value
+// arrives: k peaks at least as high are then in that item's list.
+__device__ __forceinline__ unsigned long long curve_floor(const TileArgs& args, int64_t row) {
+  return args.floors ? *(volatile unsigned long long*)(args.floors + row) : 0ull;
+}
+template <class A>
+__device__ __forceinline__ A floor_value(unsigned long long f) {
+  return f != 0ull ? (A)from_rank_bits(f) : (A)-INFINITY;
+}
+__device__ __forceinline__ void raise_floor(const TileArgs& args, int64_t row, const double* topS, const int* topI,
+                                            int kk, int lane) {
+  if (args.floors && lane == 0 && topI[kk - 1] >= 0) atomicMax(args.floors + row, rank_bits(topS[kk - 1]));
+}
+
+// Shared-memory bin access by 32-bit address. volatile: their order is the
+// program's (the next observation's bin loads follow this one's stores).
+__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void lds(unsigned a, float2& v) {
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void lds(unsigned a, float4& v) {
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(a)
+               : "memory");
+}
+__device__ __forceinline__ void lds(unsigned a, double2& v) {
+  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void lds(unsigned a, ulonglong2& v) {
+  asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void sts(unsigned a, float2 v) {
+  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void sts(unsigned a, float4 v) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ void sts(unsigned a, double2 v) {
+  asm volatile("st.shared.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v.x), "d"(v.y) : "memory");
+}
+
+// Per-warp view of shared memory and the constants every stage needs.
 template <class P>
-struct Block {
-  using Bin = typename P::Bin;
-  using In = typename P::In;
-  unsigned char* my_bins;    // this thread's column of the [r][m][thread] bin array
-  ulonglong2* sPD;           // staged {Phi_s, D} per observation
-  In* sAW;                   // staged weights per observation
-  double* candS;
-  int* candI;
-  double* topS;              // [groups][FPW_MAX_TOPK]
+struct Warp {
+  using A = typename P::S;
+  unsigned char* bins;       // this lane's column of the [r][m][lane] bin array
+  ulonglong2* pd;            // ring of staged {Phi, D} (or {P, T}, NlTile; or {t, 0})
+  typename P::In* aw;        // ring of staged weights
+  double* topS;              // [groups][kk], sorted
   int* topI;
-  double* edges;
-  double* red;
-  int* misc;
-  int T, tid, lane, warp, nwarps, M, NC, kk, W;
-  unsigned T8, MT8, j0;      // T8: bytes between bins of a column; MT8: between its R frequencies
+  int lane, M, kk;
   int64_t F;
   double df;
+  static constexpr unsigned kBinStride = 32u * (unsigned)sizeof(typename P::Bin);  // bytes between bins of a column
 };
 
 template <int R, class P>
-__device__ __forceinline__ Block<P> make_block(unsigned char* smem, const TileArgs& args) {
-  using Bin = typename P::Bin;
-  Block<P> b;
-  b.T = blockDim.x;
-  b.tid = threadIdx.x;
-  b.lane = b.tid & 31;
-  b.warp = b.tid >> 5;
-  b.nwarps = b.T >> 5;
-  b.M = args.M;
-  b.NC = args.obs_chunk;
-  b.kk = args.k;
-  b.W = b.T * R;
-  const TileLayout L = tile_layout(b.T, R, b.M, b.NC, sizeof(Bin), args.ngroups);
-  b.my_bins = smem + L.bins + (size_t)b.tid * sizeof(Bin);
-  b.sPD = reinterpret_cast<ulonglong2*>(smem + L.pd);
-  b.sAW = reinterpret_cast<typename P::In*>(smem + L.aw);
-  b.candS = reinterpret_cast<double*>(smem + L.candS);
-  b.candI = reinterpret_cast<int*>(smem + L.candI);
-  b.topS = reinterpret_cast<double*>(smem + L.topS);
-  b.topI = reinterpret_cast<int*>(smem + L.topI);
-  b.edges = reinterpret_cast<double*>(smem + L.edges);
-  b.red = reinterpret_cast<double*>(smem + L.red);
-  b.misc = reinterpret_cast<int*>(smem + L.misc);
-  b.T8 = (unsigned)b.T * (unsigned)sizeof(Bin);
-  b.MT8 = (unsigned)b.M * b.T8;
-  b.j0 = (unsigned)b.tid * R;
-  b.F = args.nfreq;
-  b.df = (b.F > 1) ? (args.freqs[b.F - 1] - args.freqs[0]) / (double)(b.F - 1) : 0.0;
-  return b;
-}
-
-// The two padding records after the staged chunk hold zeros (defined values
-// for the prefetch that reads them; made visible by the first item's barrier).
-template <class P>
-__device__ __forceinline__ void zero_padding(const Block<P>& b) {
-  if (b.tid < 2) {
-    b.sPD[b.NC + b.tid] = make_ulonglong2(0ull, 0ull);
-    typename P::In z;
-    bin_zero(z);
-    b.sAW[b.NC + b.tid] = z;
+__device__ __forceinline__ Warp<P> make_warp(unsigned char* smem, const TileArgs& args) {
+  Warp<P> w;
+  w.lane = threadIdx.x & 31;
+  w.M = args.M;
+  w.kk = args.k;
+  const WarpLayout L = warp_layout(R, w.M, sizeof(typename P::Bin), w.kk, args.ngroups);
+  unsigned char* const mine = smem + (size_t)(threadIdx.x >> 5) * L.total;
+  w.bins = mine + (size_t)w.lane * sizeof(typename P::Bin);
+  w.pd = reinterpret_cast<ulonglong2*>(mine + L.pd);
+  w.aw = reinterpret_cast<typename P::In*>(mine + L.aw);
+  w.topS = reinterpret_cast<double*>(mine + L.topS);
+  w.topI = reinterpret_cast<int*>(mine + L.topI);
+  w.F = args.nfreq;
+  w.df = args.df ? *args.df : (w.F > 1) ? (args.freqs[w.F - 1] - args.freqs[0]) / (double)(w.F - 1) : 0.0;
+  // bins start at zero (every reduce leaves them zero again), and so does the
+  // ring (the prefetch past a curve's last observation reads slots not staged)
+  for (int q = 0; q < R * w.M; ++q)
+    bin_zero(*reinterpret_cast<typename P::Bin*>(w.bins + (size_t)q * Warp<P>::kBinStride));
+  for (int q = w.lane; q < kRing; q += 32) {
+    w.pd[q] = make_ulonglong2(0ull, 0ull);
+    bin_zero(w.aw[q]);
   }
+  return w;
 }
 
-// Is the grid linear over the tile starting at s? The precomputed per-tile
-// deviation when available (tile starts sit at multiples of W-2, minus one),
-// else checked here (block-wide).
-template <int R, class P>
-__device__ __forceinline__ bool tile_is_linear(const TileArgs& args, const Block<P>& b, int64_t s, int64_t a,
-                                               double fa, double tm) {
-  if (args.tile_dev) return args.tile_dev[(s + 1) / (b.W - 2)] * tm <= kGridTolCycles;
-  bool nonlin = false;
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int64_t k = s + (int64_t)b.j0 + r;
-    if (k >= 0 && k < b.F) {
-      const double pred = fma((double)(k - a), b.df, fa);
-      if (fabs(args.freqs[k] - pred) * tm > kGridTolCycles) nonlin = true;
-    }
-  }
-  return !__syncthreads_or(nonlin);
+// v as the unevaluated sum of two FP32 numbers, by integer operations: to 2^-48
+// relative for 2^-74 <= |v| < 2^100, to 2^-98 for smaller |v|.
+__device__ __forceinline__ float2 split_f32(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned hi = (unsigned)(b >> 32), e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
+  if (e < 949u) return make_float2((e < 924u) ? 0.f : __uint_as_float(sign | (e - 896u) << 23 | ((unsigned)(b >> 29) & 0x7fffffu)), 0.f);
+  // the leading 24 significand bits are one float, the other 29 become one
+  return make_float2(__uint_as_float(sign | (e - 896u) << 23 | ((unsigned)(b >> 29) & 0x7fffffu)),
+                     __uint2float_rn((unsigned)b & 0x1fffffffu) * __uint_as_float(sign | (e - 948u) << 23));
 }
 
-// DUMP: bins m[r] of observation `obs` (global index) at tile positions j + r.
+__device__ __forceinline__ int exponent_of(double v) {  // floor(log2 |v|) for normal v; -1023 for 0 and subnormals
+  return (int)(((unsigned long long)__double_as_longlong(v) >> 52) & 0x7ffull) - 1023;
+}
+
+// How a tile's phases are formed: stepped from the first frequency on (the whole
+// grid on its line, no dense output); stepped from the exact phase at the anchor
+// of the tile's block (the block on a line), which kRecord derives from the prep
+// kernel's records and kAnchor from the product; products with the distance from
+// an exact phase (NlTile); the exact phase of every pair.
+enum TileMode { kLine, kRecord, kAnchor, kFixed, kExact };
+
+// The frequencies of a tile off the linear grid, as FP32 pairs of f_k - f_b (f_b:
+// the tile's middle frequency). An observation's phase at f_k is its exact phase
+// at f_b plus t (f_k - f_b), |t (f_k - f_b)| < 2^7 cycles, with t an FP32 pair
+// too: the product's multiple of 2^-14 cycles comes off the mantissa of one
+// fused multiply-add (kMagic), the rest is a sum of the exact remainder and the
+// cross terms, in units of 2^-36. Off by less than a unit either way; the staged
+// phase is rounded up and carries one unit more, so the sum is never below the
+// exact phase (a phase on a bin edge stays in the upper bin) and at most 3 units
+// above it. FP32 multiply-adds because integer products are slow: mul.hi runs at
+// 30 lanes/clk/SM, fma at 110 (measured); the same sum from 61-bit integer
+// factors (three mul.hi more than the linear step) ran 1.04e12 evaluations/s at
+// M = 20.
 template <int R>
-__device__ __forceinline__ void dump_bins(const TileArgs& args, int W, int64_t s, const WorkItem& wi, int64_t obs,
-                                          unsigned j, const unsigned (&m)[R]) {
+struct NlTile {
+  float dh[R], dl[R];
+};
+constexpr float kMagic = 768.f;               // 1.5 * 2^9: sums keep multiples of 2^-14 in the low mantissa bits
+constexpr unsigned kMagicLow = 0x4B400000u;   // bits of 1.5 * 2^23
+
+// pd: {P's 32 bits below the binary point | its next four and -kMagicLow, th | tl}
+__device__ __forceinline__ unsigned nl_phase(const ulonglong2& pd, float dh, float dl) {
+  const float th = __uint_as_float((unsigned)pd.y), tl = __uint_as_float((unsigned)(pd.y >> 32));
+  const float m = __fmaf_rn(th, dh, kMagic);
+  float e = __fmaf_rn(th, dh, -__fsub_rn(m, kMagic));
+  e = __fmaf_rn(th, dl, e);
+  e = __fmaf_rn(tl, dh, e);
+  e = __fmaf_rn(e, 0x1p36f, 0x1.8p23f);
+  const int low = (int)(__float_as_uint(e) + (unsigned)(pd.x >> 32));
+  return (__float_as_uint(m) << 18) + (unsigned)pd.x + (unsigned)(low >> 4);
+}
+
+// Geometry of one tile: first frequency s (-1 possible), its anchor block's first
+// position sq and anchor frequency fa (index max(sq, 0)), how its phases are
+// formed, and (kRecord) the anchor's index and distance from the line through f_0.
+struct Tile {
+  int64_t s, sq;
+  double fa;
+  TileMode mode;
+  unsigned a;
+  float delta;
+};
+
+// The tile at s. aligned: it lies in block q, whose block_delta is `delta`.
+template <int R, class P>
+__device__ __forceinline__ Tile make_tile(const TileArgs& args, const Warp<P>& w, int64_t s, int64_t q, float delta,
+                                          double tm, bool every_lin, bool aligned, NlTile<R>& nl) {
+  Tile g;
+  bool inside = true;  // one block's line serves the whole tile
+  if (!aligned && !every_lin) {
+    const unsigned k = s < 0 ? 0u : (unsigned)(s < w.F ? s : w.F - 1), A = (unsigned)args.anchor_span;
+    q = k / A;
+    delta = args.block_delta[q];
+    inside = s + 32 * R - 1 <= (q + 1) * (int64_t)A;
+  }
+  g.s = s;
+  g.sq = q * args.anchor_span - 1;
+  const int64_t a = g.sq < 0 ? 0 : g.sq;
+  g.a = (unsigned)a;
+  g.delta = delta;
+  g.fa = 0.0;
+  g.mode = aligned ? kRecord : kLine;
+  if (every_lin) return g;
+  g.fa = args.freqs[a];
+  bool lin, rec = false;
+  if (!inside) {
+    lin = false;
+  } else if (args.block_dev) {
+    lin = (double)args.block_dev[q] * tm <= kGridTolCycles;
+    rec = fabs((double)delta * 0x1p-32) * tm < 0x1p30;
+  } else {
+    bool off = false;
+    for (int64_t j = w.lane; j < args.anchor_span + 2; j += 32) {
+      const int64_t k = g.sq + j;
+      if (k >= 0 && k < w.F && fabs(args.freqs[k] - fma((double)(k - a), w.df, g.fa)) * tm > kGridTolCycles) off = true;
+    }
+    lin = !__any_sync(0xffffffffu, off);
+  }
+  if (lin) {
+    g.mode = rec ? kRecord : kAnchor;
+    return g;
+  }
+  const int64_t s0 = s < 0 ? 0 : (s < w.F ? s : w.F - 1), mid = s + 16 * R;
+  const double fb = args.freqs[mid < w.F ? mid : s0];
+  double f[R];
+  int de = -1023;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const unsigned jr = j + (unsigned)r;
-    const int64_t k = s + (int64_t)jr;
-    if (jr >= 1u && jr + 1u < (unsigned)W && k >= wi.f_lo && k < wi.f_hi && k >= args.bins_k0 && k < args.bins_k1)
-      args.bins_out[(k - args.bins_k0) * args.bins_nobs + obs] = (int32_t)m[r];
+    const int64_t k = s + (int64_t)(w.lane * R + r);
+    f[r] = k >= 0 && k < w.F ? args.freqs[k] - fb : 0.0;
+    de = max(de, exponent_of(f[r]));
+  }
+  de = __reduce_max_sync(0xffffffffu, de);
+  const int te = exponent_of(tm);
+  if (te < -20 || te > 40 || te + de + 2 > 7) {  // |t (f_k - f_b)| may reach 2^7 cycles (or split_f32's range ends)
+    g.mode = kExact;
+    return g;
+  }
+  g.mode = kFixed;
+  g.fa = fb;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const float2 d = split_f32(f[r]);
+    nl.dh[r] = d.x;
+    nl.dl[r] = d.y;
+  }
+  return g;
+}
+
+// One observation's inputs on their way from global memory to the ring.
+template <class P>
+struct Obs {
+  ulonglong2 rec;  // the prep kernel's record (kLine, kRecord), {t, 0} else
+  uint2 low;       // kRecord: what goes with it
+  typename P::In aw;
+};
+
+template <class P>
+__device__ __forceinline__ Obs<P> fetch(const TileArgs& args, TileMode mode, int64_t base, int64_t n, int64_t i) {
+  Obs<P> o;
+  o.rec = make_ulonglong2(0ull, 0ull);  // past the curve's end: t = 0 and zero weights, which add 0 to some bin
+  o.low = make_uint2(0u, 0u);
+  bin_zero(o.aw);
+  if (i < n) {
+    if (mode == kLine || mode == kRecord) {
+      o.rec = args.rec[base + i];
+      if (mode == kRecord) o.low = args.rec_low[base + i];
+    } else {
+      o.rec.x = (unsigned long long)__double_as_longlong(args.t[base + i]);
+    }
+    o.aw = reinterpret_cast<const typename P::In*>(args.aw)[base + i];
+  }
+  return o;
+}
+
+// The staged phase record: {phase, step D}, {P, T} (NlTile) or {t, 0}. The phase is
+// that of frequency -1 as the prep kernel left it (kLine: the hot loop takes s + 1
+// + j steps from it), else that of the tile's first frequency: the exact phase at
+// the block's anchor, rounded up at 2^-64, plus s - sq steps. kRecord takes the
+// anchor's from P_0 + a D with 96 bits of D (the 64-bit step's rounding adds up to
+// a 2^-64 = 10^-15 cycles, and visits a round fraction of a day apart put phases
+// that close to bin edges) plus t times the anchor frequency's distance from the
+// line (FP32 of a term below 2^-33 cycles), a fifth of the operations of the
+// product. With Df = D rounded down, a + (s - sq) = s (+ the anchor's step back in
+// block 0).
+template <class P>
+__device__ __forceinline__ ulonglong2 record(const TileArgs& args, const Warp<P>& w, const Tile& g, TileMode mode,
+                                             const Obs<P>& o) {
+  if (mode == kLine || mode == kExact) return o.rec;
+  if (mode == kRecord) {
+    const float v = __uint_as_float(o.low.y) * g.delta;  // three FP32 roundings, made up for in the next line
+    const unsigned long long low =
+        (unsigned long long)g.a * o.low.x + (unsigned long long)__float2ll_rn(__fmaf_rn(fabsf(v), 0x1p-21f, v));
+    const unsigned up = o.low.x != 0u ? 1u : 0u;  // D is rounded up
+    // the low words' carry, the rounding up, and the steps of D not of Df
+    const int more = (int)(low >> 32) + ((unsigned)low != 0u ? 1 : 0) +
+                     (up ? (int)(g.s - g.sq) - (g.sq < 0 ? 1 : 0) : 0);
+    const unsigned long long D = o.rec.y, Df = D - up;
+    return make_ulonglong2(o.rec.x + D + (unsigned long long)(long long)g.s * Df + (unsigned long long)(long long)more, D);
+  }
+  const double t = __longlong_as_double((long long)o.rec.x);
+  unsigned long long Pa = phase_fixed64(t, g.fa);
+  if (mode == kFixed) {
+    const float2 tt = split_f32(t);
+    const unsigned long long p = ((Pa + 0xfffffffull) >> 28) + 1ull;  // units of 2^-36, rounded up, one more
+    const unsigned c = (unsigned)(p & 15ull) - kMagicLow;
+    return make_ulonglong2(((unsigned long long)c << 32) | (unsigned)(p >> 4),
+                           ((unsigned long long)__float_as_uint(tt.y) << 32) | __float_as_uint(tt.x));
+  }
+  const unsigned long long D = phase_fixed64(t, w.df);
+  if (g.sq < 0) Pa -= D;  // block 0 starts one step before its anchor
+  return make_ulonglong2(Pa + (unsigned long long)(g.s - g.sq) * D, D);
+}
+
+// Chunk c of 32 observations into its half of the ring.
+template <class P>
+__device__ __forceinline__ void put(const Warp<P>& w, int64_t c, const ulonglong2& pd, const typename P::In& aw) {
+  const int slot = (int)(c & 1) * 32 + w.lane;
+  w.pd[slot] = pd;
+  w.aw[slot] = aw;
+  if (slot < 2) {
+    w.pd[slot + kSlots] = pd;
+    w.aw[slot + kSlots] = aw;
   }
 }
 
-// Stages every observation chunk of the curve for the tile starting at s and
-// accumulates its bins (steps 1 and 2). A curve that fits in one chunk keeps
-// D_i and its weights staged across the tiles of an item (keep); only the
-// anchor phase is then recomputed.
-template <int R, int PHASE, class P, bool DUMP>
-__device__ __forceinline__ void accumulate_tile(const TileArgs& args, const Block<P>& b, int64_t s, int64_t a,
-                                                double fa, bool lin, bool keep, bool& staged_lin, int64_t base,
-                                                int64_t n, const WorkItem& wi) {
+// Steps 1 and 2 for one tile. The R phases of an observation are independent
+// multiply-adds, its R bin loads precede its R stores, and the addresses of the
+// next observation are formed in between; four observations per trip rename the
+// pipelined registers instead of moving them. Against the loop that formed and
+// used an observation's bins in the same trip (probe, loop alone): M = 20, R =
+// 5, 8 warps per SM 1.85 -> 2.08e12 evaluations/s; M = 60, R = 3, 4 warps 1.15
+// -> 1.5e12. MODE kRecord serves kAnchor too (mode).
+template <int R, class P, TileMode MODE>
+__device__ __forceinline__ void accumulate(const TileArgs& args, const Warp<P>& w, const Tile& g, const NlTile<R>& nl,
+                                           int64_t base, int64_t n, TileMode mode) {
   using Bin = typename P::Bin;
   using In = typename P::In;
-  const int T = b.T, tid = b.tid, NC = b.NC;
-  const unsigned M = (unsigned)b.M, T8 = b.T8, MT8 = b.MT8, j0 = b.j0;
-  unsigned char* const my_bins = b.my_bins;
-  ulonglong2* const sPD = b.sPD;
-  In* const sAW = b.sAW;
-  for (int64_t o = 0; o < n; o += NC) {
-    const int cnt = (int)((n - o) < NC ? (n - o) : NC);
-    for (int i = tid; i < cnt; i += T) {
-      const double ti = args.t[base + o + i];
-      if (keep) {
-        const unsigned long long D = sPD[i].y;
-        unsigned long long Pa = phase_fixed64(ti, fa);
-        if (s < a) Pa -= D;  // tile starts one step before frequency 0
-        sPD[i].x = Pa;
-      } else {
-        ulonglong2 pd;
-        if (lin) {
-          const unsigned long long D = phase_fixed64(ti, b.df);
-          unsigned long long Pa = phase_fixed64(ti, fa);
-          if (s < a) Pa -= D;
-          pd = make_ulonglong2(Pa, D);
-        } else {
-          pd = make_ulonglong2((unsigned long long)__double_as_longlong(ti), 0ull);
-        }
-        sPD[i] = pd;
-        sAW[i] = reinterpret_cast<const In*>(args.aw)[base + o + i];
-      }
+  constexpr int U = 4, kChunk = 32;
+  const unsigned M = (unsigned)w.M;
+  const unsigned j0 = (unsigned)w.lane * R + (MODE == kLine ? (unsigned)(g.s + 1) : 0u);
+  const unsigned col = smem_u32(w.bins), rstride = M * Warp<P>::kBinStride;
+  const int64_t npad = (n + U - 1) / U * U, nchunk = (n + kChunk - 1) / kChunk;
+  const auto addresses = [&](const ulonglong2& p, unsigned (&ad)[R]) {
+    if (MODE == kFixed) {
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        ad[r] = col + (unsigned)r * rstride + __umulhi(nl_phase(p, nl.dh[r], nl.dl[r]), M) * Warp<P>::kBinStride;
+    } else {
+      const unsigned long long phi = p.x + (unsigned long long)j0 * p.y;
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        ad[r] = col + (unsigned)r * rstride + bin_of_phase(phi + (unsigned long long)r * p.y, M) * Warp<P>::kBinStride;
     }
-    staged_lin = lin;
-    __syncthreads();
-    if (lin && PHASE == FPW_PHASE_FIXED64) {
-      // Every thread reads each staged observation (a warp-uniform broadcast)
-      // and adds it into its own column. The next observation's staged data
-      // is loaded before this one's bin stores (the compiler cannot move it
-      // there itself: both are shared memory), so the broadcast-load latency
-      // overlaps the bin updates.
-      if (R <= 2) {
-        // Software-pipelined (measured faster at R <= 2, where the phase ->
-        // bin -> offset chain is a larger share of each iteration; slower at
-        // R = 4): the bins of observation i + 1 are computed while observation
-        // i's bin loads are in flight, from staged data loaded one iteration
-        // earlier. Same adds in the same order as the loop below.
-        unsigned m[R];
-        {
-          const ulonglong2 p0 = sPD[0];
-          const unsigned long long f0 = p0.x + (unsigned long long)j0 * p0.y;
+  };
+  Obs<P> o = fetch<P>(args, mode, base, n, w.lane);
+  const Obs<P> o1 = fetch<P>(args, mode, base, n, 32 + w.lane);
+  __syncwarp();  // every lane is done with the previous tile's ring
+  put<P>(w, 0, record<P>(args, w, g, mode, o), o.aw);
+  put<P>(w, 1, record<P>(args, w, g, mode, o1), o1.aw);
+  o = fetch<P>(args, mode, base, n, 64 + w.lane);
+  __syncwarp();
+  const unsigned pd0 = smem_u32(w.pd), aw0 = smem_u32(w.aw);
+  ulonglong2 p1;
+  In x0, x1;
+  unsigned ad[R];
+  lds(pd0, p1);
+  addresses(p1, ad);
+  lds(aw0, x0);
+  lds(pd0 + 16u, p1);
+  lds(aw0 + (unsigned)sizeof(In), x1);
+  for (int64_t c = 0; c < nchunk; ++c) {
+    const int lim = (int)((npad - c * kChunk) < kChunk ? (npad - c * kChunk) : kChunk);
+    const unsigned first = (unsigned)(c & 1) * kChunk + 2u;
+    unsigned pa = pd0 + first * 16u, xa = aw0 + first * (unsigned)sizeof(In);
+#pragma unroll 1
+    for (int i = 0; i < lim; i += U) {
 #pragma unroll
-          for (int r = 0; r < R; ++r) m[r] = bin_of_phase(f0 + (unsigned long long)r * p0.y, M);
-        }
-        In xv = sAW[0];
-        ulonglong2 pdn = sPD[1];  // a padding record when cnt == 1
-        In xn = sAW[1];
-        for (int i = 0; i < cnt; ++i) {
-          const ulonglong2 pdnn = sPD[i + 2];  // index <= cnt + 1 <= NC + 1: staged or padding
-          const In xnn = sAW[i + 2];
-          Bin v[R];
+      for (int u = 0; u < U; ++u) {
+        Bin v[R];
 #pragma unroll
-          for (int r = 0; r < R; ++r) v[r] = *reinterpret_cast<const Bin*>(my_bins + m[r] * T8 + (unsigned)r * MT8);
-          const unsigned long long fn = pdn.x + (unsigned long long)j0 * pdn.y;
-          unsigned mn[R];
-#pragma unroll
-          for (int r = 0; r < R; ++r) mn[r] = bin_of_phase(fn + (unsigned long long)r * pdn.y, M);
-#pragma unroll
-          for (int r = 0; r < R; ++r)
-            *reinterpret_cast<Bin*>(my_bins + m[r] * T8 + (unsigned)r * MT8) = bin_add(v[r], xv);
-          if (DUMP) dump_bins<R>(args, b.W, s, wi, base + o + i, j0, m);
-#pragma unroll
-          for (int r = 0; r < R; ++r) m[r] = mn[r];
-          xv = xn;
-          pdn = pdnn;
-          xn = xnn;
-        }
-      } else {
-        ulonglong2 pd = sPD[0];
-        In xv = sAW[0];
-#pragma unroll 2
-        for (int i = 0; i < cnt; ++i) {
-          const ulonglong2 pdn = sPD[i + 1];  // index <= cnt <= NC: staged or padding
-          const In xn = sAW[i + 1];
-          // the R phases are independent multiply-adds (no serial chain of 64-bit adds)
-          const unsigned long long phi0 = pd.x + (unsigned long long)j0 * pd.y;
-          unsigned m[R];
-#pragma unroll
-          for (int r = 0; r < R; ++r) m[r] = bin_of_phase(phi0 + (unsigned long long)r * pd.y, M);
-          Bin v[R];
-#pragma unroll
-          for (int r = 0; r < R; ++r) v[r] = *reinterpret_cast<const Bin*>(my_bins + m[r] * T8 + (unsigned)r * MT8);
-#pragma unroll
-          for (int r = 0; r < R; ++r)
-            *reinterpret_cast<Bin*>(my_bins + m[r] * T8 + (unsigned)r * MT8) = bin_add(v[r], xv);
-          if (DUMP) dump_bins<R>(args, b.W, s, wi, base + o + i, j0, m);
-          pd = pdn;
-          xv = xn;
-        }
-      }
-    } else if (lin) {  // FPW_PHASE_FP32: FP32 phase from an FP32 anchor every K frequencies
-      const int K = args.K;
-      float jr[R];
-      long long da[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const long long k = s + (long long)j0 + r;
-        const long long ak = (k >= 0) ? k - (k % K) : 0;
-        jr[r] = (float)(k - ak);
-        da[r] = ak - s;
-      }
-      for (int i = 0; i < cnt; ++i) {
-        const ulonglong2 pd = sPD[i];
-        const In xv = sAW[i];
-        const float d32 = (float)(unsigned)(pd.y >> 32) * 0x1p-32f;
-        unsigned m[R];
+        for (int r = 0; r < R; ++r) lds(ad[r], v[r]);
+        ulonglong2 p2;
+        In x2;
+        lds(pa + (unsigned)u * 16u, p2);  // two records ahead: staged, a copy, or a slot whose value is not used
+        lds(xa + (unsigned)u * (unsigned)sizeof(In), x2);
+        unsigned an[R];
+        addresses(p1, an);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          const unsigned long long pa = pd.x + (unsigned long long)da[r] * pd.y;
-          const float p32 = (float)(unsigned)(pa >> 32) * 0x1p-32f;
-          float p = fmaf(jr[r], d32, p32);
-          p = p - floorf(p);
-          unsigned mm = (unsigned)(p * (float)M);
-          m[r] = mm < M ? mm : M - 1u;
+          sts(ad[r], bin_add(v[r], x0));
+          ad[r] = an[r];
         }
-        Bin v[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = *reinterpret_cast<const Bin*>(my_bins + m[r] * T8 + (unsigned)r * MT8);
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-          *reinterpret_cast<Bin*>(my_bins + m[r] * T8 + (unsigned)r * MT8) = bin_add(v[r], xv);
-        if (DUMP) dump_bins<R>(args, b.W, s, wi, base + o + i, j0, m);
+        x0 = x1;
+        x1 = x2;
+        p1 = p2;
       }
-    } else {  // non-linear grid: exact anchor per (observation, frequency)
-      double fr[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        int64_t k = s + (int64_t)j0 + r;
-        k = k < 0 ? 0 : (k >= b.F ? b.F - 1 : k);
-        fr[r] = args.freqs[k];
-      }
-      for (int i = 0; i < cnt; ++i) {
-        const double ti = __longlong_as_double((long long)sPD[i].x);
-        const In xv = sAW[i];
-        unsigned m[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) m[r] = bin_of_phase(phase_fixed64(ti, fr[r]), M);
-        Bin v[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = *reinterpret_cast<const Bin*>(my_bins + m[r] * T8 + (unsigned)r * MT8);
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-          *reinterpret_cast<Bin*>(my_bins + m[r] * T8 + (unsigned)r * MT8) = bin_add(v[r], xv);
-        if (DUMP) dump_bins<R>(args, b.W, s, wi, base + o + i, j0, m);
-      }
+      pa += U * 16u;
+      xa += U * (unsigned)sizeof(In);
     }
-    __syncthreads();
+    if (c + 2 < nchunk) {  // this chunk's half of the ring is free: the next but one
+      __syncwarp();
+      put<P>(w, c + 2, record<P>(args, w, g, mode, o), o.aw);
+      o = fetch<P>(args, mode, base, n, (c + 3) * kChunk + w.lane);
+      __syncwarp();
+    }
   }
 }
 
-// Step 4: the local maxima among this tile's owned frequencies (or every owned
-// frequency in raw mode), ranked into the running top list topS/topI. The
-// ranking key of frequency k is (k << key_shift) | extra[r].
-template <int R, class P>
-__device__ __forceinline__ void tile_peaks(const TileArgs& args, const Block<P>& b, const typename P::S (&S)[R],
-                                           const int (&extra)[R], int key_shift, int64_t s, const WorkItem& wi,
-                                           double* topS, int* topI) {
-  using A = typename P::S;
-  const int lane = b.lane, warp = b.warp, kk = b.kk, W = b.W;
-  A left = __shfl_up_sync(0xffffffffu, S[R - 1], 1);
-  A right = __shfl_down_sync(0xffffffffu, S[0], 1);
-  A* const aedges = reinterpret_cast<A*>(b.edges);
-  if (lane == 0) aedges[2 * warp] = S[0];
-  if (lane == 31) aedges[2 * warp + 1] = S[R - 1];
-  __syncthreads();
-  if (lane == 0) left = (warp > 0) ? aedges[2 * warp - 1] : (A)-INFINITY;
-  if (lane == 31) right = (warp + 1 < b.nwarps) ? aedges[2 * warp + 2] : (A)-INFINITY;
-  const A thr = (topI[kk - 1] >= 0) ? (A)topS[kk - 1] : (A)-INFINITY;
+// The same sums one observation at a time, for what is not worth a loop of its
+// own: exact anchors per pair, the FP32 phase (an FP32 anchor every K
+// frequencies), and the bin dump.
+template <int R, int PHASE, class P, bool DUMP>
+__device__ __forceinline__ void accumulate_slow(const TileArgs& args, const Warp<P>& w, const Tile& g,
+                                             const NlTile<R>& nl, int64_t base, int64_t n, const WorkItem& wi) {
+  using Bin = typename P::Bin;
+  using In = typename P::In;
+  const unsigned M = (unsigned)w.M;
+  const int64_t j0 = w.lane * R, first = g.mode == kLine ? g.s + 1 : 0;  // steps from the staged phase to the tile
+  const unsigned col = smem_u32(w.bins), rstride = M * Warp<P>::kBinStride;
+  for (int64_t c = 0; c * 32 < n; ++c) {
+    const Obs<P> o = fetch<P>(args, g.mode, base, n, c * 32 + w.lane);
+    __syncwarp();
+    put<P>(w, 0, record<P>(args, w, g, g.mode, o), o.aw);
+    __syncwarp();
+    const int cnt = (int)((n - c * 32) < 32 ? (n - c * 32) : 32);
+    for (int i = 0; i < cnt; ++i) {
+      const ulonglong2 pd = w.pd[i];
+      const In x = w.aw[i];
+      unsigned m[R];
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int j = (int)b.j0 + r;
-    const int64_t k = s + j;
-    const bool owned = j > 0 && j < W - 1 && k >= wi.f_lo && k < wi.f_hi;
-    const A prev = (r > 0) ? S[r > 0 ? r - 1 : 0] : left;
-    const A next = (r < R - 1) ? S[r < R - 1 ? r + 1 : 0] : right;
-    const bool peak = args.peak_raw ? owned : (owned && S[r] > prev && S[r] >= next);
-    if (peak && S[r] > thr) {
-      const int slot = atomicAdd(&b.misc[1], 1);
-      b.candS[slot] = (double)S[r];
-      b.candI[slot] = (int)((k << key_shift) | extra[r]);
+      for (int r = 0; r < R; ++r) {
+        const int64_t k = g.s + j0 + r;
+        if (g.mode == kExact) {
+          const int64_t kc = k < 0 ? 0 : (k >= w.F ? w.F - 1 : k);
+          m[r] = bin_of_phase(phase_fixed64(__longlong_as_double((long long)pd.x), args.freqs[kc]), M);
+        } else if (g.mode == kFixed) {
+          m[r] = __umulhi(nl_phase(pd, nl.dh[r], nl.dl[r]), M);
+        } else if (PHASE == FPW_PHASE_FP32) {
+          const int64_t ak = (k >= 0) ? k - (k % args.K) : 0;
+          const unsigned long long pa = pd.x + (unsigned long long)(ak - g.s + first) * pd.y;
+          const float d32 = (float)(unsigned)(pd.y >> 32) * 0x1p-32f, p32 = (float)(unsigned)(pa >> 32) * 0x1p-32f;
+          float p = fmaf((float)(k - ak), d32, p32);
+          p = p - floorf(p);
+          const unsigned mm = (unsigned)(p * (float)M);
+          m[r] = mm < M ? mm : M - 1u;
+        } else {
+          m[r] = bin_of_phase(pd.x + (unsigned long long)(first + j0 + r) * pd.y, M);
+        }
+        if (DUMP && k >= wi.f_lo && k < wi.f_hi && k >= args.bins_k0 && k < args.bins_k1)
+          args.bins_out[(k - args.bins_k0) * args.bins_nobs + base + c * 32 + i] = (int32_t)m[r];
+      }
+      Bin v[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) lds(col + (unsigned)r * rstride + m[r] * Warp<P>::kBinStride, v[r]);
+#pragma unroll
+      for (int r = 0; r < R; ++r) sts(col + (unsigned)r * rstride + m[r] * Warp<P>::kBinStride, bin_add(v[r], x));
     }
   }
-  __syncthreads();
-  const int cnt = b.misc[1];
-  if (cnt > 0) {
-    if (warp == 0) warp_merge_topk(topS, topI, kk, b.candS, b.candI, cnt, lane);
-    __syncthreads();
-    if (b.tid == 0) b.misc[1] = 0;
+}
+
+template <int R, int PHASE, class P, bool DUMP>
+__device__ __forceinline__ void accumulate_tile(const TileArgs& args, const Warp<P>& w, const Tile& g,
+                                                const NlTile<R>& nl, int64_t base, int64_t n, const WorkItem& wi) {
+  if (DUMP || PHASE == FPW_PHASE_FP32 || g.mode == kExact)
+    accumulate_slow<R, PHASE, P, DUMP>(args, w, g, nl, base, n, wi);
+  else if (g.mode == kLine)
+    accumulate<R, P, kLine>(args, w, g, nl, base, n, kLine);
+  else if (g.mode == kFixed)
+    accumulate<R, P, kFixed>(args, w, g, nl, base, n, kFixed);
+  else
+    accumulate<R, P, kRecord>(args, w, g, nl, base, n, g.mode);
+}
+
+// Inserts (s, key) into the list topS/topI (kk entries sorted by S descending,
+// then key ascending; key < 0: empty) if it ranks there. One warp, all lanes
+// with the same s and key.
+__device__ __noinline__ void list_insert(double* topS, int* topI, int kk, double s, int key, int lane) {
+  int pos = 0;
+  double up[2];
+  int ui[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int q = lane + 32 * h;
+    const bool in = q < kk;
+    const bool ahead = in && topI[q] >= 0 && ranks_before(topS[q], topI[q], s, key);
+    pos += __popc(__ballot_sync(0xffffffffu, ahead));
+    up[h] = in && q > 0 ? topS[q - 1] : 0.0;
+    ui[h] = in && q > 0 ? topI[q - 1] : 0;
   }
-  __syncthreads();
+  __syncwarp();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int q = lane + 32 * h;
+    if (q < kk && q >= pos) {
+      topS[q] = q == pos ? s : up[h];
+      topI[q] = q == pos ? key : ui[h];
+    }
+  }
+  __syncwarp();
+}
+
+// Step 4: peaks among the frequencies whose right neighbour is known by now
+// (the tile's own except its last, and the previous tile's last), or every
+// owned one in raw mode, ranked into the list. c1, c2: S of the two
+// frequencies before the tile. The ranking key of frequency k is (k <<
+// key_shift) | extra; ce: the extra of the frequency before the tile.
+// floor: no S below it can be among the curve's k best. Returns whether the list
+// changed.
+template <int R, class P>
+__device__ __forceinline__ bool tile_peaks(const TileArgs& args, const Warp<P>& w, const typename P::S (&S)[R],
+                                           const int (&extra)[R], int key_shift, int64_t s, const WorkItem& wi,
+                                           double* topS, int* topI, typename P::S floor,
+                                           typename P::S& c1, typename P::S& c2, int& ce) {
+  using A = typename P::S;
+  const int lane = w.lane, kk = w.kk;
+  // values one and two frequencies left of the lane's first
+  A l1 = __shfl_up_sync(0xffffffffu, S[R - 1], 1);
+  A l2 = R > 1 ? __shfl_up_sync(0xffffffffu, S[R > 1 ? R - 2 : 0], 1) : __shfl_up_sync(0xffffffffu, S[0], 2);
+  int e1 = key_shift ? __shfl_up_sync(0xffffffffu, extra[R - 1], 1) : 0;
+  if (lane == 0) {
+    l1 = c1;
+    l2 = c2;
+    e1 = ce;
+  }
+  if (R == 1 && lane == 1) l2 = c1;
+  c2 = R > 1 ? __shfl_sync(0xffffffffu, S[R > 1 ? R - 2 : 0], 31) : __shfl_sync(0xffffffffu, S[0], 30);
+  c1 = __shfl_sync(0xffffffffu, S[R - 1], 31);
+  if (key_shift) ce = __shfl_sync(0xffffffffu, extra[R - 1], 31);
+  // peaks that beat the k-th best so far, of this item or (floor) of any of the
+  // curve's; the best of them is inserted, round by round, so a tile takes at
+  // most k rounds whatever its peaks' order
+  unsigned todo = 0u;  // bit r: the frequency before position r is a peak to look at
+  A v[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int64_t k = s + (int64_t)(lane * R + r) - 1;
+    v[r] = r > 0 ? S[r > 0 ? r - 1 : 0] : l1;
+    const A left = r > 1 ? S[r > 1 ? r - 2 : 0] : (r == 1 ? l1 : l2);
+    const bool owned = k >= wi.f_lo && k < wi.f_hi;
+    if (owned && (args.peak_raw || (v[r] > left && v[r] >= S[r])) && v[r] >= floor) todo |= 1u << r;
+  }
+  bool changed = false;
+  A bs = (A)-INFINITY;  // the lane's best candidate (lowest key first where equal)
+  int bk = -1, br = 0;
+  for (bool fresh = true;; fresh = false) {
+    const A thr = topI[kk - 1] >= 0 ? (A)topS[kk - 1] : (A)-INFINITY;
+    const int thrk = topI[kk - 1];
+    if (fresh || bk < 0) {
+      if (todo != 0u) {
+        bs = (A)-INFINITY;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int key = (int)(((s + (int64_t)(lane * R + r) - 1) << key_shift) | (r > 0 ? extra[r > 0 ? r - 1 : 0] : e1));
+          const bool beats = v[r] > thr || (v[r] == thr && thrk >= 0 && key < thrk);
+          if ((todo >> r & 1u) && beats && (bk < 0 || v[r] > bs)) {
+            bs = v[r];
+            bk = key;
+            br = r;
+          }
+        }
+        if (bk < 0) todo = 0u;
+      }
+    } else if (!(bs > thr || (bs == thr && thrk >= 0 && bk < thrk))) {
+      bk = -1;
+      todo = 0u;
+    }
+    if (!__any_sync(0xffffffffu, bk >= 0)) break;
+    A ws;
+    const bool mine = warp_best(bs, bk, ws);
+    const unsigned wk = __reduce_min_sync(0xffffffffu, mine ? (unsigned)bk : 0xffffffffu);
+    list_insert(topS, topI, kk, (double)ws, (int)wk, lane);
+    changed = true;
+    if (mine && (unsigned)bk == wk) {
+      todo &= ~(1u << br);
+      bk = -1;
+    }
+  }
+  return changed;
+}
+
+// Step 3: S of the lane's R frequencies, bins cleared for the next tile. The R
+// sums advance together, two bins at a time: a loop short enough to stay in the
+// instruction cache next to the hot loop (a warp reaches it at its own time; with
+// eight bins per frequency unrolled, fetching the code cost short curves a
+// quarter of their time).
+template <int R, class P, bool PLAIN>
+__device__ __forceinline__ void reduce_bins(const Warp<P>& w, typename P::S cal, typename P::S (&S)[R]) {
+  using Bin = typename P::Bin;
+  constexpr unsigned kStride = Warp<P>::kBinStride;
+  const unsigned rstride = (unsigned)w.M * kStride;
+  unsigned a = smem_u32(w.bins);
+  Bin z;
+  bin_zero(z);
+#pragma unroll
+  for (int r = 0; r < R; ++r) S[r] = (typename P::S)0;
+  int m = 0;
+#pragma unroll 1
+  for (; m + 2 <= w.M; m += 2, a += 2 * kStride) {
+    Bin v[R][2];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      lds(a + (unsigned)r * rstride, v[r][0]);
+      lds(a + (unsigned)r * rstride + kStride, v[r][1]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      sts(a + (unsigned)r * rstride, z);
+      sts(a + (unsigned)r * rstride + kStride, z);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) S[r] += PLAIN ? bin_term_plain(v[r][u], cal) : bin_term(v[r][u], cal);
+    }
+  }
+  if (m < w.M) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      Bin v;
+      lds(a + (unsigned)r * rstride, v);
+      sts(a + (unsigned)r * rstride, z);
+      S[r] += bin_term(v, cal);
+    }
+  }
 }
 
 // Item prologue shared by both kernels: invalid curves produce NaN / empty
 // candidates (returns false); otherwise the largest |t| of the curve (sets the
-// grid-linearity tolerance) and cleared top lists.
+// grid-linearity tolerance; 0 where the whole grid is linear for every curve)
+// and cleared top lists.
 template <class P>
-__device__ __forceinline__ bool item_begin(const TileArgs& args, const Block<P>& b, const WorkItem& wi, int64_t base,
-                                           int64_t n, bool grid_bad, int groups, double& tm) {
-  const int T = b.T, tid = b.tid, kk = b.kk;
-  const int64_t F = b.F, c = wi.curve;
-  if (grid_bad || args.curve_bad[c]) {
+__device__ __forceinline__ bool item_begin(const TileArgs& args, const Warp<P>& w, const WorkItem& wi, int64_t base,
+                                           int64_t n, bool grid_bad, bool all_lin, int groups, double& tm) {
+  const int lane = w.lane, kk = w.kk;
+  const int64_t c = wi.curve;
+  if (grid_bad || (args.curve_bad[c] & kCurveBad)) {
     if (args.S_out)
       for (int g = 0; g < groups; ++g)
-        for (int64_t q = wi.f_lo + tid; q < wi.f_hi; q += T)
-          args.S_out[(c * groups + g) * F + q] = __longlong_as_double(0x7ff8000000000000ll);
-    if (kk > 0)
-      for (int g = 0; g < groups; ++g)
-        for (int q = tid; q < kk; q += T) {
-          args.cand_S[(g * args.group_rows + wi.slot) * kk + q] = -INFINITY;
-          args.cand_idx[(g * args.group_rows + wi.slot) * kk + q] = -1;
-        }
-    __syncthreads();
+        for (int64_t q = wi.f_lo + lane; q < wi.f_hi; q += 32)
+          args.S_out[(c * groups + g) * w.F + q] = __longlong_as_double(0x7ff8000000000000ll);
+    for (int g = 0; g < groups; ++g)
+      for (int q = lane; q < kk; q += 32) {
+        args.cand_S[(g * args.group_rows + wi.slot) * kk + q] = -INFINITY;
+        args.cand_idx[(g * args.group_rows + wi.slot) * kk + q] = -1;
+      }
     return false;
   }
-  double m = 0.0;
-  for (int64_t i = tid; i < n; i += T) m = fmax(m, fabs(args.t[base + i]));
-  m = warp_max(m);
-  if (b.lane == 0) b.red[b.warp] = m;
-  for (int q = tid; q < kk * groups; q += T) {
-    const int g = q / kk, j = q % kk;
-    b.topS[g * FPW_MAX_TOPK + j] = -INFINITY;
-    b.topI[g * FPW_MAX_TOPK + j] = -1;
-  }
-  if (tid == 0) b.misc[1] = 0;
-  __syncthreads();
   tm = 0.0;
-  for (int w = 0; w < b.nwarps; ++w) tm = fmax(tm, b.red[w]);
+  if (!all_lin) {
+    double m = 0.0;
+    for (int64_t i = lane; i < n; i += 32) m = fmax(m, fabs(args.t[base + i]));
+    tm = warp_max(m);
+  }
+  __syncwarp();
+  for (int q = lane; q < kk * groups; q += 32) {
+    w.topS[q] = -INFINITY;
+    w.topI[q] = -1;
+  }
+  __syncwarp();
   return true;
 }
 
 template <class P>
-__device__ __forceinline__ void item_end(const TileArgs& args, const Block<P>& b, const WorkItem& wi, int groups) {
-  const int kk = b.kk;
-  if (kk > 0)
-    for (int q = b.tid; q < kk * groups; q += b.T) {
-      const int g = q / kk, j = q % kk;
-      args.cand_S[(g * args.group_rows + wi.slot) * kk + j] = b.topS[g * FPW_MAX_TOPK + j];
-      args.cand_idx[(g * args.group_rows + wi.slot) * kk + j] = b.topI[g * FPW_MAX_TOPK + j];
-    }
-  __syncthreads();
+__device__ __forceinline__ void item_end(const TileArgs& args, const Warp<P>& w, const WorkItem& wi, int groups) {
+  const int kk = w.kk;
+  __syncwarp();
+  for (int q = w.lane; q < kk * groups; q += 32) {
+    const int g = q / kk, j = q % kk;
+    args.cand_S[(g * args.group_rows + wi.slot) * kk + j] = w.topS[q];
+    args.cand_idx[(g * args.group_rows + wi.slot) * kk + j] = w.topI[q];
+  }
 }
 
-// (512, 1) sets the same 128-register ceiling as a bare 512-thread bound; with
-// it the compiler gives every instantiation the registers it needs, where the
-// bare bound led it to hold some to 64 registers and spill.
+// The warp's next item (>= nitems: none): the first by index, warp by warp
+// over the blocks, so that few items spread over all SMs; then from the queue.
+__device__ __forceinline__ int next_item(const TileArgs& args, bool first, int lane) {
+  if (first) return (int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x);
+  unsigned q = 0;
+  if (lane == 0) q = atomicAdd(args.counter, 1u);
+  return (int)(gridDim.x * (blockDim.x >> 5) + __shfl_sync(0xffffffffu, q, 0));
+}
+
+// Does the whole grid lie on the line through its first frequency, for every
+// curve's times (the usual case: a curve's own times are then not looked at)? A
+// frequency is off it by its block's deviation, its anchor's distance, and the
+// rounding of the step over F steps. And do all terms t delta fit record()'s 31
+// bits? Else every tile is looked at, and tiles keep to their blocks.
+__device__ __forceinline__ bool grid_is_linear(const TileArgs& args) {
+  if (!args.rec) return false;
+  const double dev = __uint_as_float(args.grid_dev[0]), tmax = __uint_as_float(args.grid_dev[1]);
+  const double far = __uint_as_float(args.grid_dev[2]);  // units of 2^-96
+  return (dev + far * 0x1p-96) * tmax + (double)args.nfreq * 0x1p-64 <= kGridTolCycles && far * tmax < 0x1p62;
+}
+
+// At most kTileMaxThreads threads a block (wider shapes are launched as more
+// blocks): 168 registers, where 128 made the R = 8 loop spill (N = 85, M = 10:
+// 1.81 -> 1.85e12 evaluations/s).
 template <int R, int PHASE, class P, bool DUMP>
-__global__ void __launch_bounds__(512, 1) tile_kernel(const TileArgs args) {
+__global__ void __launch_bounds__(kTileMaxThreads, 1) tile_kernel(const __grid_constant__ TileArgs args) {
   using Bin = typename P::Bin;
   using A = typename P::S;
+  constexpr int W = 32 * R;
   extern __shared__ __align__(16) unsigned char smem[];
-  const Block<P> b = make_block<R, P>(smem, args);
-  const int64_t F = b.F;
+  const Warp<P> w = make_warp<R, P>(smem, args);
+  const int64_t F = w.F;
   const bool grid_bad = (*(volatile unsigned*)args.status & kStatusGrid) != 0u;
   const A cal = (A)args.inv_alpha2;
+  const bool every_lin = grid_is_linear(args);
+  const bool aligned = args.aligned;
+  const bool plain_prior = args.inv_alpha2 == 0.0 || (args.inv_alpha2 > 0x1p-90 && args.inv_alpha2 < 0x1p+90);
+  const int halo = w.kk > 0 ? 1 : 0;  // peaks need both neighbours of every owned frequency
+  const int M = w.M, j0 = w.lane * R;
 
-  // bins start at zero; every reduce leaves them zero again
-  for (int q = 0; q < R * b.M; ++q) {
-    Bin z;
-    bin_zero(z);
-    *reinterpret_cast<Bin*>(b.my_bins + (size_t)q * b.T8) = z;
-  }
-  zero_padding(b);
-
-  for (;;) {
-    if (b.tid == 0) b.misc[0] = (int)atomicAdd(args.counter, 1u);
-    __syncthreads();
-    const int it = b.misc[0];
-    if (it >= args.nitems) break;
-    const WorkItem wi = args.items[it];
+  for (int it = next_item(args, true, w.lane); it < args.nitems; it = next_item(args, false, w.lane)) {
+    WorkItem wi = args.items[it];
     const int c = wi.curve;
     int64_t base = 0, n = args.n_single;
     if (args.offsets) {
@@ -630,65 +908,52 @@ __global__ void __launch_bounds__(512, 1) tile_kernel(const TileArgs args) {
       n = args.offsets[c + 1] - base;
     }
     double tm;
-    if (!item_begin(args, b, wi, base, n, grid_bad, 1, tm)) continue;
-    const bool resident = n <= b.NC;
-    bool staged_lin = false;
+    if (!item_begin(args, w, wi, base, n, grid_bad, every_lin, 1, tm)) continue;
+    const bool plain = !(args.curve_bad[c] & kCurveWide) && plain_prior;
+    A c1 = (A)-INFINITY, c2 = (A)-INFINITY;
+    int ce = 0;
+    const int64_t f_end = wi.f_hi;
+    int64_t s = (int64_t)wi.f_lo - halo;
+    int64_t q = aligned ? (unsigned)wi.f_lo / (unsigned)args.anchor_span : 0;  // the range's anchor block
+    float delta = aligned && args.rec && wi.f_lo < f_end ? args.block_delta[q] : 0.f;
+    while (wi.f_lo < f_end) {
+      if (aligned) wi.f_hi = (int32_t)min(f_end, (q + 1) * args.anchor_span);
+      NlTile<R> nl;
+      const Tile g = make_tile<R, P>(args, w, s, q, delta, tm, every_lin, aligned, nl);
+      // the next tile: on from this one, or the start of the next block's range
+      const bool last = s + W >= (int64_t)wi.f_hi + halo;
+      const int64_t sn = last ? (int64_t)wi.f_hi - halo : s + W, lon = last ? wi.f_hi : wi.f_lo;
+      if (aligned && last) {
+        ++q;
+        if (args.rec && lon < f_end) delta = args.block_delta[q];
+      }
+      const unsigned long long floor = w.kk > 0 ? curve_floor(args, c) : 0ull;
+      accumulate_tile<R, PHASE, P, DUMP>(args, w, g, nl, base, n, wi);
 
-    for (int64_t s = (int64_t)wi.f_lo - 1; s + 1 < wi.f_hi; s += b.W - 2) {
-      const int64_t a = s < 0 ? 0 : s;
-      const double fa = args.freqs[a];
-      const bool lin = tile_is_linear<R>(args, b, s, a, fa, tm);
-      accumulate_tile<R, PHASE, P, DUMP>(args, b, s, a, fa, lin, resident && staged_lin && lin, staged_lin, base, n,
-                                         wi);
-
-      // reduce to S (and clear the bins for the next tile); S and the peak test
-      // stay in the policy's reduce type
+      // S and the peak test stay in the policy's reduce type
       A S[R];
+      if (plain)
+        reduce_bins<R, P, true>(w, cal, S);
+      else
+        reduce_bins<R, P, false>(w, cal, S);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        A acc = (A)0;
-        unsigned char* col = b.my_bins + (size_t)r * b.MT8;
-        Bin z;
-        bin_zero(z);
-        int m = 0;
-        for (; m + 8 <= b.M; m += 8) {  // eight bins loaded before any is cleared: their loads overlap
-          Bin v[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) v[u] = *reinterpret_cast<const Bin*>(col + (size_t)(m + u) * b.T8);
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            *reinterpret_cast<Bin*>(col + (size_t)(m + u) * b.T8) = z;
-            acc += bin_term(v[u], cal);
-          }
-        }
-        for (; m < b.M; ++m) {
-          Bin* p = reinterpret_cast<Bin*>(col + (size_t)m * b.T8);
-          const Bin v = *p;
-          *p = z;
-          acc += bin_term(v, cal);
-        }
-        const int64_t k = s + (int64_t)b.j0 + r;
-        S[r] = (k >= 0 && k < F) ? acc : (A)-INFINITY;
+        const int64_t k = s + (int64_t)(j0 + r);
+        if (args.S_out && k >= wi.f_lo && k < wi.f_hi) args.S_out[(int64_t)c * F + k] = (double)S[r];
+        if (k < 0 || k >= F) S[r] = (A)-INFINITY;
       }
-      // dense output of owned frequencies
-      if (args.S_out) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const int j = (int)b.j0 + r;
-          const int64_t k = s + j;
-          if (j > 0 && j < b.W - 1 && k >= wi.f_lo && k < wi.f_hi) args.S_out[(int64_t)c * F + k] = (double)S[r];
-        }
-      }
-      if (b.kk > 0) {
+      if (w.kk > 0) {
         int zero[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) zero[r] = 0;
-        tile_peaks<R, P>(args, b, S, zero, 0, s, wi, b.topS, b.topI);
-      } else {
-        __syncthreads();
+        if (tile_peaks<R, P>(args, w, S, zero, 0, s, wi, w.topS, w.topI, floor_value<A>(floor), c1, c2, ce))
+          raise_floor(args, c, w.topS, w.topI, w.kk, w.lane);
       }
+      if (last) c1 = c2 = (A)-INFINITY;
+      s = sn;
+      wi.f_lo = (int32_t)lon;
     }
-    item_end(args, b, wi, 1);
+    item_end(args, w, wi, 1);
   }
 }
 
@@ -696,10 +961,7 @@ __global__ void __launch_bounds__(512, 1) tile_kernel(const TileArgs args) {
 // bins; for each requested group g (M = M_max / g) it reports, per frequency,
 // the largest S over the g bin offsets and that offset (ranking key
 // (k << 6) | offset). FP32 sums. At most 256 threads per block (the host
-// rejects more): with that bound the compiler keeps the combination's
-// registers (72-114) instead of spilling them, which it did at 40 registers
-// under a 512-thread bound.
-constexpr int kMultiMaxThreads = 256;
+// rejects more): that bound leaves the combination the registers it needs.
 // Several-M combinations compiled for one M_max and three groups: the ones
 // Section 3.4 suggests (M_max = 60 or 40, giving M = 20, 10 and 4) and the
 // M = 20, 10, 5 split of M_max = 20. SPEC 0 is the generic combination.
@@ -724,9 +986,9 @@ struct MultiSpec<3> {
 template <int G, int M, int MX>
 __device__ __forceinline__ void fixed_window(const float2 (&Q)[MX], float (&acc)[G], float cal) {
   if constexpr (M >= G) {
-    acc[(M + 1) % G] += bin_term(f2sub(Q[M], Q[M - G]), cal);
+    acc[(M + 1) % G] += bin_term_plain(f2sub(Q[M], Q[M - G]), cal);
   } else if constexpr (M == G - 1) {
-    acc[0] += bin_term(f2sub(Q[M], make_float2(0.f, 0.f)), cal);
+    acc[0] += bin_term_plain(f2sub(Q[M], make_float2(0.f, 0.f)), cal);
   }
 }
 
@@ -737,7 +999,7 @@ __device__ __forceinline__ void fixed_finish(const float2 (&Q)[MX], float (&acc)
                                              int& bo) {
   const float2 total = Q[MX - 1];
 #pragma unroll
-  for (int o = 1; o < G; ++o) acc[o] += bin_term(bin_add(f2sub(total, Q[MX - G + o - 1]), Q[o - 1]), cal);
+  for (int o = 1; o < G; ++o) acc[o] += bin_term_plain(bin_add(f2sub(total, Q[MX - G + o - 1]), Q[o - 1]), cal);
   best = -INFINITY;
   bo = 0;
 #pragma unroll
@@ -797,7 +1059,7 @@ __device__ __forceinline__ void fixed_chunks(float2* col, int st, float2 (&Q)[MX
 // sums, then per group and offset the windows in order, the wrapping one last),
 // so S is the same bit for bit, while each bin costs one shared-memory read and
 // one store instead of a read-modify-write for the prefix sums, a read per
-// group and a clearing store.
+// group and a clearing store. Curves whose weights allow bin_term_plain only.
 template <int SPEC>
 __device__ __forceinline__ void combine_fixed(float2* col, int st, float cal, float (&best)[3], int (&bo)[3]) {
   using SP = MultiSpec<SPEC>;
@@ -821,29 +1083,132 @@ __device__ __forceinline__ void combine_fixed(float2* col, int st, float cal, fl
   fixed_finish<G2, MX>(Q, a2, cal, best[2], bo[2]);
 }
 
+// The combination of one tile's M_max bins for any groups: in-place prefix sums first, then per
+// group and offset the windows in order (window j of offset o spans bins [j g +
+// o, j g + o + g - 1]; its sum is Q[end] - Q[start - 1], and its end is the next
+// window's start - 1), the one that wraps past bin M_max - 1 last. The lane's R
+// frequencies advance together. Short loops, as in reduce_bins.
+template <int R>
+__device__ __forceinline__ void prefix_bins(const Warp<AccF32>& w, float2 (&total)[R]) {
+  constexpr unsigned kStride = Warp<AccF32>::kBinStride;
+  const unsigned rstride = (unsigned)w.M * kStride;
+  unsigned a = smem_u32(w.bins);
+#pragma unroll
+  for (int r = 0; r < R; ++r) total[r] = make_float2(0.f, 0.f);
+  int m = 0;
+#pragma unroll 1
+  for (; m + 4 <= w.M; m += 4, a += 4 * kStride) {  // four bins loaded before any is stored back
+    float2 v[R][4];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) lds(a + (unsigned)r * rstride + u * kStride, v[r][u]);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        total[r] = bin_add(total[r], v[r][u]);
+        sts(a + (unsigned)r * rstride + u * kStride, total[r]);
+      }
+  }
+#pragma unroll 1
+  for (; m < w.M; ++m, a += kStride)
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      float2 v;
+      lds(a + (unsigned)r * rstride, v);
+      total[r] = bin_add(total[r], v);
+      sts(a + (unsigned)r * rstride, total[r]);
+    }
+}
 
+// S_g of the lane's R frequencies: the largest S over the gs offsets (ties to
+// the lower). OB offsets advance together (R OB independent sums: a window's
+// load, reciprocal and addition take ~110 clk one after the other); offsets past
+// gs - 1 repeat the last one, which changes nothing.
+template <int R, int OB, bool PLAIN>
+__device__ __forceinline__ void best_offset(const Warp<AccF32>& w, const float2 (&total)[R], int gs, float cal,
+                                            float (&S)[R], int (&off)[R]) {
+  constexpr unsigned kStride = Warp<AccF32>::kBinStride;
+  const unsigned rstride = (unsigned)w.M * kStride, col = smem_u32(w.bins), step = (unsigned)gs * kStride;
+  const int Mg = w.M / gs;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    S[r] = -INFINITY;
+    off[r] = 0;
+  }
+#pragma unroll 1
+  for (int o0 = 0; o0 < gs; o0 += OB) {
+    float2 prev[OB][R], q[OB][R];
+    float acc[OB][R];
+    unsigned e[OB];
+#pragma unroll
+    for (int b = 0; b < OB; ++b) {
+      const int o = o0 + b < gs ? o0 + b : gs - 1;
+      e[b] = col + (unsigned)(o + gs - 1) * kStride;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        prev[b][r] = make_float2(0.f, 0.f);
+        if (o > 0) lds(col + (unsigned)r * rstride + (unsigned)(o - 1) * kStride, prev[b][r]);
+        q[b][r] = make_float2(0.f, 0.f);
+        if (Mg > 1) lds(e[b] + (unsigned)r * rstride, q[b][r]);
+        acc[b][r] = 0.f;
+      }
+    }
+    const auto add = [&](float& a, float2 d) { a += PLAIN ? bin_term_plain(d, cal) : bin_term(d, cal); };
+    float2 q0[OB][R];
+#pragma unroll
+    for (int b = 0; b < OB; ++b)
+#pragma unroll
+      for (int r = 0; r < R; ++r) q0[b][r] = prev[b][r];
+#pragma unroll 1
+    for (int j = 1; j < Mg; ++j) {  // the windows before the last; the next one's end is loaded ahead
+#pragma unroll
+      for (int b = 0; b < OB; ++b) {
+        e[b] += step;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          float2 n = make_float2(0.f, 0.f);
+          if (j + 1 < Mg) lds(e[b] + (unsigned)r * rstride, n);
+          add(acc[b][r], f2sub(q[b][r], prev[b][r]));
+          prev[b][r] = q[b][r];
+          q[b][r] = n;
+        }
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < OB; ++b)
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        // the last window: up to bin M_max - 1, and for o > 0 on to bin o - 1
+        add(acc[b][r], bin_add(f2sub(total[r], prev[b][r]), q0[b][r]));
+        if (acc[b][r] > S[r]) {
+          S[r] = acc[b][r];
+          off[r] = o0 + b;
+        }
+      }
+  }
+}
 
 template <int R, int PHASE, int SPEC>
-__global__ void __launch_bounds__(kMultiMaxThreads, 2) tile_kernel_multi(const TileArgs args) {
+__global__ void __launch_bounds__(kMultiMaxThreads, 1) tile_kernel_multi(const __grid_constant__ TileArgs args) {
   using P = AccF32;
   using A = float;
-  using A2 = float2;
+  constexpr int W = 32 * R;
   extern __shared__ __align__(16) unsigned char smem[];
-  const Block<P> b = make_block<R, P>(smem, args);
-  const int64_t F = b.F;
-  const int Mx = b.M, ng = args.ngroups;
+  const Warp<P> w = make_warp<R, P>(smem, args);
+  const int64_t F = w.F;
+  const int Mx = w.M, ng = args.ngroups, kk = w.kk;
   const bool grid_bad = (*(volatile unsigned*)args.status & kStatusGrid) != 0u;
   const A cal = (A)args.inv_alpha2;
+  const bool every_lin = grid_is_linear(args);
+  const bool aligned = args.aligned;
+  const bool plain_prior = args.inv_alpha2 == 0.0 || (args.inv_alpha2 > 0x1p-90 && args.inv_alpha2 < 0x1p+90);
+  const int halo = kk > 0 ? 1 : 0;
+  const int j0 = w.lane * R;
 
-  for (int q = 0; q < R * Mx; ++q) *reinterpret_cast<A2*>(b.my_bins + (size_t)q * b.T8) = make_float2(0.f, 0.f);
-  zero_padding(b);
-
-  for (;;) {
-    if (b.tid == 0) b.misc[0] = (int)atomicAdd(args.counter, 1u);
-    __syncthreads();
-    const int it = b.misc[0];
-    if (it >= args.nitems) break;
-    const WorkItem wi = args.items[it];
+  for (int it = next_item(args, true, w.lane); it < args.nitems; it = next_item(args, false, w.lane)) {
+    WorkItem wi = args.items[it];
     const int c = wi.curve;
     int64_t base = 0, n = args.n_single;
     if (args.offsets) {
@@ -851,127 +1216,113 @@ __global__ void __launch_bounds__(kMultiMaxThreads, 2) tile_kernel_multi(const T
       n = args.offsets[c + 1] - base;
     }
     double tm;
-    if (!item_begin(args, b, wi, base, n, grid_bad, ng, tm)) continue;
-    const bool resident = n <= b.NC;
-    bool staged_lin = false;
-
-    for (int64_t s = (int64_t)wi.f_lo - 1; s + 1 < wi.f_hi; s += b.W - 2) {
-      const int64_t a = s < 0 ? 0 : s;
-      const double fa = args.freqs[a];
-      const bool lin = tile_is_linear<R>(args, b, s, a, fa, tm);
-      accumulate_tile<R, PHASE, P, false>(args, b, s, a, fa, lin, resident && staged_lin && lin, staged_lin, base,
-                                          n, wi);
+    if (!item_begin(args, w, wi, base, n, grid_bad, every_lin, ng, tm)) continue;
+    const bool plain = !(args.curve_bad[c] & kCurveWide) && plain_prior;
+    // S and offset of the two frequencies before the tile, per group (lane g holds group g's)
+    A carry1 = -INFINITY, carry2 = -INFINITY;
+    int carrye = 0;
+    const int64_t f_end = wi.f_hi;
+    int64_t s = (int64_t)wi.f_lo - halo;
+    int64_t q = aligned ? (unsigned)wi.f_lo / (unsigned)args.anchor_span : 0;  // the range's anchor block
+    float delta = aligned && args.rec && wi.f_lo < f_end ? args.block_delta[q] : 0.f;
+    while (wi.f_lo < f_end) {
+      if (aligned) wi.f_hi = (int32_t)min(f_end, (q + 1) * args.anchor_span);
+      NlTile<R> nl;
+      const Tile g0 = make_tile<R, P>(args, w, s, q, delta, tm, every_lin, aligned, nl);
+      // the next tile: on from this one, or the start of the next block's range
+      const bool last = s + W >= (int64_t)wi.f_hi + halo;
+      const int64_t sn = last ? (int64_t)wi.f_hi - halo : s + W, lon = last ? wi.f_hi : wi.f_lo;
+      if (aligned && last) {
+        ++q;
+        if (args.rec && lon < f_end) delta = args.block_delta[q];
+      }
+      accumulate_tile<R, PHASE, P, false>(args, w, g0, nl, base, n, wi);
 
       // the reported S of group g per owned frequency, and the peaks
       auto emit = [&](int g, const A (&S)[R], const int (&off)[R]) {
         if (args.S_out) {
 #pragma unroll
           for (int r = 0; r < R; ++r) {
-            const int j = (int)b.j0 + r;
-            const int64_t k = s + j;
-            if (j > 0 && j < b.W - 1 && k >= wi.f_lo && k < wi.f_hi)
-              args.S_out[((int64_t)c * ng + g) * F + k] = (double)S[r];
+            const int64_t k = s + (int64_t)(j0 + r);
+            if (k >= wi.f_lo && k < wi.f_hi) args.S_out[((int64_t)c * ng + g) * F + k] = (double)S[r];
           }
         }
-        if (b.kk > 0) tile_peaks<R, P>(args, b, S, off, 6, s, wi, b.topS + g * FPW_MAX_TOPK, b.topI + g * FPW_MAX_TOPK);
+        if (kk > 0) {
+          A c1 = __shfl_sync(0xffffffffu, carry1, g), c2 = __shfl_sync(0xffffffffu, carry2, g);
+          int ce = __shfl_sync(0xffffffffu, carrye, g);
+          const int64_t row = (int64_t)c * ng + g;
+          if (tile_peaks<R, P>(args, w, S, off, 6, s, wi, w.topS + g * kk, w.topI + g * kk,
+                               floor_value<A>(curve_floor(args, row)), c1, c2, ce))
+            raise_floor(args, row, w.topS + g * kk, w.topI + g * kk, kk, w.lane);
+          if (w.lane == g) {
+            carry1 = c1;
+            carry2 = c2;
+            carrye = ce;
+          }
+        }
       };
       if constexpr (SPEC != 0) {
-        // compiled (M_max, groups): one pass per slot, bins cleared on the way
-        A Sg[3][R];
-        int offg[3][R];
+        if (plain) {
+          A Sg[3][R];
+          int offg[3][R];
 #pragma unroll 1
-        for (int r = 0; r < R; ++r) {  // one slot at a time: the pass holds its prefix sums in registers
-          float best[3];
-          int bo[3];
-          combine_fixed<SPEC>(reinterpret_cast<A2*>(b.my_bins + (size_t)r * b.MT8), b.T, cal, best, bo);
-          const int64_t k = s + (int64_t)b.j0 + r;
+          for (int r = 0; r < R; ++r) {  // one frequency at a time: the pass holds its prefix sums in registers
+            float best[3];
+            int bo[3];
+            combine_fixed<SPEC>(reinterpret_cast<float2*>(w.bins) + r * Mx * 32, 32, cal, best, bo);
+            const int64_t k = s + (int64_t)(j0 + r);
 #pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            Sg[q][r] = (k >= 0 && k < F) ? best[q] : (A)-INFINITY;
-            offg[q][r] = bo[q];
-          }
-        }
-#pragma unroll
-        for (int g = 0; g < 3; ++g) emit(g, Sg[g], offg[g]);
-      } else {
-        // inclusive prefix sums Q[m] of the M_max bins, in place, per r; eight
-        // bins are loaded before any of them is stored back, so the loads of a
-        // chunk are in flight together (the bins of one thread form a dependent
-        // chain otherwise: a load cannot pass the previous bin's store)
-        float2 total[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          A2* col = reinterpret_cast<A2*>(b.my_bins + (size_t)r * b.MT8);
-          const int st = b.T;  // stride between bins, in A2 units
-          A2 run = make_float2(0.f, 0.f);
-          int m = 0;
-          for (; m + 8 <= Mx; m += 8) {
-            A2 v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = col[(m + u) * st];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              run = bin_add(run, v[u]);
-              col[(m + u) * st] = run;
+            for (int q = 0; q < 3; ++q) {
+              Sg[q][r] = (k >= 0 && k < F) ? best[q] : (A)-INFINITY;
+              offg[q][r] = bo[q];
             }
           }
-          for (; m < Mx; ++m) {
-            run = bin_add(run, col[m * st]);
-            col[m * st] = run;
-          }
-          total[r] = run;
-        }
-        for (int g = 0; g < ng; ++g) {
-          const int gs = args.group_g[g], Mg = Mx / gs;
-          A S[R];
-          int off[R];
+#pragma unroll 1
+          for (int g = 0; g < 3; ++g) {
+            A S[R];
+            int off[R];
 #pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const A2* col = reinterpret_cast<const A2*>(b.my_bins + (size_t)r * b.MT8);
-            const int st = b.T;
-            A best = (A)-INFINITY;
-            int bo = 0;
-            for (int o = 0; o < gs; ++o) {
-              A acc = (A)0;
-              // window j spans bins [j gs + o, j gs + o + gs - 1]: its sum is
-              // Q[end] - Q[start - 1], and its end is the next window's start - 1,
-              // so one prefix value is read per window (carried in `prev`)
-              const A2 q0 = (o > 0) ? col[(o - 1) * st] : make_float2(0.f, 0.f);
-              A2 prev = q0;
-              // the windows that end below bin M_max: independent loads (no
-              // stores here), unrolled so that they issue together; the terms
-              // are added in window order
-              const int nin = (o > 0) ? Mg - 1 : Mg;
-              const A2* e = col + (size_t)(o + gs - 1) * st;
-#pragma unroll 4
-              for (int j = 0; j < nin; ++j) {
-                const A2 q = e[(size_t)j * gs * st];
-                acc += bin_term(f2sub(q, prev), cal);
-                prev = q;
-              }
-              // o >= 1: the last window wraps past bin M_max - 1 and ends at o - 1
-              if (o > 0) acc += bin_term(bin_add(f2sub(total[r], prev), q0), cal);
-              if (acc > best) {
-                best = acc;
-                bo = o;
-              }
+            for (int r = 0; r < R; ++r) {
+              S[r] = Sg[g][r];
+              off[r] = offg[g][r];
             }
-            const int64_t k = s + (int64_t)b.j0 + r;
-            S[r] = (k >= 0 && k < F) ? best : (A)-INFINITY;
-            off[r] = bo;
+            emit(g, S, off);
           }
-          emit(g, S, off);
-        }
-        // clear the bins for the next tile
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          A2* col = reinterpret_cast<A2*>(b.my_bins + (size_t)r * b.MT8);
-          for (int m = 0; m < Mx; ++m) col[m * b.T] = make_float2(0.f, 0.f);
         }
       }
-      __syncthreads();
+      float2 total[R];
+      if (SPEC == 0 || !plain) prefix_bins<R>(w, total);
+#pragma unroll 1
+      for (int g = 0; g < ng && (SPEC == 0 || !plain); ++g) {
+        A S[R];
+        int off[R];
+        const int gs = args.group_g[g];
+        // as many offsets together as leave the registers for R frequencies each
+        constexpr int kOb = R <= 3 ? 3 : (R <= 5 ? 2 : 1);
+        if (!plain)
+          best_offset<R, 1, false>(w, total, gs, cal, S, off);
+        else if (gs == 1)
+          best_offset<R, 1, true>(w, total, gs, cal, S, off);
+        else if (R <= 2 && gs % 5 == 0)
+          best_offset<R, R <= 2 ? 5 : 1, true>(w, total, gs, cal, S, off);
+        else if (R <= 3 && gs % 3 != 0 && gs % 2 == 0)
+          best_offset<R, 2, true>(w, total, gs, cal, S, off);
+        else
+          best_offset<R, kOb, true>(w, total, gs, cal, S, off);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int64_t k = s + (int64_t)(j0 + r);
+          if (k < 0 || k >= F) S[r] = (A)-INFINITY;
+        }
+        emit(g, S, off);
+      }
+      // clear the bins for the next tile
+      for (int q = 0; q < R * Mx && (SPEC == 0 || !plain); ++q) reinterpret_cast<float2*>(w.bins)[q * 32] = make_float2(0.f, 0.f);
+      if (last) carry1 = carry2 = -INFINITY;
+      s = sn;
+      wi.f_lo = (int32_t)lon;
     }
-    item_end(args, b, wi, ng);
+    item_end(args, w, wi, ng);
   }
 }
 
