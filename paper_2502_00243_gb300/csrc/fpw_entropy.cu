@@ -17,6 +17,7 @@ namespace {
 
 constexpr int kEntThreads = 128;
 constexpr int kEntChunk = 256;
+constexpr unsigned kEntTable = 256;  // counts whose logarithm is read from a table
 
 // H from bin counts: log N - (1/N) sum_m N_m log N_m, in FP32 (the count
 // terms are exact integers; the logarithms carry the rounding).
@@ -24,102 +25,128 @@ __device__ __forceinline__ float entropy_from_counts_sum(float sum_clogc, float 
   return N > 0.f ? logf(N) - sum_clogc / N : 0.f;
 }
 
+// One more in a count of this thread's, and its value.
+__device__ __forceinline__ void count_up(unsigned a) { asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(a) : "memory"); }
+__device__ __forceinline__ unsigned read_count(unsigned a) {
+  unsigned v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+
 // R consecutive frequencies per thread, blocks of kEntThreads R frequencies;
-// counts per (frequency slot, bin, thread) as 32-bit integers, [r][m][thread]
-// (conflict-free). Per staged observation the block holds the exact anchor
-// phase at its first frequency, P_i = frac(t_i f_0), and the step D_i =
-// frac(t_i df) as 64-bit fixed point; where the block's frequencies lie on the
-// linear grid (the tile kernels' bound on the phase error) frequency j of the
-// block has phase P_i + j D_i (mod 2^64), as in the periodogram kernels, else
-// the exact anchor at its own frequency. One observation per iteration: its R
-// counts (in disjoint slots) are all loaded before any store, and the next
-// observation's staged data is loaded before them.
+// counts per (bin, frequency slot, thread) as 32-bit integers, [m][r][thread]
+// (conflict-free). Anchors lie every `span` frequencies (a multiple of the
+// block's: the phases, and with them the counts, do not depend on the launch).
+// Per staged observation the block holds the exact anchor phase P_i = frac(t_i
+// f_a) and the step D_i = frac(t_i df) as 64-bit fixed point; where the block's
+// frequencies lie on the linear grid (the tile kernels' bound on the phase
+// error) frequency j past the anchor has phase P_i + j D_i (mod 2^64), else the
+// exact anchor at its own frequency.
+//
+// Bound by the instructions and the shared-memory pipe together, about 2.8
+// clocks per SM and 32 counts. A count is one red.shared.add: nothing comes
+// back, so an observation's R counts wait for nothing (load, add and store ran
+// M = 20 at 2.49e12 counts/s, this at 3.05e12; 1000 times x 1e6 frequencies).
+// With the slots inside the bin, r T is an offset of the instruction; outside
+// it the address cost one more (2.87e12). Two 16-bit counts to a word, for
+// twice the blocks per SM, cost three more (2.10e12), phases by a tree of
+// 64-bit adds the shifts (2.74e12), the bin from a 32 x 32 -> 64 product
+// instead of its upper half 2.77e12. Four observations a trip against two: 6 %.
 template <int R>
 __global__ void __launch_bounds__(kEntThreads) entropy_dense_kernel(const double* t, int64_t n, const double* freqs,
-                                                                    int64_t nfreq, int M, float* H_out) {
+                                                            int64_t nfreq, int M, int span, float* H_out) {
   extern __shared__ __align__(16) unsigned char smem[];
   ulonglong2* const sPD = reinterpret_cast<ulonglong2*>(smem);
-  unsigned* const cnt = reinterpret_cast<unsigned*>(sPD + kEntChunk + 1);  // one record of padding after the chunk
-  __shared__ double s_tm[kEntThreads / 32];
+  float* const logq = reinterpret_cast<float*>(sPD + kEntChunk + 1);  // one record of padding after the chunk
+  unsigned* const cnt = reinterpret_cast<unsigned*>(logq + kEntTable);
+  __shared__ unsigned long long s_tm[kEntThreads / 32];
+  __shared__ double s_df;
+  constexpr int T = kEntThreads;
   const int tid = threadIdx.x;
-  const int64_t f0 = (int64_t)blockIdx.x * (kEntThreads * R);
-  const int j0 = tid * R;  // the thread's first frequency within the block
-  const double fa = freqs[f0];
-  const double df = (nfreq > 1) ? (freqs[nfreq - 1] - freqs[0]) / (double)(nfreq - 1) : 0.0;
-  double fk[R];
+  const int64_t f0 = (int64_t)blockIdx.x * (T * R);
+  const int64_t fanchor = f0 & -(int64_t)span;
+  const int j0 = (int)(f0 - fanchor) + tid * R;  // the thread's first frequency past the anchor
+  const double fa = freqs[fanchor];
+  // max |t| as the largest bit pattern (NaN left out), and one division a block: a warp's binary64
+  // instruction occupies the SM for about 20 clocks
+  unsigned long long tb = 0ull;
+  for (int64_t i = tid; i < n; i += T) {
+    const unsigned long long v = (unsigned long long)__double_as_longlong(t[i]) & 0x7fffffffffffffffull;
+    if (v <= 0x7ff0000000000000ull && v > tb) tb = v;
+  }
+  double dev[R];  // of frequencies f0 + tid + r T (coalesced), |f - f on the line|
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const int64_t k = f0 + j0 + r;
-    fk[r] = freqs[k < nfreq ? k : nfreq - 1];
+    const int64_t k = f0 + tid + r * T;
+    dev[r] = freqs[k < nfreq ? k : nfreq - 1];
   }
-  double tm = 0.0;
-  for (int64_t i = tid; i < n; i += kEntThreads) tm = fmax(tm, fabs(t[i]));
+  if (tid == 0) s_df = (nfreq > 1) ? (freqs[nfreq - 1] - freqs[0]) / (double)(nfreq - 1) : 0.0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) tm = fmax(tm, __shfl_xor_sync(0xffffffffu, tm, o));
-  if ((tid & 31) == 0) s_tm[tid >> 5] = tm;
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(0xffffffffu, tb, o);
+    tb = v > tb ? v : tb;
+  }
+  if ((tid & 31) == 0) s_tm[tid >> 5] = tb;
+  for (int q = tid; q < (int)kEntTable; q += T) logq[q] = q > 1 ? logf((float)q) : 0.f;
+  unsigned* const mine = cnt + tid;  // this thread's column of the [r][m][thread] counts
+  for (int q = 0; q < R * M; ++q) mine[q * T] = 0u;
   __syncthreads();
-  tm = 0.0;
-#pragma unroll
-  for (int q = 0; q < kEntThreads / 32; ++q) tm = fmax(tm, s_tm[q]);
+  tb = s_tm[0];
+  for (int q = 1; q < T / 32; ++q) tb = s_tm[q] > tb ? s_tm[q] : tb;
+  const double tm = __longlong_as_double((long long)tb), df = s_df;
   bool nonlin = false;
+  double x = (double)((int)(f0 - fanchor) + tid);
 #pragma unroll
-  for (int r = 0; r < R; ++r)
-    if (f0 + j0 + r < nfreq && fabs(fk[r] - fma((double)(j0 + r), df, fa)) * tm > kGridTolCycles) nonlin = true;
+  for (int r = 0; r < R; ++r) {
+    if (f0 + tid + r * T < nfreq && fabs(dev[r] - fma(x, df, fa)) * tm > kGridTolCycles) nonlin = true;
+    x += (double)T;
+  }
   const bool lin = !__syncthreads_or(nonlin);
-  const int MT = M * kEntThreads;
-  for (int q = 0; q < R * M; ++q) cnt[q * kEntThreads + tid] = 0u;
+  const unsigned col = (unsigned)__cvta_generic_to_shared(mine);
+  constexpr unsigned step = 4u * (unsigned)(T * R);
   for (int64_t o = 0; o < n; o += kEntChunk) {
     const int c = (int)((n - o) < kEntChunk ? (n - o) : kEntChunk);
-    __syncthreads();
-    for (int i = tid; i < c; i += kEntThreads) {
+    if (o > 0) __syncthreads();
+    for (int i = tid; i < c; i += T) {
       const double ti = t[o + i];
       sPD[i] = lin ? make_ulonglong2(phase_fixed64(ti, fa), phase_fixed64(ti, df))
                    : make_ulonglong2((unsigned long long)__double_as_longlong(ti), 0ull);
     }
     if (tid == 0) sPD[c] = make_ulonglong2(0ull, 0ull);  // read by the last iteration's prefetch, never used
     __syncthreads();
-    unsigned* const mine = cnt + tid;  // this thread's column of the [r][m][thread] counts
     if (lin) {
       ulonglong2 pd = sPD[0];
-#pragma unroll 2
+#pragma unroll 4
       for (int i = 0; i < c; ++i) {
         const ulonglong2 pdn = sPD[i + 1];  // i + 1 <= c <= kEntChunk: staged or the zeroed record
         // the R phases are independent multiply-adds (no serial chain of 64-bit adds)
-        const unsigned long long phi0 = pd.x + (unsigned long long)j0 * pd.y;
-        unsigned* sl[R];
+        unsigned long long phi[R];
+        phi[0] = pd.x + (unsigned long long)j0 * pd.y;
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-          sl[r] = mine + r * MT + bin_of_phase(phi0 + (unsigned long long)r * pd.y, (unsigned)M) * kEntThreads;
-        unsigned v[R];
+        for (int r = 1; r < R; ++r) phi[r] = phi[0] + (unsigned long long)r * pd.y;
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = *sl[r];
-#pragma unroll
-        for (int r = 0; r < R; ++r) *sl[r] = v[r] + 1u;
+        for (int r = 0; r < R; ++r) count_up(col + 4u * (unsigned)(r * T) + bin_of_phase(phi[r], (unsigned)M) * step);
         pd = pdn;
       }
     } else {
       for (int i = 0; i < c; ++i) {
         const double ti = __longlong_as_double((long long)sPD[i].x);
-        unsigned* sl[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-          sl[r] = mine + r * MT + bin_of_phase(phase_fixed64(ti, fk[r]), (unsigned)M) * kEntThreads;
-        unsigned v[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = *sl[r];
-#pragma unroll
-        for (int r = 0; r < R; ++r) *sl[r] = v[r] + 1u;
+        for (int r = 0; r < R; ++r) {
+          const int64_t k = fanchor + j0 + r;
+          count_up(col + 4u * (unsigned)(r * T) + bin_of_phase(phase_fixed64(ti, freqs[k < nfreq ? k : nfreq - 1]), (unsigned)M) * step);
+        }
       }
     }
   }
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const int64_t k = f0 + j0 + r;
+    const int64_t k = fanchor + j0 + r;
     if (k < nfreq) {
       float s = 0.f;
       for (int m = 0; m < M; ++m) {
-        const unsigned q = cnt[r * MT + m * kEntThreads + tid];
-        if (q > 1u) s += (float)q * logf((float)q);
+        const unsigned q = read_count(col + 4u * (unsigned)(r * T) + (unsigned)m * step);
+        if (q > 1u) s += (float)q * (q < kEntTable ? logq[q] : logf((float)q));
       }
       H_out[k] = entropy_from_counts_sum(s, (float)n);
     }
@@ -180,26 +207,29 @@ __global__ void __launch_bounds__(kPeakWarps * 32) entropy_peaks_kernel(const in
 
 }  // namespace
 
-cudaError_t launch_entropy_dense(const double* t, int64_t n, const double* freqs, int64_t nfreq, int M, float* H_out,
-                                 cudaStream_t st) {
+cudaError_t launch_entropy_dense(const double* t, int64_t n, const double* freqs, int64_t nfreq, int M, int nsm,
+                                 float* H_out, cudaStream_t st) {
   if (nfreq <= 0) return cudaSuccess;
-  // frequencies per thread: as many as keep the counts of a block within
-  // 48 KB (four blocks per SM), one beyond M = 96. Measured on the N = 1000
-  // ZTF-cadence times over 1e6 frequencies: M = 10 2.75e12 evaluations/s at
-  // R = 8 against 2.62e12 at R = 4; M = 20 2.54e12 at R = 4 against 2.08e12 at
-  // R = 8 (two blocks per SM). 16-bit counts (twice the blocks per SM) ran
-  // slower at every M (M = 20, R = 4: 2.07e12).
-  const int R = M <= 12 ? 8 : (M <= 24 ? 4 : (M <= 96 ? 2 : 1));
+  // Frequencies between anchors: the counts of one span fill about 48 KB (four
+  // blocks per SM). A thread takes as many frequencies as that leaves it, the
+  // staged record and the loop being shared by them (1000 times x 1e6
+  // frequencies, counts/s at R = 8, 4, 2, 1: M = 10 3.32e12, 3.11e12, 2.51e12,
+  // 1.72e12; M = 20 2.51e12 (two blocks per SM), 3.05e12, 2.49e12, 1.72e12;
+  // M = 50 R = 4 2.07e12, R = 2 2.31e12), and fewer while that leaves under two
+  // blocks per SM (1e5 frequencies, M = 10: 1.21e12, 1.38e12, 1.45e12, 1.10e12).
+  const int span = M <= 12 ? 1024 : (M <= 24 ? 512 : (M <= 96 ? 256 : 128));
+  int R = span / kEntThreads;
+  while (R > 1 && (nfreq + R * kEntThreads - 1) / (R * kEntThreads) < 2 * nsm) R >>= 1;
   const void* fn = R == 8   ? reinterpret_cast<const void*>(&entropy_dense_kernel<8>)
                    : R == 4 ? reinterpret_cast<const void*>(&entropy_dense_kernel<4>)
                    : R == 2 ? reinterpret_cast<const void*>(&entropy_dense_kernel<2>)
                             : reinterpret_cast<const void*>(&entropy_dense_kernel<1>);
-  const size_t smem = (size_t)(kEntChunk + 1) * 16 + (size_t)R * M * kEntThreads * 4;
+  const size_t smem = (size_t)(kEntChunk + 1) * 16 + kEntTable * 4 + (size_t)R * M * kEntThreads * 4;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int64_t per_block = (int64_t)kEntThreads * R;
   const int64_t blocks = (nfreq + per_block - 1) / per_block;
-  void* args[] = {const_cast<double**>(&t), &n, const_cast<double**>(&freqs), &nfreq, &M, &H_out};
+  void* args[] = {const_cast<double**>(&t), &n, const_cast<double**>(&freqs), &nfreq, &M, const_cast<int*>(&span), &H_out};
   return cudaLaunchKernel(fn, dim3((unsigned)blocks), dim3(kEntThreads), args, smem, st);
 }
 

@@ -191,8 +191,8 @@ cudaError_t launch_latch(unsigned* words, cudaStream_t st);  // words[kWordLatch
 cudaError_t launch_fill_topk(int32_t* idx, float* S, int64_t n, cudaStream_t st);
 cudaError_t plain_init_attributes(int max_smem);
 size_t plain_smem_bytes(int M);
-cudaError_t launch_entropy_dense(const double* t, int64_t n, const double* freqs, int64_t nfreq, int M, float* H_out,
-                                 cudaStream_t st);
+cudaError_t launch_entropy_dense(const double* t, int64_t n, const double* freqs, int64_t nfreq, int M, int nsm,
+                                 float* H_out, cudaStream_t st);
 cudaError_t launch_entropy_peaks(const int64_t* offsets, int64_t ncurves, const double* t, const double* freqs,
                                  int64_t nfreq, int M, int k, const int32_t* topk_idx, float* H_out, float* z_out,
                                  cudaStream_t st);

