@@ -30,13 +30,16 @@
 // triangle of the symmetric H) and the K x K Cholesky solve run in binary64.
 #include <math.h>
 
+#include <type_traits>
+
 #include "fpw_shared.cuh"
 
 namespace fpw {
 namespace {
 
 constexpr int kDrMaxK = 4;
-constexpr int kDrChunk = 128;  // observations staged at a time
+constexpr int kDrStage = 128;  // observations the staging area has room for
+constexpr int kDrChunk = 120;  // staged at a time; the block's constants lie behind them
 
 // Per observation, written once by the prep kernel.
 struct DriftObs {
@@ -146,7 +149,7 @@ __global__ void __launch_bounds__(256) drift_prep_kernel(const DriftArgs a) {
     tl[0] = a0;
     tl[1] = a1;
     a.tabs[c] = (a1 >= a0) ? fmax(fabs(a0), fabs(a1)) : 0.0;  // max |t| (0 with no finite time)
-    a.curve_bad[c] = b > 0.0 ? 1 : 0;
+    a.curve_bad[c] = b > 0.0 ? kCurveBad : 0;
     if (b > 0.0) atomicOr(a.status, kStatusData);
   }
   __syncthreads();
@@ -233,7 +236,17 @@ __global__ void __launch_bounds__(256) drift_prep_kernel(const DriftArgs a) {
   // The bins sum w (x - B g), the residuals of the curve's baseline fit: their
   // bin sums are z_m = Y_m - Q_m . g itself, so a drift far above the noise
   // does not cancel inside FP32 sums of w x.
-  if (K > 0 && !cbad)
+  // The pair reduction's range: H0 with a trace of at most 2^25, which bounds
+  // its condition (a pair's 2^-46 then costs S under 1e-7 where the FP32 bins
+  // leave it no digit; measured 2e-11 with beta = 1 and weights to 1e4); with
+  // weights in [2^-30, 2^30], residuals at most 2^30 and not all below 2^-25,
+  // beta <= 2^20, 1/alpha^2 zero or in [2^-60, 2^30] and under 2^20
+  // observations, no product leaves FP32 and none that matters loses its low part.
+  double trace = 0.0;
+  for (int k = 0; k < K; ++k) trace += a.H0[c * kDrMaxK * kDrMaxK + k * (kDrMaxK + 1)];
+  bool wide = !cbad && (n >= (1 << 20) || !a.pairs || !(trace <= 0x1p25));
+  double rmax = 0.0;
+  if (!cbad)
     for (int64_t i = tid; i < n; i += blockDim.x) {
       const double s = a.sigma[o0 + i];
       const double tau = (span > 0.0) ? 2.0 * (a.t[o0 + i] - lo) / span - 1.0 : 0.0;
@@ -243,11 +256,147 @@ __global__ void __launch_bounds__(256) drift_prep_kernel(const DriftArgs a) {
 #pragma unroll
       for (int k = 0; k < kDrMaxK; ++k)
         if (k < K) r -= Bk[k] * sg[k];
-      reinterpret_cast<DriftObs*>(a.payload)[o0 + i].q.x = (float)(r / (s * s));
+      if (K > 0) reinterpret_cast<DriftObs*>(a.payload)[o0 + i].q.x = (float)(r / (s * s));
+      wide = wide || !(s >= 0x1p-15 && s <= 0x1p15) || !(fabs(r) <= 0x1p30);
+      rmax = fmax(rmax, fabs(r));
     }
+  wide = __syncthreads_or(wide);
+  const bool small = !__syncthreads_or(rmax >= 0x1p-25);
+  if (tid == 0 && !cbad && (wide || small)) a.curve_bad[c] = kCurveWide;
   if (blockIdx.x == 0)
     for (int64_t q = tid; q < a.nfreq; q += blockDim.x)
       if (!isfinite(a.freqs[q])) atomicOr(a.status, kStatusGrid);
+}
+
+// FP32 pairs (value h + l, |l| a few ulp of h). Products are rounded once
+// (2^-47 relative), sums carry the exact error of the leading parts in l.
+// mul_rn / fma_rn: the exact error of a product must not be contracted away.
+static_assert((kDrStage - kDrChunk) * 32 >= kDrMaxK * kDrMaxK * 8 + 8, "room for H0 and df");
+
+struct Pair {
+  float h, l;
+};
+__device__ __forceinline__ Pair pmul(float a, float b) {
+  const float p = __fmul_rn(a, b);
+  return Pair{p, __fmaf_rn(a, b, -p)};
+}
+__device__ __forceinline__ Pair pmul(Pair a, float b) {
+  const float p = __fmul_rn(a.h, b);
+  return Pair{p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p))};
+}
+__device__ __forceinline__ Pair pmul(Pair a, Pair b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return Pair{p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)))};
+}
+__device__ __forceinline__ void padd(Pair& s, Pair p) {
+  const float t = __fadd_rn(s.h, p.h), z = __fsub_rn(t, s.h);
+  const float e = __fadd_rn(__fsub_rn(s.h, __fsub_rn(t, z)), __fsub_rn(p.h, z));
+  s.h = t;
+  s.l = __fadd_rn(s.l, __fadd_rn(p.l, e));
+}
+__device__ __forceinline__ void psub(Pair& s, Pair p) { padd(s, Pair{-p.h, -p.l}); }
+__device__ __forceinline__ Pair pnorm(Pair s) {
+  const float t = __fadd_rn(s.h, s.l);
+  return Pair{t, __fsub_rn(s.l, __fsub_rn(t, s.h))};
+}
+
+// The reduction of one frequency from its bins (slots slot0 + m T), in FP32
+// pairs; drift_reduce below is the same in binary64 and holds the formulas.
+// The bins are FP32 sums (2^-24 relative), so a pair's 2^-46 is as far below
+// them as binary64 for every S; a binary64 instruction of a warp occupies the
+// SM for about 20 clocks, an FP32 one for a quarter: the 310 of a K = 3, M = 20
+// frequency were 6200 clocks beside about 10000 of bin updates at N = 1000.
+// Taken where no product leaves FP32 (kCurveWide clear).
+template <int K>
+__device__ __forceinline__ Pair drift_reduce_pairs(const DriftArgs& a, const unsigned char* bins, const float* bQ3,
+                                                   int slot0, int T, const float2* h0) {
+  constexpr bool kWide = K >= 2;
+  constexpr int KK = K > 0 ? K : 1;
+  const int M = a.M;
+  Pair H[KK][KK], v[KK];
+#pragma unroll
+  for (int p = 0; p < K; ++p) {
+    v[p] = Pair{0.f, 0.f};
+#pragma unroll
+    for (int q = 0; q <= p; ++q) H[p][q] = q == 0 ? Pair{0.f, 0.f} : Pair{h0[p * kDrMaxK + q].x, h0[p * kDrMaxK + q].y};
+  }
+  const Pair cal{a.cal.x, a.cal.y};
+  const bool finite_alpha = a.inv_alpha2 != 0.0;
+  Pair S{0.f, 0.f};
+#pragma unroll 1
+  for (int m = 0; m < M; ++m) {
+    const int sl = slot0 + m * T;
+    float z, bw, Q[kDrMaxK];
+    if (kWide) {
+      const float4 b = reinterpret_cast<const float4*>(bins)[sl];
+      z = b.x;
+      bw = b.y;
+      Q[1] = b.z;
+      if (K > 2) Q[2] = b.w;
+    } else {
+      const float2 b = reinterpret_cast<const float2*>(bins)[sl];
+      z = b.x;
+      bw = b.y;
+    }
+    if (K > 3) Q[3] = bQ3[sl];
+    Pair L = cal;
+    padd(L, Pair{bw, 0.f});
+    if (!(L.h > 0.f)) continue;  // empty bin with 1/alpha^2 = 0: dropped
+    Pair rL;
+    rL.h = __frcp_rn(L.h);
+    rL.l = __fmul_rn(rL.h, __fmaf_rn(-L.l, rL.h, __fmaf_rn(-L.h, rL.h, 1.f)));
+    const Pair zl = pmul(rL, z);
+    padd(S, pmul(zl, z));
+    if (K > 0) {
+      padd(v[0], pmul(zl, bw));
+      if (finite_alpha) padd(H[0][0], pmul(rL, bw));
+    }
+#pragma unroll
+    for (int p = 1; p < K; ++p) {
+      padd(v[p], pmul(zl, Q[p]));
+      const Pair qs = pmul(rL, Q[p]);
+      if (finite_alpha) padd(H[p][0], qs);
+#pragma unroll
+      for (int q = 1; q <= p; ++q) psub(H[p][q], pmul(qs, Q[q]));
+    }
+  }
+  if (K > 0) {
+    v[0] = pmul(pnorm(v[0]), Pair{a.beta_p.x, a.beta_p.y});
+    Pair h{1.f, 0.f};
+    padd(h, pmul(pnorm(H[0][0]), Pair{a.b2cal.x, a.b2cal.y}));
+    H[0][0] = h;
+#pragma unroll
+    for (int p = 1; p < K; ++p) H[p][0] = pmul(pnorm(H[p][0]), Pair{a.bcal.x, a.bcal.y});
+  }
+  Pair Lc[KK][KK], di[KK], y[KK];
+#pragma unroll
+  for (int p = 0; p < K; ++p)
+#pragma unroll
+    for (int q = 0; q <= p; ++q) {
+      Pair s = H[p][q];
+#pragma unroll
+      for (int r = 0; r < q; ++r) psub(s, pmul(Lc[p][r], Lc[q][r]));
+      s = pnorm(s);
+      if (p == q) {
+        // 1 / sqrt(s): the FP32 estimate u and one Newton step, u + u (1 - s u^2) / 2
+        const float u = rsqrtf(s.h);
+        const Pair u2 = pmul(u, u);
+        const Pair su = pmul(s, u2);
+        const float d = __fsub_rn(__fsub_rn(1.f, su.h), su.l);
+        di[p] = s.h > 0.f ? Pair{u, 0.5f * u * d} : Pair{0.f, 0.f};
+      } else {
+        Lc[p][q] = pnorm(pmul(s, di[q]));
+      }
+    }
+#pragma unroll
+  for (int p = 0; p < K; ++p) {
+    Pair s = v[p];
+#pragma unroll
+    for (int r = 0; r < p; ++r) psub(s, pmul(Lc[p][r], y[r]));
+    y[p] = pnorm(pmul(pnorm(s), di[p]));
+    padd(S, pmul(y[p], y[p]));
+  }
+  return pnorm(S);
 }
 
 // The binary64 reduction of one frequency from its bins (slots slot0 + m T):
@@ -260,7 +409,7 @@ __global__ void __launch_bounds__(256) drift_prep_kernel(const DriftArgs a) {
 //   v_0  = beta sum_m Bw_m z_m / L_m,
 // (1 and 0 when 1/alpha^2 = 0) instead of H0 minus sums that cancel it.
 template <int K>
-__device__ __forceinline__ double drift_reduce(const DriftArgs& a, const unsigned char* bins, const float* bQ3,
+__device__ __noinline__ double drift_reduce(const DriftArgs& a, const unsigned char* bins, const float* bQ3,
                                                int slot0, int T, int64_t c) {
   constexpr bool kWide = K >= 2;
   const int M = a.M;
@@ -344,163 +493,74 @@ __device__ __forceinline__ double drift_reduce(const DriftArgs& a, const unsigne
   return S;
 }
 
-// One block per (tile of T frequencies, curve); thread = frequency. Bins
-// thread-private (bank = lane), [M][T] slots of drift_bin_bytes(K): one packed
-// read-modify-write per evaluation for K <= 3 (two for K = 4), two
-// observations per iteration with all loads issued before the stores.
-template <int K>
+// One block per (tile of T R frequencies, curve), R consecutive frequencies per
+// thread. Bins thread-private (bank = lane), [R][M][T] slots of
+// drift_bin_bytes(K): one packed read-modify-write per evaluation for K <= 3
+// (two for K = 4). The slots of the next observation are formed while this
+// one's bins are loaded. Anchors lie every a.span frequencies, a multiple of
+// the block's: phases do not depend on how the span is divided among blocks.
+//
+// Bound by shared memory: 8 passes per 16-byte update of a warp and 4 / R for
+// the staged record. With one frequency per thread, two observations per trip
+// and a binary64 reduction, 64 curves of 1000 observations x 20000 frequencies,
+// K = 3, M = 20 took 1846 us; with the pair reduction and the slots ahead 1668;
+// R = 2 1456 (M = 10: R = 4 1295; M = 50: R = 1 2185, R = 2 2543).
+template <int K, int R>
 __global__ void __launch_bounds__(128) drift_kernel(const DriftArgs a) {
   constexpr bool kWide = K >= 2;  // (Y, Bw, Q_1, Q_2) as float4, else (Y, Bw) as float2
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int T = blockDim.x, tid = threadIdx.x;
-  const int M = a.M;
-  const int64_t c = blockIdx.y, F = a.nfreq;
-  const int64_t f0 = (int64_t)blockIdx.x * T, k = f0 + tid;
-  unsigned char* const bins = smem;                                                     // [M][T] main slots
-  float* const bQ3 = reinterpret_cast<float*>(bins + (size_t)M * T * (kWide ? 16 : 8));  // [M][T] (K = 4)
-  ulonglong2* const sPD = reinterpret_cast<ulonglong2*>(smem + (size_t)M * T * drift_bin_bytes(K));  // [chunk]
-  float4* const sQ = reinterpret_cast<float4*>(sPD + kDrChunk);                         // [chunk]
-  float* const sQ3 = reinterpret_cast<float*>(sQ + kDrChunk);                           // [chunk] (K = 4)
-  const bool grid_bad = (*(volatile unsigned*)a.status & kStatusGrid) != 0u;
-  if (grid_bad) return;
-  const bool cbad = a.curve_bad[c] != 0;
-  const int64_t o0 = a.offsets[c], n = a.offsets[c + 1] - o0;
-  const double df = (F > 1) ? (a.freqs[F - 1] - a.freqs[0]) / (double)(F - 1) : 0.0;
-  const double fa = a.freqs[f0];
-  // linear grid over this tile (the tile kernels' bound on the phase error)?
-  const double tm = a.tabs[c];
-  const double fk = k < F ? a.freqs[k] : fa;
-  const bool nonlin = k < F && fabs(fk - fma((double)tid, df, fa)) * tm > kGridTolCycles;
-  const bool lin = !__syncthreads_or(nonlin);
-  for (int m = 0; m < M; ++m) {
-    if (kWide)
-      reinterpret_cast<float4*>(bins)[m * T + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
-    else
-      reinterpret_cast<float2*>(bins)[m * T + tid] = make_float2(0.f, 0.f);
-    if (K > 3) bQ3[m * T + tid] = 0.f;
-  }
-  const DriftObs* const obs = reinterpret_cast<const DriftObs*>(a.payload) + o0;
-  for (int64_t oc = 0; oc < n; oc += kDrChunk) {
-    const int cnt = (int)((n - oc) < kDrChunk ? (n - oc) : kDrChunk);
-    __syncthreads();
-    for (int i = tid; i < cnt; i += T) {
-      const double ti = a.t[o0 + oc + i];
-      const DriftObs ob = obs[oc + i];
-      sPD[i] = lin ? make_ulonglong2(phase_fixed64(ti, fa), ob.D)
-                   : make_ulonglong2((unsigned long long)__double_as_longlong(ti), 0ull);
-      sQ[i] = ob.q;
-      if (K > 3) sQ3[i] = ob.q3;
-    }
-    __syncthreads();
-    if (!cbad) {
-      auto slot = [&](const ulonglong2 pd) {
-        const unsigned long long phi =
-            lin ? pd.x + (unsigned long long)tid * pd.y : phase_fixed64(__longlong_as_double((long long)pd.x), fk);
-        return (int)bin_of_phase(phi, (unsigned)M) * T + tid;
-      };
-      // two observations per iteration: both read-modify-write chains are in
-      // flight at once; where both fall in one bin the second update starts
-      // from the first one's sum (same additions in the same order)
-      int i = 0;
-      for (; i + 1 < cnt; i += 2) {
-        const int ma = slot(sPD[i]), mb = slot(sPD[i + 1]);
-        const float4 pa = sQ[i], pb = sQ[i + 1];
-        if (kWide) {
-          float4* const b4 = reinterpret_cast<float4*>(bins);
-          const float4 va = b4[ma];
-          float4 vb = b4[mb];
-          const float4 ua = make_float4(va.x + pa.x, va.y + pa.y, va.z + pa.z, va.w + pa.w);
-          if (ma == mb) vb = ua;
-          b4[ma] = ua;
-          b4[mb] = make_float4(vb.x + pb.x, vb.y + pb.y, vb.z + pb.z, vb.w + pb.w);
-        } else {
-          float2* const b2 = reinterpret_cast<float2*>(bins);
-          const float2 va = b2[ma];
-          float2 vb = b2[mb];
-          const float2 ua = make_float2(va.x + pa.x, va.y + pa.y);
-          if (ma == mb) vb = ua;
-          b2[ma] = ua;
-          b2[mb] = make_float2(vb.x + pb.x, vb.y + pb.y);
-        }
-        if (K > 3) {
-          const float qa = bQ3[ma];
-          float qb = bQ3[mb];
-          const float ra = qa + sQ3[i];
-          if (ma == mb) qb = ra;
-          bQ3[ma] = ra;
-          bQ3[mb] = qb + sQ3[i + 1];
-        }
-      }
-      if (i < cnt) {
-        const int ma = slot(sPD[i]);
-        const float4 pa = sQ[i];
-        if (kWide) {
-          float4* const b4 = reinterpret_cast<float4*>(bins);
-          const float4 va = b4[ma];
-          b4[ma] = make_float4(va.x + pa.x, va.y + pa.y, va.z + pa.z, va.w + pa.w);
-        } else {
-          float2* const b2 = reinterpret_cast<float2*>(bins);
-          const float2 va = b2[ma];
-          b2[ma] = make_float2(va.x + pa.x, va.y + pa.y);
-        }
-        if (K > 3) bQ3[ma] += sQ3[i];
-      }
-    }
-  }
-  if (k >= F) return;
-  const double S = drift_reduce<K>(a, bins, bQ3, tid, T, c);
-  const float Sf = cbad ? __int_as_float(0x7fc00000) : (float)S;
-  if (a.S32) a.S32[c * F + k] = Sf;
-  if (a.S_out) a.S_out[c * F + k] = cbad ? (double)Sf : S;
-}
-
-// As drift_kernel, with R consecutive frequencies per thread: tiles of T R
-// frequencies, [r][M][T] bin slots, each staged observation serving the
-// thread's R frequencies (half the broadcast per evaluation for R = 2, twice
-// the bins per thread). A separate kernel: the one-frequency loop above runs
-// faster in its own form.
-template <int K, int R>
-__global__ void __launch_bounds__(128) drift_kernel_rf(const DriftArgs a) {
-  constexpr bool kWide = K >= 2;  // (Y, Bw, Q_1, Q_2) as float4, else (Y, Bw) as float2
+  constexpr int kUnroll = kWide && R > 1 ? 2 : 4;  // the longer body of the others ran up to 3 % slower at 4
+  using Bin = std::conditional_t<kWide, float4, float2>;
   extern __shared__ __align__(16) unsigned char smem[];
   const int T = blockDim.x, tid = threadIdx.x;
   const int M = a.M, MT = M * T;
   const int64_t c = blockIdx.y, F = a.nfreq;
   const int64_t f0 = (int64_t)blockIdx.x * (T * R);
-  const int j0 = tid * R;  // the thread's first frequency within the tile
-  unsigned char* const bins = smem;                                                         // [R][M][T] main slots
-  float* const bQ3 = reinterpret_cast<float*>(bins + (size_t)R * MT * (kWide ? 16 : 8));    // [R][M][T] (K = 4)
+  const int64_t fanchor = (int64_t)((unsigned)f0 / (unsigned)a.span) * a.span;  // f0 < 2^31
+  const int j0 = (int)(f0 - fanchor) + tid * R;  // the thread's first frequency past the anchor
+  Bin* const bins = reinterpret_cast<Bin*>(smem);                                           // [R][M][T] main slots
+  float* const bQ3 = reinterpret_cast<float*>(bins + (size_t)R * MT);                       // [R][M][T] (K = 4)
   ulonglong2* const sPD = reinterpret_cast<ulonglong2*>(smem + (size_t)R * MT * drift_bin_bytes(K));  // [chunk]
   float4* const sQ = reinterpret_cast<float4*>(sPD + kDrChunk);                             // [chunk]
   float* const sQ3 = reinterpret_cast<float*>(sQ + kDrChunk);                               // [chunk] (K = 4)
+  float2* const s_h0 = reinterpret_cast<float2*>(sQ3 + (K > 3 ? kDrChunk : 0));             // [16] H0 as pairs
+  double& s_df = *reinterpret_cast<double*>(s_h0 + kDrMaxK * kDrMaxK);
   const bool grid_bad = (*(volatile unsigned*)a.status & kStatusGrid) != 0u;
   if (grid_bad) return;
-  const bool cbad = a.curve_bad[c] != 0;
+  const unsigned flags = a.curve_bad[c];
+  const bool cbad = flags & kCurveBad;
   const int64_t o0 = a.offsets[c], n = a.offsets[c + 1] - o0;
-  const double df = (F > 1) ? (a.freqs[F - 1] - a.freqs[0]) / (double)(F - 1) : 0.0;
-  const double fa = a.freqs[f0];
+  const double fa = a.freqs[fanchor];
   // linear grid over this tile (the tile kernels' bound on the phase error)?
   const double tm = a.tabs[c];
   double fk[R];
-  bool nonlin = false;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const int64_t k = f0 + j0 + r;
+    const int64_t k = fanchor + j0 + r;
     fk[r] = k < F ? a.freqs[k] : fa;
-    if (k < F && fabs(fk[r] - fma((double)(j0 + r), df, fa)) * tm > kGridTolCycles) nonlin = true;
   }
-  const bool lin = !__syncthreads_or(nonlin);
+  if (tid < 32) {  // one warp's binary64 work for the block
+    if (tid == 0) s_df = (F > 1) ? (a.freqs[F - 1] - a.freqs[0]) / (double)(F - 1) : 0.0;
+    if (tid < kDrMaxK * kDrMaxK) {
+      const double h = a.H0[c * kDrMaxK * kDrMaxK + tid];
+      s_h0[tid] = make_float2((float)h, (float)(h - (double)(float)h));
+    }
+  }
+#pragma unroll 4
   for (int q = 0; q < R * M; ++q) {
-    if (kWide)
-      reinterpret_cast<float4*>(bins)[q * T + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
-    else
-      reinterpret_cast<float2*>(bins)[q * T + tid] = make_float2(0.f, 0.f);
+    bins[q * T + tid] = Bin{};
     if (K > 3) bQ3[q * T + tid] = 0.f;
   }
+  __syncthreads();
+  const double df = s_df;
+  bool nonlin = false;
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    if (fanchor + j0 + r < F && fabs(fk[r] - fma((double)(j0 + r), df, fa)) * tm > kGridTolCycles) nonlin = true;
+  const bool lin = !__syncthreads_or(nonlin);
   const DriftObs* const obs = reinterpret_cast<const DriftObs*>(a.payload) + o0;
   for (int64_t oc = 0; oc < n; oc += kDrChunk) {
     const int cnt = (int)((n - oc) < kDrChunk ? (n - oc) : kDrChunk);
-    __syncthreads();
+    if (oc > 0) __syncthreads();
     for (int i = tid; i < cnt; i += T) {
       const double ti = a.t[o0 + oc + i];
       const DriftObs ob = obs[oc + i];
@@ -510,125 +570,99 @@ __global__ void __launch_bounds__(128) drift_kernel_rf(const DriftArgs a) {
       if (K > 3) sQ3[i] = ob.q3;
     }
     __syncthreads();
-    if (!cbad) {
-      // the observation's slot for each of the thread's R frequencies
-      auto slots = [&](const ulonglong2 pd, int (&sl)[R]) {
-        if (lin) {
-          unsigned long long phi = pd.x + (unsigned long long)j0 * pd.y;
+    if (cbad) continue;
+    // the observation's slot for each of the thread's R frequencies
+    auto slots = [&](const ulonglong2 pd, int (&sl)[R]) {
+      const unsigned long long phi = pd.x + (unsigned long long)j0 * pd.y;
 #pragma unroll
-          for (int r = 0; r < R; ++r) {
-            sl[r] = r * MT + (int)bin_of_phase(phi, (unsigned)M) * T + tid;
-            phi += pd.y;
-          }
-        } else {
-          const double ti = __longlong_as_double((long long)pd.x);
+      for (int r = 0; r < R; ++r)
+        sl[r] = r * MT + (int)bin_of_phase(phi + (unsigned long long)r * pd.y, (unsigned)M) * T + tid;
+    };
+    auto update = [&](const Bin (&b)[R], const int (&sl)[R], const float4 q) {
 #pragma unroll
-          for (int r = 0; r < R; ++r) sl[r] = r * MT + (int)bin_of_phase(phase_fixed64(ti, fk[r]), (unsigned)M) * T + tid;
-        }
-      };
-      // two observations per iteration: all read-modify-write chains are in
-      // flight at once; where both observations fall in one bin the second
-      // update starts from the first one's sum (same additions in the same order)
-      int i = 0;
-      for (; i + 1 < cnt; i += 2) {
-        int sa[R], sb[R];
-        slots(sPD[i], sa);
-        slots(sPD[i + 1], sb);
-        const float4 pa = sQ[i], pb = sQ[i + 1];
-        if (kWide) {
-          float4* const b4 = reinterpret_cast<float4*>(bins);
-          float4 va[R], vb[R];
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            va[r] = b4[sa[r]];
-            vb[r] = b4[sb[r]];
-          }
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const float4 ua = make_float4(va[r].x + pa.x, va[r].y + pa.y, va[r].z + pa.z, va[r].w + pa.w);
-            const float4 wb = sa[r] == sb[r] ? ua : vb[r];
-            b4[sa[r]] = ua;
-            b4[sb[r]] = make_float4(wb.x + pb.x, wb.y + pb.y, wb.z + pb.z, wb.w + pb.w);
-          }
-        } else {
-          float2* const b2 = reinterpret_cast<float2*>(bins);
-          float2 va[R], vb[R];
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            va[r] = b2[sa[r]];
-            vb[r] = b2[sb[r]];
-          }
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const float2 ua = make_float2(va[r].x + pa.x, va[r].y + pa.y);
-            const float2 wb = sa[r] == sb[r] ? ua : vb[r];
-            b2[sa[r]] = ua;
-            b2[sb[r]] = make_float2(wb.x + pb.x, wb.y + pb.y);
-          }
-        }
-        if (K > 3) {
-          const float ra = sQ3[i], rb = sQ3[i + 1];
-          float qa[R], qb[R];
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            qa[r] = bQ3[sa[r]];
-            qb[r] = bQ3[sb[r]];
-          }
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const float ua = qa[r] + ra;
-            bQ3[sa[r]] = ua;
-            bQ3[sb[r]] = (sa[r] == sb[r] ? ua : qb[r]) + rb;
-          }
-        }
+      for (int r = 0; r < R; ++r) {
+        if constexpr (kWide)
+          bins[sl[r]] = make_float4(b[r].x + q.x, b[r].y + q.y, b[r].z + q.z, b[r].w + q.w);
+        else
+          bins[sl[r]] = make_float2(b[r].x + q.x, b[r].y + q.y);
       }
-      if (i < cnt) {
-        int sa[R];
-        slots(sPD[i], sa);
-        const float4 pa = sQ[i];
+    };
+    if (lin) {
+      int sl[R];
+      slots(sPD[0], sl);
+#pragma unroll(kUnroll)
+      for (int i = 0; i < cnt; ++i) {
+        Bin b[R];
+        float b3[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          if (kWide) {
-            float4* const b4 = reinterpret_cast<float4*>(bins);
-            const float4 va = b4[sa[r]];
-            b4[sa[r]] = make_float4(va.x + pa.x, va.y + pa.y, va.z + pa.z, va.w + pa.w);
-          } else {
-            float2* const b2 = reinterpret_cast<float2*>(bins);
-            const float2 va = b2[sa[r]];
-            b2[sa[r]] = make_float2(va.x + pa.x, va.y + pa.y);
-          }
-          if (K > 3) bQ3[sa[r]] += sQ3[i];
+          b[r] = bins[sl[r]];
+          if (K > 3) b3[r] = bQ3[sl[r]];
         }
+        const float4 q = sQ[i];
+        const float q3 = K > 3 ? sQ3[i] : 0.f;
+        int sn[R];
+        slots(sPD[i + 1 < cnt ? i + 1 : i], sn);
+        update(b, sl, q);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (K > 3) bQ3[sl[r]] = b3[r] + q3;
+          sl[r] = sn[r];
+        }
+      }
+    } else {
+      for (int i = 0; i < cnt; ++i) {
+        const double ti = __longlong_as_double((long long)sPD[i].x);
+        int sl[R];
+        Bin b[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          sl[r] = r * MT + (int)bin_of_phase(phase_fixed64(ti, fk[r]), (unsigned)M) * T + tid;
+          b[r] = bins[sl[r]];
+        }
+        update(b, sl, sQ[i]);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          if (K > 3) bQ3[sl[r]] += sQ3[i];
       }
     }
   }
-#pragma unroll
+#pragma unroll 1
   for (int r = 0; r < R; ++r) {
-    const int64_t k = f0 + j0 + r;
+    const int64_t k = fanchor + j0 + r;
     if (k >= F) break;
-    const double S = drift_reduce<K>(a, bins, bQ3, r * MT + tid, T, c);
-    const float Sf = cbad ? __int_as_float(0x7fc00000) : (float)S;
+    float Sf;
+    double S;
+    if (cbad) {
+      Sf = __int_as_float(0x7fc00000);
+      S = (double)Sf;
+    } else if (flags & kCurveWide) {
+      S = drift_reduce<K>(a, smem, bQ3, r * MT + tid, T, c);
+      Sf = (float)S;
+    } else {
+      const Pair s = drift_reduce_pairs<K>(a, smem, bQ3, r * MT + tid, T, s_h0);
+      Sf = s.h;
+      S = a.S_out ? (double)s.h + (double)s.l : 0.0;
+    }
     if (a.S32) a.S32[c * F + k] = Sf;
-    if (a.S_out) a.S_out[c * F + k] = cbad ? (double)Sf : S;
+    if (a.S_out) a.S_out[c * F + k] = S;
   }
 }
 
+template <int K>
+const void* drift_fn_k(int R) {
+  return R == 4 ? reinterpret_cast<const void*>(&drift_kernel<K, 4>)
+                : (R == 2 ? reinterpret_cast<const void*>(&drift_kernel<K, 2>)
+                          : reinterpret_cast<const void*>(&drift_kernel<K, 1>));
+}
+
 const void* drift_fn(int K, int R) {
-  if (R == 2) {
-    switch (K) {
-      case 0: return reinterpret_cast<const void*>(&drift_kernel_rf<0, 2>);
-      case 1: return reinterpret_cast<const void*>(&drift_kernel_rf<1, 2>);
-      case 2: return reinterpret_cast<const void*>(&drift_kernel_rf<2, 2>);
-      case 3: return reinterpret_cast<const void*>(&drift_kernel_rf<3, 2>);
-      default: return reinterpret_cast<const void*>(&drift_kernel_rf<4, 2>);
-    }
-  }
   switch (K) {
-    case 0: return reinterpret_cast<const void*>(&drift_kernel<0>);
-    case 1: return reinterpret_cast<const void*>(&drift_kernel<1>);
-    case 2: return reinterpret_cast<const void*>(&drift_kernel<2>);
-    case 3: return reinterpret_cast<const void*>(&drift_kernel<3>);
-    default: return reinterpret_cast<const void*>(&drift_kernel<4>);
+    case 0: return drift_fn_k<0>(R);
+    case 1: return drift_fn_k<1>(R);
+    case 2: return drift_fn_k<2>(R);
+    case 3: return drift_fn_k<3>(R);
+    default: return drift_fn_k<4>(R);
   }
 }
 
@@ -638,7 +672,7 @@ const void* drift_fn(int K, int R) {
 // static shared memory.
 static size_t drift_dynamic_limit(int smem_optin) {
   cudaFuncAttributes fa{};
-  if (cudaFuncGetAttributes(&fa, drift_fn(4, 2)) != cudaSuccess) return 0;
+  if (cudaFuncGetAttributes(&fa, drift_fn(4, 4)) != cudaSuccess) return 0;
   return smem_optin > (int)fa.sharedSizeBytes ? (size_t)(smem_optin - (int)fa.sharedSizeBytes) : 0;
 }
 
@@ -649,12 +683,29 @@ int drift_threads(int M, int K, int smem_optin) {
   return 0;
 }
 
+// The span's frequencies as T threads of R: the record read for an observation
+// is shared by R evaluations, so the largest R that leaves eight warps on an SM
+// (the bins of a span take the same room however it is divided), else R = 1
+// (measured at 8 warps against 4: M = 50, K = 3 2185 us against 2543, K = 4, M =
+// 20 1971 at R = 2, 8 warps, against 2412 at R = 4; at 10 against 20: M = 20,
+// K = 3 1456 against 1668).
+void drift_split(int M, int K, int span, int smem_optin, int* T, int* R) {
+  const size_t block = drift_smem_bytes(M, K, span, 1) + 1024;
+  for (int r = 4; r >= 1; r >>= 1) {
+    const int t = span / r;
+    if (span % r || t % 32 || t > 128) continue;
+    *T = t;
+    *R = r;
+    if ((smem_optin + 1024) / block * (size_t)(t / 32) >= 8) return;
+  }
+}
+
 bool drift_fits(int M, int K, int T, int R, int smem_optin) {
   return drift_smem_bytes(M, K, T, R) <= drift_dynamic_limit(smem_optin);
 }
 
 size_t drift_smem_bytes(int M, int K, int T, int R) {
-  return (size_t)R * M * T * drift_bin_bytes(K) + (size_t)kDrChunk * drift_stage_bytes(K);
+  return (size_t)R * M * T * drift_bin_bytes(K) + (size_t)kDrStage * drift_stage_bytes(K);
 }
 
 int drift_max_basis() { return kDrMaxK; }
@@ -664,7 +715,7 @@ size_t drift_payload_bytes() { return sizeof(DriftObs); }
 cudaError_t drift_init_attributes(int max_smem) {
   const int lim = (int)drift_dynamic_limit(max_smem);
   for (int K = 0; K <= kDrMaxK; ++K)
-    for (int R = 1; R <= 2; ++R) {
+    for (int R = 1; R <= 4; R *= 2) {
       const cudaError_t e = cudaFuncSetAttribute(drift_fn(K, R), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
       if (e != cudaSuccess) return e;
     }

@@ -1330,10 +1330,9 @@ int fpw_periodogram_drift(fpw_ctx* ctx, void* stream, const fpw_params* params, 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->last_stream = st;
   // threads (32..128) and frequencies per thread (1 or 2) from params when
-  // set; by default the largest block with one frequency per thread, and two
-  // frequencies per thread for K <= 1 where they fit (8-byte bins: measured
-  // 16 % faster at K = 0; slower from K = 2 on, where 16-byte bins halve the
-  // resident warps)
+  // set. By default their product is the span between phase anchors, the
+  // largest block with one frequency per thread (two for K <= 1, 8-byte bins),
+  // and drift_split chooses how a block holds it.
   if (p.threads != 0 && (p.threads % 32 != 0 || p.threads < 32 || p.threads > 128)) return FPW_ENOTSUP;
   if (p.freqs_per_thread != 0 && p.freqs_per_thread != 1 && p.freqs_per_thread != 2) return FPW_ENOTSUP;
   const int T = p.threads != 0 ? p.threads : drift_threads(M, K, ctx->smem_optin);
@@ -1374,6 +1373,15 @@ int fpw_periodogram_drift(fpw_ctx* ctx, void* stream, const fpw_params* params, 
   a.K = K;
   a.beta = beta;
   a.inv_alpha2 = p.inv_alpha2;
+  const auto pair = [](double v) { return make_float2((float)v, (float)(v - (double)(float)v)); };
+  a.pairs = beta <= 0x1p20 && (p.inv_alpha2 == 0.0 || (p.inv_alpha2 >= 0x1p-60 && p.inv_alpha2 <= 0x1p30));
+  a.cal = pair(p.inv_alpha2);
+  a.beta_p = pair(beta);
+  a.bcal = pair(beta * p.inv_alpha2);
+  a.b2cal = pair(beta * beta * p.inv_alpha2);
+  a.span = T * R;
+  int Tl = T, Rl = R;
+  if (p.threads == 0 && p.freqs_per_thread == 0) drift_split(M, K, T * R, ctx->smem_optin, &Tl, &Rl);
   a.payload = ctx->dr_payload.p;
   a.tabs = static_cast<double*>(ctx->dr_tabs.p);
   a.H0 = static_cast<double*>(ctx->dr_H0.p);
@@ -1397,7 +1405,7 @@ int fpw_periodogram_drift(fpw_ctx* ctx, void* stream, const fpw_params* params, 
     ctx->ev_used += 2;
   }
   FPW_CK(cudaMemsetAsync(words, 0, 2 * sizeof(unsigned), st));
-  FPW_CK(launch_drift(a, T, R, st));
+  FPW_CK(launch_drift(a, Tl, Rl, st));
   FPW_CK(launch_latch(words, st));
   return FPW_OK;
 }

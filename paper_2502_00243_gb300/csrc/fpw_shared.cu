@@ -699,7 +699,7 @@ __global__ void __launch_bounds__(kShTopkThreads) dense_topk32_kernel(const Dens
   const int64_t F = a.nfreq;
   const float* S = a.S32 + c * F;
   const bool grid_bad = (*(volatile unsigned*)a.status & kStatusGrid) != 0u;
-  const bool bad = grid_bad || a.curve_bad[c];
+  const bool bad = grid_bad || (a.curve_bad[c] & kCurveBad);
   int32_t* oi = a.topk_idx + c * a.k;
   float* os = a.topk_S + c * a.k;
   float ps = INFINITY;

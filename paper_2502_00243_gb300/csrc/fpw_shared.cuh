@@ -46,7 +46,7 @@ struct DenseTopk32Args {
   int64_t nfreq;
   int k;
   int peak_raw;
-  const uint8_t* curve_bad;  // [ncurves]: no peaks for a bad curve
+  const uint8_t* curve_bad;  // [ncurves] flags: no peaks where kCurveBad
   const unsigned* status;    // kStatusGrid: no peaks at all
   int32_t* topk_idx;         // [ncurves][k]
   float* topk_S;
@@ -66,11 +66,14 @@ struct DriftArgs {
   int K;                    // Chebyshev basis functions (0..4)
   double beta;              // prior standard deviation of each basis coefficient
   double inv_alpha2;
+  int span;                 // frequencies between phase anchors (a multiple of the block's)
+  bool pairs;               // beta and inv_alpha2 lie where the FP32-pair reduction may be taken
+  float2 cal, beta_p, bcal, b2cal;  // inv_alpha2, beta, beta inv_alpha2, beta^2 inv_alpha2 as FP32 pairs
   void* payload;            // [nobs] 32-byte per-observation records (prep kernel)
   double* tabs;             // [ncurves] max |t| of the curve's finite times
   double* H0;               // [ncurves][4][4]: I + B^T D B
   double* g;                // [ncurves][4]: H0^-1 B^T D x
-  uint8_t* curve_bad;       // [ncurves]
+  uint8_t* curve_bad;       // [ncurves] flags kCurveBad, kCurveWide
   unsigned* status;
   float* S32;               // dense [ncurves][nfreq] (required when k > 0), or NULL
   double* S_out;            // dense [ncurves][nfreq] or NULL
@@ -81,6 +84,7 @@ struct DriftArgs {
   cudaEvent_t timing_start;
   cudaEvent_t timing_stop;
 };
+void drift_split(int M, int K, int span, int smem_optin, int* T, int* R);  // the launch of a span of frequencies
 int drift_threads(int M, int K, int smem_optin);  // threads per block, 0 if M is too large
 size_t drift_smem_bytes(int M, int K, int T, int R);  // R frequencies per thread (1 or 2)
 bool drift_fits(int M, int K, int T, int R, int smem_optin);
