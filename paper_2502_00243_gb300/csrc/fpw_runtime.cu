@@ -1268,7 +1268,6 @@ int fpw_periodogram_shared(fpw_ctx* ctx, void* stream, const fpw_params* params,
   a.M = M;
   a.fpm = fpm;
   a.n_mma = n_mma;
-  a.npass = (nfreq + 2 * fpm - 1) / (2 * fpm);
   a.ngroups = (ncurves + per - 1) / per;
   a.nchunks = (n + 31) / 32;
   a.inv_alpha2 = p.inv_alpha2;

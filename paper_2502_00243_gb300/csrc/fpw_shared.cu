@@ -18,13 +18,16 @@
 // * H is built in shared memory for each chunk of 32 observations from exact
 //   phases (phase_fixed64: the integer product of the binary64 significands),
 //   so bins equal floor(M frac(t f)) except within 2^-32 of a cycle below an edge.
-// * One CTA per SM (persistent over (group of 64 curves, frequency pass) work
-//   items) holds two accumulators of 128 x N (N = frequencies per pass x M
-//   <= 256) in 512 TMEM columns; V chunks arrive by bulk copy (TMA) into a
+// * Groups of 64 curves are taken two at a time, one accumulator for part 0 and
+//   one for part 1 of their 128 curves; a group left over has its own launch,
+//   parts in neighbouring rows, an accumulator for each half of the pass.
+// * One CTA per SM (persistent over (groups, frequency pass) work items) holds
+//   two accumulators of 128 x N (N = frequencies per accumulator x M <= 256) in
+//   512 TMEM columns; V chunks arrive by bulk copy (TMA) into a
 //   double buffer, H is double-buffered too, and the single issuing thread's
 //   MMAs signal an mbarrier per buffer (tcgen05.commit).
-// * The epilogue reads D with tcgen05.ld (lane = (curve, part) row), pairs the
-//   two parts of a curve with one shuffle, and reduces S = sum_m A_m^2 / (B_m +
+// * The epilogue reads D with tcgen05.ld (a pair of groups: lane = curve; one
+//   group: lane = (curve, part), paired with one shuffle), and reduces S = sum_m A_m^2 / (B_m +
 //   1/alpha^2) per frequency into a dense FP32 array; a per-curve top-k pass
 //   follows.
 //
@@ -49,7 +52,7 @@ constexpr int kShThreads = 576;  // 16 builder/epilogue warps + 2 issuer warps
 constexpr int kShNMax = 256;                    // MMA N limit (M = 128)
 constexpr int kShMaxFpm = 64;                   // frequencies per accumulator, at most
 constexpr int kShHOperandMax = kShNMax * kShK * 2;   // one H operand of a chunk: 32 KB
-constexpr int kShHSlotBytes = 2 * kShHOperandMax;    // two H operands (two accumulators)
+constexpr int kShHSlotBytes = 2 * kShHOperandMax;    // two H operands (two accumulators of one group)
 constexpr int kShTmemCols = 512;
 constexpr unsigned kOneOne = 0x3C003C00u;       // two fp16 1.0
 constexpr long long kWaitClocks = 4000000000LL; // default wait limit, ~2 s at 2 GHz
@@ -63,9 +66,8 @@ constexpr int kShStage = 1024;                  // observations staged at a time
 constexpr int kShStageChunks = kShStage / kShObs;
 
 // Shared-memory carve-up (bytes).
-constexpr int kOffV = 0;                                   // V chunks: 4 x 16 KB
-constexpr int kOffH = kOffV + kShVSlots * kShChunkBytes;   // H chunks: 2 x 64 KB
-constexpr int kOffOld = kOffH + 2 * kShHSlotBytes;         // bin of every (frequency, observation) pair in H, per slot
+constexpr int kOffV = 0;                                   // V chunks: 4 x 16 KB, or 4 x 32 KB for two groups
+constexpr int kOffOld = kOffV + kShVSlots * kShChunkBytes + 2 * kShHSlotBytes;  // (H chunks: 2 x 64 KB, or 2 x 32 KB) bin of every (frequency, observation) pair in H, per slot
 constexpr int kOffF = kOffOld + 2 * kMaxPairs;             // the pass's frequencies (binary64)
 constexpr int kOffStage = kOffF + kMaxPassFreqs * 8;       // t, P, D of kShStage observations
 constexpr int kOffPart = kOffStage + 3 * kShStage * 8;    // epilogue: partial S of a frequency split between warps
@@ -163,8 +165,11 @@ __device__ __forceinline__ bool builders_or(bool v, int nthreads) {
   return r != 0u;
 }
 
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+__device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                    smem_addr(dst)),
                "l"(src), "r"(bytes), "r"(smem_addr(bar))
@@ -260,10 +265,16 @@ __global__ void __launch_bounds__(256) shared_prep_kernel(const SharedArgs a) {
     a.curve_bad[c] = (uint8_t)(real && bad);
     if (real && bad) atomicOr(a.status, kStatusData);
   }
+  // rows of the curve's parts: in a pair of groups one image holds a, the other
+  // w of the pair's 128 curves; in a group by itself the parts are neighbours
   const int64_t g = c / kShCurves;
-  const uint32_t row = (uint32_t)(c % kShCurves) * 2u;
+  const size_t gbytes = (size_t)a.nchunks * kShChunkBytes;
+  const bool paired = g < (a.ngroups & ~(int64_t)1);
+  const uint32_t row = paired ? (uint32_t)(c % (2 * kShCurves)) : (uint32_t)(c % kShCurves) * 2u;
+  unsigned char* const img = a.image + (size_t)(paired ? (g & ~(int64_t)1) : g) * gbytes;
+  const size_t wpart = paired ? gbytes : 0;
+  const uint32_t wrow = paired ? row : row + 1u;
   const bool zero = !real || bad;
-  unsigned char* img = a.image + (size_t)g * (size_t)a.nchunks * kShChunkBytes;
   const int64_t npad = a.nchunks * kShObs;
   for (int64_t i = tid; i < npad; i += blockDim.x) {
     float av = 0.f, wv = 0.f;
@@ -278,7 +289,7 @@ __global__ void __launch_bounds__(256) shared_prep_kernel(const SharedArgs a) {
     unsigned char* ch = img + (size_t)(i / kShObs) * kShChunkBytes;
     const uint32_t q = 2u * (uint32_t)(i % kShObs);
     *reinterpret_cast<__half2*>(ch + km_off(row, q, kShRows)) = __halves2half2(ah, al);
-    *reinterpret_cast<__half2*>(ch + km_off(row + 1u, q, kShRows)) = __halves2half2(wh, wl);
+    *reinterpret_cast<__half2*>(ch + wpart + km_off(wrow, q, kShRows)) = __halves2half2(wh, wl);
   }
   if (blockIdx.x == 0)
     for (int64_t q = tid; q < a.nfreq; q += blockDim.x)
@@ -320,10 +331,104 @@ constexpr int kShBuilderWarps = 16;
 constexpr int kShBuilders = kShBuilderWarps * 32;
 constexpr int kShIssuers = kShThreads / 32 - kShBuilderWarps;  // one per accumulator
 
+// Epilogue of a pair of groups: accumulator 0 holds the sums of a, accumulator 1
+// those of w, of the pair's 128 curves (TMEM lane = curve) at fpm frequencies,
+// so a lane reads both sums of a bin and forms S by itself. Warp w takes lanes
+// 32 (w % 4) .. + 31 and the (w / 4)-th quarter of the frequencies; 8 columns
+// per step, the next step's loads in flight.
+__device__ __forceinline__ void pair_epilogue(const SharedArgs& a, uint32_t tmem, int64_t c, int64_t f0, bool cbad, float2 scale,
+                                              int warp, int lane) {
+  const int M = a.M, quarter = warp & 3, seg = warp >> 2;
+  const int64_t F = a.nfreq;
+  const bool cvalid = c < a.ncurves;
+  const float sa = scale.x, sw = scale.y, cal = (float)a.inv_alpha2;
+  int jl = seg * a.fpm / 4;
+  const int jend = (seg + 1) * a.fpm / 4;
+  if (jl >= jend) return;
+  const int cb = jl * M, ce = jend * M;
+  const int jmax = (int)((F - f0) < jend ? (F - f0) : jend);
+  float* const s32 = a.S32 ? (cvalid ? a.S32 + c * F + f0 : a.scratch32 + lane * kShMaxFpm) : nullptr;
+  double* const s64 = a.S_out ? (cvalid ? a.S_out + c * F + f0 : a.scratch64 + lane * kShMaxFpm) : nullptr;
+  const float nan = __int_as_float(0x7fc00000);
+  const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16), tb = ta + 256u;
+  float acc0 = 0.f, acc1 = 0.f;  // even and odd columns
+  int fend = cb + M;             // where frequency jl ends (warp-uniform)
+  auto term = [&](uint32_t va, uint32_t vb) {
+    const float A = __uint_as_float(va) * sa, den = __uint_as_float(vb) * sw + cal;
+    return den >= 1.17549435e-38f ? (A * A) * rcp_approx(den) : 0.f;
+  };
+  if (a.nchunks == 0) {  // no observations: no MMA has written the accumulators
+    for (; jl < jmax; ++jl) {
+      if (s32) s32[jl] = 0.f;
+      if (s64) s64[jl] = 0.0;
+    }
+    return;
+  }
+  uint32_t na[8], nb[8];
+  int c0 = cb & ~7;
+  const int clast = (ce - 1) & ~7;
+  tmem_ld8_issue(ta + (uint32_t)c0, na);
+  tmem_ld8_issue(tb + (uint32_t)c0, nb);
+#pragma unroll 1
+  for (; c0 < ce; c0 += 8) {
+    uint32_t va[8], vb[8];
+    tmem_wait_ld8(na);
+    tmem_wait_ld8(nb);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      va[u] = na[u];
+      vb[u] = nb[u];
+    }
+    // (the last step loads its own columns again: no load is conditional, so none is moved before its wait)
+    const uint32_t cn = (uint32_t)(c0 < clast ? c0 + 8 : clast);
+    tmem_ld8_issue(ta + cn, na);
+    tmem_ld8_issue(tb + cn, nb);
+    if (c0 >= cb && fend > c0 + 8) {
+#pragma unroll
+      for (int u = 0; u < 8; u += 2) {
+        acc0 += term(va[u], vb[u]);
+        acc1 += term(va[u + 1], vb[u + 1]);
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int col = c0 + u;
+        if (col >= cb && col < ce) {  // warp-uniform, as all conditions on columns
+          (u & 1 ? acc1 : acc0) += term(va[u], vb[u]);
+          if (col + 1 == fend) {  // frequency jl complete
+            if (jl < jmax) {
+              const float S = cbad ? nan : acc0 + acc1;
+              if (s32) s32[jl] = S;
+              if (s64) s64[jl] = (double)S;
+            }
+            acc0 = acc1 = 0.f;
+            ++jl;
+            fend += M;
+          }
+        }
+      }
+    }
+  }
+  tmem_wait_ld8(na);
+  tmem_wait_ld8(nb);
+}
+
+// kPaired: the two accumulators hold the two parts of two groups of curves at
+// fpm frequencies: both multiply one H operand, and the epilogue finds a
+// curve's sums in one lane. Else both parts of one group, rows side by side, at
+// 2 fpm frequencies, two operands. A chunk's MMAs are the same, its one-hot
+// stores halve; V, read from L2, doubles. A chunk takes 0.69 us either way, the
+// MMAs' own time (1.76e15 FLOP/s with what the padding leaves); what the pair
+// saves is the epilogue, without shuffles: 512 curves x 50000 frequencies, M =
+// 20, 100 times 1133 us -> 895 with the epilogue below, 805 with it deferred;
+// 1000 times 3187 -> 2930; M = 50 7219 -> 6927.
+template <bool kPaired>
 __global__ void __launch_bounds__(kShThreads, 1) shared_mma_kernel(const SharedArgs a) {
+  constexpr int kVSlot = (kPaired ? 2 : 1) * kShChunkBytes, kHSlot = kShHSlotBytes / (kPaired ? 2 : 1);
+  static_assert(kShVSlots * kVSlot + 2 * kHSlot <= kShVSlots * kShChunkBytes + 2 * kShHSlotBytes, "same area");
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* sV = smem + kOffV;
-  unsigned char* sH = smem + kOffH;
+  unsigned char* sH = sV + kShVSlots * kVSlot;
   uint8_t* sOld = smem + kOffOld;
   double* sF = reinterpret_cast<double*>(smem + kOffF);
   double* sT = reinterpret_cast<double*>(smem + kOffStage);
@@ -338,12 +443,12 @@ __global__ void __launch_bounds__(kShThreads, 1) shared_mma_kernel(const SharedA
   volatile int* s_abort = reinterpret_cast<volatile int*>(tslot + 1);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int M = a.M, fpm = a.fpm, Nm = a.n_mma, FP = 2 * fpm, rows_used = fpm * M;
+  const int M = a.M, fpm = a.fpm, Nm = a.n_mma, FP = kPaired ? fpm : 2 * fpm, rows_used = fpm * M;
   const int npairs = FP * kShObs;
   const int64_t F = a.nfreq, n = a.n, nch = a.nchunks;
   const bool resident = n <= kShStage;
   const bool grid_bad = (*(volatile unsigned*)a.status & kStatusGrid) != 0u;
-  const int64_t items = grid_bad ? 0 : a.ngroups * a.npass;
+  const int64_t items = grid_bad ? 0 : a.units * a.npass;
   const int64_t my_items = (int64_t)blockIdx.x < items ? (items - 1 - blockIdx.x) / gridDim.x + 1 : 0;
   const float cal = (float)a.inv_alpha2;
   const double df = (F > 1) ? (a.freqs[F - 1] - a.freqs[0]) / (double)(F - 1) : 0.0;
@@ -371,7 +476,7 @@ __global__ void __launch_bounds__(kShThreads, 1) shared_mma_kernel(const SharedA
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   // H starts as all pairs in bin 0 (rows beyond fpm * M stay zero for good)
-  for (int e = tid; e < 2 * kShHSlotBytes / 16; e += kShThreads)
+  for (int e = tid; e < 2 * kHSlot / 16; e += kShThreads)
     reinterpret_cast<uint4*>(sH)[e] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
   for (int e = tid; e < npairs; e += kShThreads) {
@@ -380,7 +485,7 @@ __global__ void __launch_bounds__(kShThreads, 1) shared_mma_kernel(const SharedA
     const uint32_t r = (uint32_t)((j - op * fpm) * M);
     const uint32_t w = lane_off + (uint32_t)op * op_bytes + (r >> 3) * 256u + (r & 7u) * 16u;
     for (int q = 0; q < 2; ++q) {
-      *reinterpret_cast<uint32_t*>(sH + q * kShHSlotBytes + w) = kOneOne;
+      *reinterpret_cast<uint32_t*>(sH + q * kHSlot + w) = kOneOne;
       sOld[q * kMaxPairs + e] = 0;
     }
   }
@@ -409,14 +514,21 @@ __global__ void __launch_bounds__(kShThreads, 1) shared_mma_kernel(const SharedA
       // the V-load cursor (item lk of this CTA, chunk lch) runs two chunks ahead
       // of the MMA cursor; both advance incrementally (no 64-bit division per chunk)
       int64_t lk = 0, lch = 0;
-      const unsigned char* limg = a.image + (size_t)(blockIdx.x / a.npass) * (size_t)nch * kShChunkBytes;
+      const size_t gbytes = (size_t)nch * kShChunkBytes;  // one group's image
+      auto unit_image = [&](int64_t it) {
+        return a.image + (size_t)(a.group0 + (it / a.npass) * (kPaired ? 2 : 1)) * gbytes;
+      };
+      const unsigned char* limg = unit_image(blockIdx.x);
       auto load_next = [&](int slot) {
-        bulk_load(sV + slot * kShChunkBytes, limg + (size_t)lch * kShChunkBytes, kShChunkBytes, &bar_v[slot]);
+        mbar_expect(&bar_v[slot], kVSlot);
+        bulk_load(sV + slot * kVSlot, limg + (size_t)lch * kShChunkBytes, kShChunkBytes, &bar_v[slot]);
+        if (kPaired)
+          bulk_load(sV + slot * kVSlot + kShChunkBytes, limg + gbytes + (size_t)lch * kShChunkBytes, kShChunkBytes,
+                    &bar_v[slot]);
         if (++lch == nch) {
           lch = 0;
           ++lk;
-          const int64_t it = blockIdx.x + lk * gridDim.x;
-          limg = a.image + (size_t)(it / a.npass) * (size_t)nch * kShChunkBytes;
+          limg = unit_image(blockIdx.x + lk * gridDim.x);  // past the last item: formed, not read
         }
       };
       if (iop == 0)
@@ -444,8 +556,8 @@ __global__ void __launch_bounds__(kShThreads, 1) shared_mma_kernel(const SharedA
           ph_tfree ^= 1u;
         }
         fence_after_sync();
-        const uint64_t dvs = dv0 + (uint64_t)((vs * kShChunkBytes) >> 4);
-        const uint64_t dhs = dh0 + (uint64_t)((s * kShHSlotBytes + iop * (int)op_bytes) >> 4);
+        const uint64_t dvs = dv0 + (uint64_t)((vs * kVSlot + (kPaired ? iop * kShChunkBytes : 0)) >> 4);
+        const uint64_t dhs = dh0 + (uint64_t)((s * kHSlot + (kPaired ? 0 : iop * (int)op_bytes)) >> 4);
 #pragma unroll
         for (int ks = 0; ks < kShKSteps; ++ks) {
           const uint32_t acc = (ch > 0 || ks > 0) ? 1u : 0u;
@@ -476,18 +588,39 @@ __global__ void __launch_bounds__(kShThreads, 1) shared_mma_kernel(const SharedA
     uint32_t ph_empty = 0u, ph_acc = 0u;  // per-slot parities as bits
     bool staged = false;
     int64_t gc = 0;
+    // a pair's epilogue runs once the next item's first chunk is built, so that
+    // staging and building overlap the last MMAs
+    int64_t gprev = 0, fprev = 0;
+    auto finish_pair = [&]() {
+      const int64_t c = gprev * kShCurves + (warp & 3) * 32 + lane;  // loads before the wait
+      const bool cbad = c < a.ncurves && a.curve_bad[c];
+      const float2 scale = reinterpret_cast<const float2*>(a.inv_scale)[c];
+      if (!fail && nch > 0) {
+        fail = !mbar_wait_ab(bar_acc, ph_acc, s_abort, wait_limit, suspend_ns);
+        fence_after_sync();
+      }
+      fail = __any_sync(0xffffffffu, fail);
+      if (fail && lane == 0) *s_abort = 1;
+      if (!fail) pair_epilogue(a, tmem, c, fprev, cbad, scale, warp, lane);
+      fence_before_sync();
+      __syncwarp();
+      if (!fail && nch > 0 && lane == 0) mbar_arrive(bar_tfree);
+      ph_acc ^= 1u;
+    };
     for (int64_t k = 0; k < my_items; ++k) {
       const int64_t item = blockIdx.x + k * gridDim.x;
-      const int64_t g = item / a.npass, p = item % a.npass;
+      const int64_t g = a.group0 + (item / a.npass) * (kPaired ? 2 : 1), p = item % a.npass;
       const int64_t f0 = p * FP;
-      const double fa = a.freqs[f0];
+      // anchors every 2 fpm frequencies, whichever way a pass takes them
+      const int jo = kPaired && (p & 1) ? fpm : 0;
+      const double fa = a.freqs[f0 - jo];
       if (k > 0) builders_sync(kShBuilders);  // every builder is done with the previous item's sF and stage
       bool nonlin = false;
       for (int j = tid; j < FP; j += kShBuilders) {
         const int64_t fi = f0 + j;
         const double f = fi < F ? a.freqs[fi] : 0.0;
         sF[j] = f;
-        if (fi < F && fabs(f - fma((double)j, df, fa)) * tmax > kGridTolCycles) nonlin = true;
+        if (fi < F && fabs(f - fma((double)(jo + j), df, fa)) * tmax > kGridTolCycles) nonlin = true;
       }
       const bool lin = !builders_or(nonlin, kShBuilders);
       for (int64_t ch = 0; ch < nch; ++ch, ++gc) {
@@ -513,7 +646,7 @@ __global__ void __launch_bounds__(kShThreads, 1) shared_mma_kernel(const SharedA
         fail = __any_sync(0xffffffffu, fail);
         if (fail && lane == 0) *s_abort = 1;  // the other roles stop waiting
         if (!fail) {
-          unsigned char* hs = sH + s * kShHSlotBytes;
+          unsigned char* hs = sH + s * kHSlot;
           uint8_t* old = sOld + s * kMaxPairs;
           const int ib = (int)(ch % kShStageChunks) * kShObs + lane;
           const bool obs_ok = ch * kShObs + lane < n;
@@ -538,9 +671,9 @@ __global__ void __launch_bounds__(kShThreads, 1) shared_mma_kernel(const SharedA
               const int e2 = e + kShBuilders;
               const bool two = e2 < npairs;  // warp-uniform
               const int ja = e >> 5, jb = e2 >> 5;
-              const unsigned ma = (obs_ok && f0 + ja < F) ? bin_of_phase(P + (unsigned long long)ja * D, (unsigned)M) : 0u;
+              const unsigned ma = (obs_ok && f0 + ja < F) ? bin_of_phase(P + (unsigned long long)(jo + ja) * D, (unsigned)M) : 0u;
               const unsigned mb =
-                  (two && obs_ok && f0 + jb < F) ? bin_of_phase(P + (unsigned long long)jb * D, (unsigned)M) : 0u;
+                  (two && obs_ok && f0 + jb < F) ? bin_of_phase(P + (unsigned long long)(jo + jb) * D, (unsigned)M) : 0u;
               const unsigned oa = old[e], ob = two ? old[e2] : 0u;
               put(e, ma, oa);
               if (two) put(e2, mb, ob);
@@ -556,19 +689,26 @@ __global__ void __launch_bounds__(kShThreads, 1) shared_mma_kernel(const SharedA
           __syncwarp();
           if (lane == 0) mbar_arrive(&bar_full[s]);
         }
+        if (kPaired && ch == 0 && k > 0) finish_pair();
       }
-      // epilogue: all builder warps. Warp w reads TMEM lanes 32 (w % 4) .. + 31
-      // of accumulator (w / 4) % 2, columns [0, split) for w < 8 and
-      // [split, fpm M) above (split a multiple of 8 near the middle); the
-      // partial sum of a frequency that straddles the split is handed over
-      // through shared memory.
-      float* sPart = reinterpret_cast<float*>(smem + kOffPart);
+      if constexpr (kPaired) {
+        gprev = g;
+        fprev = f0;
+        if (nch == 0 || k + 1 == my_items) finish_pair();
+        continue;
+      }
       if (!fail && nch > 0) {
         fail = !mbar_wait_ab(bar_acc, ph_acc, s_abort, wait_limit, suspend_ns);
         fence_after_sync();
       }
       fail = __any_sync(0xffffffffu, fail);
       if (fail && lane == 0) *s_abort = 1;
+      // epilogue: all builder warps. Warp w reads TMEM lanes 32 (w % 4) .. + 31
+      // of accumulator (w / 4) % 2, columns [0, split) for w < 8 and
+      // [split, fpm M) above (split a multiple of 8 near the middle); the
+      // partial sum of a frequency that straddles the split is handed over
+      // through shared memory.
+      float* sPart = reinterpret_cast<float*>(smem + kOffPart);
       const int quarter = warp & 3, op = (warp >> 2) & 1, half = warp >> 3;
       const int row = quarter * 32 + lane;
       const int64_t c = g * kShCurves + (row >> 1);
@@ -798,7 +938,9 @@ cudaError_t launch_dense_topk32(const DenseTopk32Args& t, int64_t ncurves, cudaS
 }
 
 cudaError_t shared_init_attributes() {
-  return cudaFuncSetAttribute(shared_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+  const cudaError_t e = cudaFuncSetAttribute(shared_mma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(shared_mma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
 }
 
 size_t shared_smem_bytes() { return kSmemBytes; }
@@ -817,13 +959,27 @@ cudaError_t launch_shared(const SharedArgs& a, int nsm, cudaStream_t st) {
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  const int64_t items = a.ngroups * a.npass;
-  if (items > 0) {
-    const int grid = (int)(items < nsm ? items : nsm);
+  if (a.ngroups > 0 && a.nfreq > 0) {
     if (a.timing_start) cudaEventRecord(a.timing_start, st);
-    shared_mma_kernel<<<grid, kShThreads, kSmemBytes, st>>>(a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    // groups two at a time, the one left over by itself
+    SharedArgs b = a;
+    b.group0 = 0;
+    b.units = a.ngroups / 2;
+    b.npass = (a.nfreq + a.fpm - 1) / a.fpm;
+    if (b.units > 0) {
+      const int64_t items = b.units * b.npass;
+      shared_mma_kernel<true><<<(int)(items < nsm ? items : nsm), kShThreads, kSmemBytes, st>>>(b);
+      e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+    }
+    if (a.ngroups % 2) {
+      b.group0 = a.ngroups - 1;
+      b.units = 1;
+      b.npass = (a.nfreq + 2 * a.fpm - 1) / (2 * a.fpm);
+      shared_mma_kernel<false><<<(int)(b.npass < nsm ? b.npass : nsm), kShThreads, kSmemBytes, st>>>(b);
+      e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+    }
     if (a.timing_stop) cudaEventRecord(a.timing_stop, st);
   }
   if (a.k > 0 && a.ncurves > 0) {

@@ -17,8 +17,11 @@ struct SharedArgs {
   int M;
   int fpm;                  // frequencies per accumulator (256 / M)
   int n_mma;                // MMA N: fpm * M rounded up to 16
-  int64_t npass;            // frequency passes of 2 * fpm frequencies
   int64_t ngroups;          // groups of 64 curves
+  // of one launch of the MMA kernel (launch_shared):
+  int64_t group0;           // its first group
+  int64_t units;            // groups, or pairs of groups
+  int64_t npass;            // frequency passes of 2 fpm frequencies (a group), fpm (a pair)
   int64_t nchunks;          // chunks of 32 observations
   unsigned char* image;     // fp16 hi/lo operand image [ngroups][nchunks][16 KB]
   float* inv_scale;         // [ngroups * 64][2]: 2^-e for a and w
