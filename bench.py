@@ -42,9 +42,9 @@ WORKLOAD = "sweep_100k"
 NSM_NOMINAL = 152
 SM_MAX_MHZ_NOMINAL = 2070.0
 SMEM_EVALS_PER_CLK_SM = 8  # 16 B (A, B) read-modify-write per evaluation at 128 B/clk/SM
-KERNELS_PER_STEP = 5  # prep, tile_dev, tile, merge, latch
+KERNELS_PER_STEP = 3  # prep, tile, merge
 SWEEP_MS = (10, 20, 50)  # bin counts of the throughput sweep
-ENTROPY_INST_PER_EVAL = 9.86  # thread instructions per evaluation of the dense phase-entropy kernel (ncu, M = 20)
+ENTROPY_INST_PER_EVAL = 6.94  # thread instructions per evaluation of the dense phase-entropy kernel (ncu, M = 20)
 
 
 def entropy_R(M: int) -> int:
@@ -53,10 +53,10 @@ def entropy_R(M: int) -> int:
     return 8 if M <= 12 else (4 if M <= 24 else (2 if M <= 96 else 1))
 # DRAM bytes (read + write) of one tile-kernel launch at M = 20, from an ncu capture of a 1e4-curve sweep
 # batch over 2e4 frequencies (dram__bytes_read.sum + dram__bytes_write.sum). The kernel reads each curve
-# from DRAM once per launch (t and the staged weights, about 16.7 B per observation; per-tile re-reads
-# hit L2), so a full launch adds only the larger grid (8 B per extra frequency). Valid only for the
+# from DRAM once per launch (its phase records and weights, about 33 B per observation; per-tile
+# re-reads hit L2), so a full launch adds only the larger grid (8 B per extra frequency). Valid only for the
 # kernel source it was measured on (sha256 prefix of the tile-kernel sources, tile_source_hash).
-TILE_TRAFFIC = {"source_sha256_16": "ce9276e3f4830ec5", "bytes": 142.63e6, "nfreq": 20_000}
+TILE_TRAFFIC = {"source_sha256_16": "9a63431f73948b4e", "bytes": 283.59e6, "nfreq": 20_000}
 
 
 # ---------------------------------------------------------------- workload generation (spawned workers)
@@ -794,12 +794,12 @@ def run_configs_entropy(ctx, peak):
         torch.cuda.synchronize()
         ev = float(w.t.size) * w.nfreq
         rate = ev / (e0.elapsed_time(e1) / reps / 1e3)
-        # shared-memory term: per observation and warp, R count loads and R
-        # count stores of 4 B per lane (one wavefront each) plus the staged
-        # 16-byte record read by every lane (two wavefronts), over 32 R
-        # evaluations; the kernel's frequencies per thread R follow M
+        # shared-memory term: per observation and warp, R count reductions of
+        # 4 B per lane (one wavefront each) plus the staged 16-byte record read
+        # by every lane (two wavefronts), over 32 R evaluations; the kernel's
+        # frequencies per thread R follow M
         R = entropy_R(M)
-        smem_roof = peak / SMEM_EVALS_PER_CLK_SM * (32.0 * R / (2.0 * R + 2.0))
+        smem_roof = peak / SMEM_EVALS_PER_CLK_SM * (32.0 * R / (R + 2.0))
         issue_roof = peak / SMEM_EVALS_PER_CLK_SM * 128.0 / ENTROPY_INST_PER_EVAL
         terms = {"smem": smem_roof}
         if R == 4:  # the instruction mix was measured at R = 4 (M = 20)
@@ -812,8 +812,8 @@ def run_configs_entropy(ctx, peak):
                                        "binding": binding, "frac_binding": rate / terms[binding],
                                        "frac_smem": rate / smem_roof, "R": R},
                           "status": ctx.status(),
-                          "note": f"roof terms: R count read-modify-writes (4 B per lane) and one 16 B broadcast "
-                                  f"record per observation and warp, 2 R + 2 wavefronts per 32 R evaluations; "
+                          "note": f"roof terms: R count reductions (4 B per lane) and one 16 B broadcast "
+                                  f"record per observation and warp, R + 2 wavefronts per 32 R evaluations; "
                                   f"128 thread instructions/clk/SM over {ENTROPY_INST_PER_EVAL} instructions per "
                                   f"evaluation (ncu, M = 20, R = 4)"}),
               flush=True)

@@ -169,8 +169,8 @@ FPW_API int fpw_periodogram_batch_ex(fpw_ctx* ctx, void* stream, const fpw_param
  * Other arguments as fpw_periodogram_batch_ex. FP32 sums only and at most 256
  * threads per block (FPW_ENOTSUP otherwise); nfreq < 2^25 when k > 0.
  * (M_max; groups) = (60; 3, 6, 15), (40; 2, 4, 10) and (20; 1, 2, 4), listed in
- * that order, run a combination compiled for them (same results bit for bit,
- * 7-14 % faster at the default shapes). Stream-ordered. */
+ * that order, run a combination compiled for them where a curve's weights
+ * lie in [2^-60, 2^60] (same results bit for bit). Stream-ordered. */
 FPW_API int fpw_periodogram_batch_multi(fpw_ctx* ctx, void* stream, const fpw_params* params, const int64_t* offsets,
                                         const int64_t* offsets_host, int64_t ncurves, const double* t,
                                         const double* x, const double* sigma, const double* freqs, int64_t nfreq,
@@ -180,8 +180,8 @@ FPW_API int fpw_periodogram_batch_multi(fpw_ctx* ctx, void* stream, const fpw_pa
 /* Curves that share one set of observation times (Section 4 and the batch
  * routine of Appendix D: many light curves of one field observed in the same
  * exposures). Eq. 1 per curve with the bins computed once per (observation,
- * frequency); on GB300 the bin sums of 64 curves at a time are one tensor-core
- * product of the fp16 hi/lo split of (x w, w) with the one-hot bin matrix
+ * frequency); on GB300 the bin sums of 128 or 64 curves at a time are tensor-core
+ * products of the fp16 hi/lo split of (x w, w) with the one-hot bin matrix
  * (FP32 accumulation), so the result matches FP32 bin sums of the batched call.
  *   t:        device float64[n], the shared times (finite)
  *   x, sigma: device float64[ncurves * n], curve c's values at [c * n + i]
@@ -206,8 +206,9 @@ FPW_API int fpw_periodogram_shared(fpw_ctx* ctx, void* stream, const fpw_params*
  * curve's times mapped to [-1, 1] over its span), and
  *   S = u^T (I / alpha^2 + E^T W E)^-1 u,  u = E^T W x,  W = (C_B + C_sigma)^-1,
  * E the one-hot bin matrix; with 1/alpha^2 = 0 empty bins are dropped. K = 0
- * (or beta = 0) gives Eq. 1. Bin sums are FP32, the per-frequency K x K solve
- * binary64.
+ * (or beta = 0) gives Eq. 1. Bin sums are FP32; the per-frequency reduction and K x
+ * K solve carry FP32 pairs (2^-46), or binary64 where a curve's weights or
+ * residuals leave [2^-30, 2^30] or its I + B^T D B has a trace above 2^25.
  *   offsets, t, x, sigma, freqs, k, topk_idx, topk_S, S_out: as
  *       fpw_periodogram_batch_ex (device pointers; ncurves <= 65535)
  *   K: 0..4 basis functions; beta >= 0: prior standard deviation of each
@@ -217,8 +218,7 @@ FPW_API int fpw_periodogram_shared(fpw_ctx* ctx, void* stream, const fpw_params*
  *       per bin (FPW_ENOTSUP beyond)
  * params: FPW_PHASE_FIXED64 and FPW_ACCUM_FP32 only; inv_alpha2 and
  * peak_mode apply; threads (32..128) and freqs_per_thread (1 or 2) set the
- * block shape (0 = 128 threads, fewer where M needs it, and two frequencies
- * per thread for K <= 1 where they fit); a shape whose bins do not fit (R
+ * block shape (0 = chosen by M and K); a shape whose bins do not fit (R
  * times the bound on M above) or any other value gives FPW_ENOTSUP.
  * Scratch held by the context: 32 bytes per observation,
  * 168 bytes per curve and,
@@ -321,8 +321,9 @@ FPW_API int fpw_ctx_set_shape(fpw_ctx* ctx, int M_lo, int M_hi, int64_t n_lo, in
 FPW_API int fpw_ctx_clear_shapes(fpw_ctx* ctx);
 
 /* The tile-kernel shape of the context's most recent batched or single-curve
- * call that ran the tile kernel: threads per block, frequencies per thread,
- * observations staged per pass and the persistent grid (blocks). All zero
+ * call that ran the tile kernel: threads per block, frequencies per thread and
+ * observations per pass of the shape that placed its phase anchors, and the
+ * persistent grid (blocks). All zero
  * before the first such call. Pass the first three as fpw_params threads /
  * freqs_per_thread / obs_chunk to launch another call with the same tiles.
  * Errors: FPW_EINVAL (null pointer). */
