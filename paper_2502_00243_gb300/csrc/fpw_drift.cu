@@ -717,15 +717,16 @@ int drift_threads(int M, int K, int smem_optin) {
 // (the bins of a span take the same room however it is divided), else R = 1
 // (measured at 8 warps against 4: M = 50, K = 3 2185 us against 2543, K = 4, M =
 // 20 1971 at R = 2, 8 warps, against 2412 at R = 4; at 10 against 20: M = 20,
-// K = 3 1456 against 1668).
-void drift_split(int M, int K, int span, int smem_optin, int* T, int* R) {
+// K = 3 1456 against 1668) and eight per SM in the whole call: fewer spans than
+// that are over sooner the more threads each has.
+void drift_split(int M, int K, int span, int64_t nspans, int nsm, int smem_optin, int* T, int* R) {
   const size_t block = drift_smem_bytes(M, K, span, 1) + 1024;
   for (int r = 4; r >= 1; r >>= 1) {
     const int t = span / r;
     if (span % r || t % 32 || t > 128) continue;
     *T = t;
     *R = r;
-    if ((smem_optin + 1024) / block * (size_t)(t / 32) >= 8) return;
+    if ((smem_optin + 1024) / block * (size_t)(t / 32) >= 8 && nspans * (t / 32) >= 8 * (int64_t)nsm) return;
   }
 }
 

@@ -1380,7 +1380,8 @@ int fpw_periodogram_drift(fpw_ctx* ctx, void* stream, const fpw_params* params, 
   a.b2cal = pair(beta * beta * p.inv_alpha2);
   a.span = T * R;
   int Tl = T, Rl = R;
-  if (p.threads == 0 && p.freqs_per_thread == 0) drift_split(M, K, T * R, ctx->smem_optin, &Tl, &Rl);
+  if (p.threads == 0 && p.freqs_per_thread == 0)
+    drift_split(M, K, T * R, (nfreq + T * R - 1) / (T * R) * ncurves, ctx->nsm, ctx->smem_optin, &Tl, &Rl);
   a.payload = ctx->dr_payload.p;
   a.tabs = static_cast<double*>(ctx->dr_tabs.p);
   a.H0 = static_cast<double*>(ctx->dr_H0.p);

@@ -19,7 +19,8 @@
 //   phases (phase_fixed64: the integer product of the binary64 significands),
 //   so bins equal floor(M frac(t f)) except within 2^-32 of a cycle below an edge.
 // * Groups of 64 curves are taken two at a time, one accumulator for part 0 and
-//   one for part 1 of their 128 curves; a group left over has its own launch,
+//   one for part 1 of their 128 curves; a group left over (or every group, where
+//   few items make pairs the slower way) is taken by itself,
 //   parts in neighbouring rows, an accumulator for each half of the pass.
 // * One CTA per SM (persistent over (groups, frequency pass) work items) holds
 //   two accumulators of 128 x N (N = frequencies per accumulator x M <= 256) in
@@ -285,7 +286,7 @@ __global__ void __launch_bounds__(256) shared_prep_kernel(const SharedArgs a) {
   // w of the pair's 128 curves; in a group by itself the parts are neighbours
   const int64_t g = c / kShCurves;
   const size_t gbytes = (size_t)a.nchunks * kShChunkBytes;
-  const bool paired = g < (a.ngroups & ~(int64_t)1);
+  const bool paired = g < a.pair_groups;
   const uint32_t row = paired ? (uint32_t)(c % (2 * kShCurves)) : (uint32_t)(c % kShCurves) * 2u;
   unsigned char* const img = a.image + (size_t)(paired ? (g & ~(int64_t)1) : g) * gbytes;
   const size_t wpart = paired ? gbytes : 0;
@@ -927,9 +928,9 @@ __global__ void __launch_bounds__(kShTopkThreads) dense_topk32_kernel(const Dens
       best = v > best ? v : best;
     }
     if (lane == 0) {
-      const unsigned e = 0xFFFFFFFFu - (unsigned)best;
-      oi[q] = best ? (int32_t)e : -1;
-      os[q] = best ? S[e] : __int_as_float(0x7fc00000);
+      const unsigned rank = (unsigned)(best >> 32);
+      oi[q] = best ? (int32_t)(0xFFFFFFFFu - (unsigned)best) : -1;
+      os[q] = __uint_as_float(rank <= 1u ? 0x7fc00000u : ((rank >> 31) ? rank & 0x7FFFFFFFu : ~rank));
     }
     best = __shfl_sync(0xffffffffu, best, 0);
     if (best && head == best) head = ++h < k ? lists[lane][h] : 0ull;
@@ -968,9 +969,22 @@ cudaError_t shared_init_attributes() {
 
 size_t shared_smem_bytes() { return kSmemBytes; }
 
-cudaError_t launch_shared(const SharedArgs& a, int nsm, cudaStream_t st) {
-  const int64_t slots = a.ngroups * kShCurves;
+// Groups taken in pairs: all but an odd one, where that is over sooner than
+// group by group, in rounds of items over the SMs (a pair's item takes 0.9 of a
+// group's, and the odd group's launch fills rounds of its own: 130 curves, M =
+// 35, 2449 frequencies took 110 us in pairs, 3 + 2 rounds, and 100 in 4).
+static int64_t shared_pair_groups(int64_t ngroups, int64_t nfreq, int fpm, int nsm) {
+  const int64_t np = (nfreq + fpm - 1) / fpm, ns = (nfreq + 2 * fpm - 1) / (2 * fpm);
+  auto rounds = [&](int64_t items) { return (items + nsm - 1) / nsm; };
+  const int64_t pairs = 9 * rounds(ngroups / 2 * np) + 10 * rounds(ngroups % 2 * ns);
+  return pairs <= 10 * rounds(ngroups * ns) ? (ngroups & ~(int64_t)1) : 0;
+}
+
+cudaError_t launch_shared(const SharedArgs& args, int nsm, cudaStream_t st) {
+  const int64_t slots = args.ngroups * kShCurves;
   if (slots <= 0) return cudaSuccess;
+  SharedArgs a = args;
+  a.pair_groups = shared_pair_groups(a.ngroups, a.nfreq, a.fpm, nsm);
   shared_prep_kernel<<<(unsigned)slots, 256, 0, st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -984,10 +998,9 @@ cudaError_t launch_shared(const SharedArgs& a, int nsm, cudaStream_t st) {
   }
   if (a.ngroups > 0 && a.nfreq > 0) {
     if (a.timing_start) cudaEventRecord(a.timing_start, st);
-    // groups two at a time, the one left over by itself
     SharedArgs b = a;
     b.group0 = 0;
-    b.units = a.ngroups / 2;
+    b.units = a.pair_groups / 2;
     b.npass = (a.nfreq + a.fpm - 1) / a.fpm;
     if (b.units > 0) {
       const int64_t items = b.units * b.npass;
@@ -995,11 +1008,12 @@ cudaError_t launch_shared(const SharedArgs& a, int nsm, cudaStream_t st) {
       e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }
-    if (a.ngroups % 2) {
-      b.group0 = a.ngroups - 1;
-      b.units = 1;
-      b.npass = (a.nfreq + 2 * a.fpm - 1) / (2 * a.fpm);
-      shared_mma_kernel<false><<<(int)(b.npass < nsm ? b.npass : nsm), kShThreads, kSmemBytes, st>>>(b);
+    b.group0 = a.pair_groups;
+    b.units = a.ngroups - a.pair_groups;
+    b.npass = (a.nfreq + 2 * a.fpm - 1) / (2 * a.fpm);
+    if (b.units > 0) {
+      const int64_t items = b.units * b.npass;
+      shared_mma_kernel<false><<<(int)(items < nsm ? items : nsm), kShThreads, kSmemBytes, st>>>(b);
       e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }

@@ -18,7 +18,8 @@ struct SharedArgs {
   int fpm;                  // frequencies per accumulator (256 / M)
   int n_mma;                // MMA N: fpm * M rounded up to 16
   int64_t ngroups;          // groups of 64 curves
-  // of one launch of the MMA kernel (launch_shared):
+  // set by launch_shared; the last three for each launch of the MMA kernel:
+  int64_t pair_groups;      // groups taken in pairs: the first of them
   int64_t group0;           // its first group
   int64_t units;            // groups, or pairs of groups
   int64_t npass;            // frequency passes of 2 fpm frequencies (a group), fpm (a pair)
@@ -87,7 +88,8 @@ struct DriftArgs {
   cudaEvent_t timing_start;
   cudaEvent_t timing_stop;
 };
-void drift_split(int M, int K, int span, int smem_optin, int* T, int* R);  // the launch of a span of frequencies
+// the launch of nspans spans of `span` frequencies
+void drift_split(int M, int K, int span, int64_t nspans, int nsm, int smem_optin, int* T, int* R);
 int drift_threads(int M, int K, int smem_optin);  // threads per block, 0 if M is too large
 size_t drift_smem_bytes(int M, int K, int T, int R);  // R frequencies per thread (1 or 2)
 bool drift_fits(int M, int K, int T, int R, int smem_optin);
