@@ -216,10 +216,11 @@ cudaError_t launch_entropy_dense(const double* t, int64_t n, const double* freqs
   // frequencies, counts/s at R = 8, 4, 2, 1: M = 10 3.32e12, 3.11e12, 2.51e12,
   // 1.72e12; M = 20 2.51e12 (two blocks per SM), 3.05e12, 2.49e12, 1.72e12;
   // M = 50 R = 4 2.07e12, R = 2 2.31e12), and fewer while that leaves under two
-  // blocks per SM (1e5 frequencies, M = 10: 1.21e12, 1.38e12, 1.45e12, 1.10e12).
+  // blocks per SM (1e5 frequencies, M = 10: 1.21e12, 1.38e12, 1.45e12, 1.10e12),
+  // under one from R = 2 on (6e4 frequencies, M = 31: R = 1 2 % slower; 1e4: 10 % faster).
   const int span = M <= 12 ? 1024 : (M <= 24 ? 512 : (M <= 96 ? 256 : 128));
   int R = span / kEntThreads;
-  while (R > 1 && (nfreq + R * kEntThreads - 1) / (R * kEntThreads) < 2 * nsm) R >>= 1;
+  while (R > 1 && (nfreq + R * kEntThreads - 1) / (R * kEntThreads) < (R > 2 ? 2 : 1) * nsm) R >>= 1;
   const void* fn = R == 8   ? reinterpret_cast<const void*>(&entropy_dense_kernel<8>)
                    : R == 4 ? reinterpret_cast<const void*>(&entropy_dense_kernel<4>)
                    : R == 2 ? reinterpret_cast<const void*>(&entropy_dense_kernel<2>)

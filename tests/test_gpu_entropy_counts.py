@@ -20,8 +20,8 @@ def test_counts_at_the_edges(M, F, n):
     _check(M, F, n)
 
 
-# blocks of 128 R frequencies while at least 304 of them: one frequency before and after each change of R
-@pytest.mark.parametrize("M,F", [(M, 303 * 128 * R + d) for M, rs in ((5, (8, 4, 2)), (20, (4, 2)), (50, (2,)))
+# blocks of 128 R frequencies while at least 304 of them (152 for R = 2): one frequency before and after each change of R
+@pytest.mark.parametrize("M,F", [(M, (303 if R > 2 else 151) * 128 * R + d) for M, rs in ((5, (8, 4, 2)), (20, (4, 2)), (50, (2,)))
                                  for R in rs for d in (0, 1)])
 def test_counts_where_the_launch_changes(M, F):
     _check(M, F, 9)
