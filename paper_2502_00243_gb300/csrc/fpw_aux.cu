@@ -1,7 +1,8 @@
 // Auxiliary FPW kernels:
-//   prep         w_i = 1/sigma_i^2, a_i = x_i w_i (Eq. 1's weights) and the
-//                phase at f_0 and step per observation, once per call; input
-//                validation; the grid's deviation from a line per anchor block
+//   prep         w_i = 1/sigma_i^2, a_i = x_i w_i (Eq. 1's weights), the time as
+//                a fixed-point number and the phase step per observation, once
+//                per call; input validation; the grid's deviation from a line
+//                per anchor block
 //   merge        per-curve top-k peaks from the per-item candidates (Section 3.5)
 //   plain        the binary64 reference form: fl(t f) per evaluation, binary64
 //                bins (Appendix A.1) and sums (Eq. 1), one curve per launch
@@ -37,30 +38,32 @@ __global__ void prep_kernel(const PrepArgs a) {
   // one division a block: a binary64 operation takes a warp 50 clocks, a division
   // 25 of them
   __shared__ double s_df;
+  __shared__ int s_bits;
   if (threadIdx.x == 0) {
     s_df = (a.nfreq > 1) ? (a.freqs[a.nfreq - 1] - f0) / (double)(a.nfreq - 1) : 0.0;
     if (a.df && blockIdx.x == 0) *a.df = s_df;
+    if (a.rec) {
+      s_bits = a.nobs > 0 ? fixed_time_bits(a.t[0], a.t[a.nobs - 1]) : 0;
+      if (blockIdx.x == 0) *a.time_bits = s_bits;
+    }
   }
   __syncthreads();
   const double df = s_df;
   float tmax = 0.f;
-  const bool grid_ok = isfinite(f0) && isfinite(df);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.nobs; i += stride) {
     const double s = a.sigma[i], x = a.x[i], t = a.t[i];
     const bool ok = isfinite(s) && isfinite(x) && isfinite(t) && s > 0.0;
     const double w = ok ? 1.0 / (s * s) : 0.0;
     const double xa = ok ? x * w : 0.0;
     if (ok) tmax = fmaxf(tmax, __double2float_ru(fabs(t)));
+    bool fits = true;
     if (a.rec) {
-      unsigned long long p = 0ull, d = 0ull;
-      unsigned dl = 0u;
-      if (ok && isfinite(f0) && isfinite(df)) {
-        phase_fixed96(t, df, d, dl);
-        if (dl != 0u) ++d;
-        p = phase_fixed64(t, f0) - d;
-      }
-      a.rec[i] = make_ulonglong2(p, d);
-      a.rec_low[i] = make_uint2(dl, __float_as_uint((float)t));
+      unsigned long long p = 0ull;
+      unsigned top = 0u;
+      const bool phases = ok && isfinite(df);
+      if (phases) fits = fixed_time(t, s_bits, p, top);
+      a.rec[i] = make_ulonglong2(p, phases ? phase_fixed64(t, df) : 0ull);
+      a.rec_top[i] = top;
     }
     if (a.aw == nullptr) {
     } else if (a.accum == FPW_ACCUM_FP64) {
@@ -72,9 +75,11 @@ __global__ void prep_kernel(const PrepArgs a) {
     } else {
       reinterpret_cast<float2*>(a.aw)[i] = make_float2((float)xa, (float)w);
     }
-    if (!ok || !(w > 0x1p-60 && w < 0x1p+60)) {
+    const bool wide = !(w > 0x1p-60 && w < 0x1p+60);
+    if (!ok || wide || !fits) {
       const int64_t c = a.offsets ? curve_of(a.offsets, a.ncurves, i) : 0;
-      atomicOr(reinterpret_cast<unsigned*>(a.curve_bad) + (c >> 2), (ok ? kCurveWide : kCurveBad) << (8 * (c & 3)));
+      const unsigned flags = ok ? (wide ? kCurveWide : 0u) | (fits ? 0u : kCurveUnfit) : kCurveBad;
+      atomicOr(reinterpret_cast<unsigned*>(a.curve_bad) + (c >> 2), flags << (8 * (c & 3)));
       if (!ok) report(a, kStatusData);
     }
   }
@@ -88,10 +93,8 @@ __global__ void prep_kernel(const PrepArgs a) {
     if ((threadIdx.x & 31) == 0 && m > *(volatile unsigned*)(a.grid_dev + 1)) atomicMax(a.grid_dev + 1, m);
   }
   // per anchor block: the largest deviation of its frequencies (and one more on
-  // either side) from the line through its anchor with the mean spacing, and the
-  // anchor's own distance from the line through f_0 (exact to about 2^-50 of the
-  // frequencies' rounding errors, which it is made of). From the last block of
-  // threads on: the first ones have the observations.
+  // either side) from the line through its anchor with the mean spacing. From the
+  // last block of threads on: the first ones have the observations.
   __shared__ unsigned wd[8];
   const int64_t A = a.anchor_span, blocks = (a.nfreq + A - 1) / A;
   for (int64_t q = gridDim.x - 1 - blockIdx.x; q < blocks; q += gridDim.x) {
@@ -111,13 +114,7 @@ __global__ void prep_kernel(const PrepArgs a) {
       if (threadIdx.x == 0) {
         a.block_dev[q] = __uint_as_float(d);
         if (d > *(volatile unsigned*)a.grid_dev) atomicMax(a.grid_dev, d);
-        const double pr = __dmul_rn((double)an, df), pe = __fma_rn((double)an, df, -pr);  // an df = pr + pe
-        const double sm = __dadd_rn(pr, f0), bb = __dsub_rn(sm, pr);                        // pr + f0 = sm + se
-        const double se = __dadd_rn(__dsub_rn(pr, __dsub_rn(sm, bb)), __dsub_rn(f0, bb));
-        const float delta = (float)((__dsub_rn(fa, sm) - (pe + se)) * 0x1p96);
-        a.block_delta[q] = delta;
-        const unsigned far = __float_as_uint(fabsf(delta));
-        if (far > *(volatile unsigned*)(a.grid_dev + 2)) atomicMax(a.grid_dev + 2, far);
+        if (!fixed_anchor(fa, s_bits).ok) a.grid_dev[2] = 1u;
       }
     }
   }

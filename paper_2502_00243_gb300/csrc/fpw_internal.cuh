@@ -24,8 +24,9 @@ constexpr double kGridTolCycles = 2e-10;
 // Largest number of derived bin counts computed from one M_max pass.
 constexpr int kMaxGroups = 8;
 
-// Per-curve flags (curve_bad): invalid data; a weight outside [2^-60, 2^60].
-constexpr unsigned kCurveBad = 1u, kCurveWide = 2u;
+// Per-curve flags (curve_bad): invalid data; a weight outside [2^-60, 2^60]; a
+// time that fixed_time does not hold.
+constexpr unsigned kCurveBad = 1u, kCurveWide = 2u, kCurveUnfit = 4u;
 
 // Several-M calls whose (M_max, groups) have a compiled combination in the
 // tile kernel (1: M_max = 60 with groups 3, 6, 15; 2: 40 with 2, 4, 10; 3: 20
@@ -59,11 +60,13 @@ struct TileArgs {
   int nitems;
   unsigned* counter;         // work-queue head (zeroed before launch)
   unsigned* status;          // latched status bits
-  const uint8_t* curve_bad;  // [ncurves] flags kCurveBad, kCurveWide
+  const uint8_t* curve_bad;  // [ncurves] flags kCurveBad, kCurveWide, kCurveUnfit
   unsigned long long* floors;  // [ncurves * max(ngroups, 1)] zeroed before launch, or NULL: the k-th best S that an
                              // item of the curve has found (its order-preserving bits)
   double* cand_S;            // [slots * k] candidate peaks (S), or NULL when k == 0
   int32_t* cand_idx;         // [slots * k]
+  ulonglong2* meetings;      // [slots] zeroed before launch: what items that meet inside an anchor block leave each
+                             // other, at the right one's slot; or NULL, no item begins inside a block
   double* S_out;             // dense [ncurves * nfreq] or NULL
   int M;
   int k;
@@ -72,16 +75,16 @@ struct TileArgs {
   double inv_alpha2;
   // Phase anchors: block q of the grid holds frequencies [q A, (q + 1) A), A =
   // anchor_span, and its phases step from the exact phase at frequency max(q A -
-  // 1, 0) (so they don't depend on how the kernel cuts its tiles).
+  // 1, 0). No tile reaches into another block: a phase depends on the observation
+  // and its frequency's block alone, not on the curves, output or launch around it.
   int64_t anchor_span;
-  int aligned;               // 1: no tile reaches into another block (dense output; no prep records)
-  const ulonglong2* rec;     // [nobs] {frac(t_i f_0) - D_i, D_i = frac(t_i df)} as 64-bit fixed point, rounded up
-                             // (prep), or NULL
-  const uint2* rec_low;      // [nobs] {D_i's next 32 bits before the rounding, t_i as FP32}
+  const ulonglong2* rec;     // [nobs] {low 64 bits of t_i (fixed_time), frac(t_i df) as 64-bit fixed point rounded
+                             // up} (prep), or NULL
+  const unsigned* rec_top;   // [nobs] top 32 bits of t_i
   const float* block_dev;    // [blocks] largest deviation of a block's frequencies from its line (prep), or NULL
-  const float* block_delta;  // [blocks] 2^96 (anchor frequency - (f_0 + a df)) (prep)
   const double* df;          // the grid's mean spacing (prep), or NULL
-  const unsigned* grid_dev;  // FP32 bits of the largest block_dev, |t| and |block_delta| (prep)
+  const unsigned* grid_dev;  // FP32 bits of the largest block_dev and |t|, 1 if fixed_anchor fails on some block (prep)
+  const int* time_bits;      // binary places of fixed_time (prep)
   int ngroups;               // several-M kernel: number of groups (0 = the single-M kernel)
   int group_g[kMaxGroups];   // M = M / group_g[q] for group q
   int64_t group_rows;        // candidate rows per group (cand tables are [group][slot][k])
@@ -103,13 +106,13 @@ struct PrepArgs {
   uint8_t* curve_bad;      // [ncurves] flags, zeroed before launch, 4-byte aligned and padded
   unsigned* status;
   unsigned* latch;         // NULL, or the word that keeps the status between calls
-  int64_t anchor_span;     // TileArgs, likewise the next five (rec NULL: none of them)
+  int64_t anchor_span;     // TileArgs, likewise the next six (rec NULL: none of them)
   ulonglong2* rec;
-  uint2* rec_low;
+  unsigned* rec_top;
   float* block_dev;
-  float* block_delta;
   double* df;              // NULL, or receives the grid's mean spacing
   unsigned* grid_dev;      // [3], zeroed before launch
+  int* time_bits;
 };
 
 struct MergeArgs {          // ngroups groups: rows of group g at + g * group_rows, its output at + g * k
@@ -256,28 +259,78 @@ __device__ __forceinline__ unsigned long long phase_fixed64(double t, double f) 
   return neg ? (0ull - r) : (r + (inexact ? 1ull : 0ull));
 }
 
-// The same to 96 bits (hi: the leading 64, lo: the next 32), rounded up at the last.
-__device__ __forceinline__ void phase_fixed96(double t, double f, unsigned long long& hi, unsigned& lo) {
-  unsigned long long mt, mf;
-  int et, ef;
-  split_binary64(t, mt, et);
-  split_binary64(f, mf, ef);
-  const unsigned __int128 q = (unsigned __int128)mt * mf;
-  const int s = et + ef + 96;  // frac * 2^96 = (q * 2^s) mod 2^96
-  unsigned __int128 r = 0;
-  bool inexact = false;
-  if (s >= 0) {
-    if (s < 128) r = q << s;
-  } else if (s > -128) {
-    r = q >> -s;
-    inexact = (r << -s) != q;
-  } else {
-    inexact = q != 0;
+// A time as a 96-bit integer, 2^95 - t 2^L (low 64 bits, top 32), where t 2^L is
+// an integer below 2^94 in size: its product with an anchor frequency's significand
+// then takes six 32-bit multiplications and one shift that is the same for all
+// times (FixedAnchor), where phase_fixed64 takes both numbers apart and shifts
+// by their exponents (about 60 instructions). Negated, so that rounding the
+// product down rounds the phase up. Returns whether t is such a time.
+__device__ __forceinline__ bool fixed_time(double t, int L, unsigned long long& low, unsigned& top) {
+  unsigned long long m;
+  int e;
+  split_binary64(t, m, e);
+  e += L;
+  if (m == 0ull) e = 0;
+  low = 0ull;
+  top = 0u;
+  if (e < 0) {
+    if (e < -52 || (m & ((1ull << -e) - 1ull)) != 0ull) return false;
+    m >>= -e;
+    e = 0;
   }
-  const bool neg = ((__double_as_longlong(t) ^ __double_as_longlong(f)) < 0) && q != 0;
-  r = neg ? -r : r + (inexact ? 1u : 0u);
-  hi = (unsigned long long)(r >> 32);
-  lo = (unsigned)r;
+  if (e > 41) return false;  // m < 2^53
+  const unsigned __int128 v = (unsigned __int128)m << e, off = (unsigned __int128)1 << 95;
+  const unsigned __int128 r = __double_as_longlong(t) < 0 ? off + v : off - v;
+  low = (unsigned long long)r;
+  top = (unsigned)(r >> 64);
+  return true;
+}
+// L for a call: its first and last times (the largest, as times come) fit with two bits to spare.
+__device__ __forceinline__ int fixed_time_bits(double t_first, double t_last) {
+  int e = -1023;
+  for (double t : {t_first, t_last}) {
+    const int b = (int)(((unsigned long long)__double_as_longlong(t) >> 52) & 0x7ffull) - 1023;
+    if (b < 1024 && b > e) e = b;
+  }
+  e = e < -64 ? -64 : (e > 64 ? 64 : e);
+  return 91 - e;
+}
+
+// An anchor frequency for times of L binary places: f = F 2^-K, F < 2^64, with
+// 128 <= L + K < 160, so that a product's 64 bits below the binary point are its
+// bits 64 + sh ... 127 + sh.
+struct FixedAnchor {
+  unsigned long long F, off;  // off: 2^95 F in those bits
+  int sh;
+  bool ok;                    // f >= 0 and in reach of the shift
+};
+__device__ __forceinline__ FixedAnchor fixed_anchor(double f, int L) {
+  unsigned long long m;
+  int e;
+  split_binary64(f, m, e);
+  int g = 128 - (L - e);
+  g = g < 0 ? 0 : (g > 11 ? 11 : g);
+  FixedAnchor r;
+  r.sh = L - e + g - 128;
+  r.F = m << g;
+  r.ok = __double_as_longlong(f) >= 0 && r.sh >= 0 && r.sh < 32;
+  if (m == 0ull) r.sh = 0;
+  r.ok = r.ok || m == 0ull;
+  r.off = r.F << ((31 - r.sh) & 31);
+  return r;
+}
+// phase_fixed64(t, f) from both.
+__device__ __forceinline__ unsigned long long fixed_phase(unsigned long long low, unsigned top, const FixedAnchor& a) {
+  const unsigned t0 = (unsigned)low, t1 = (unsigned)(low >> 32), f0 = (unsigned)a.F, f1 = (unsigned)(a.F >> 32);
+  const unsigned long long p00 = (unsigned long long)t0 * f0, p10 = (unsigned long long)t1 * f0,
+                           p01 = (unsigned long long)t0 * f1, p20 = (unsigned long long)top * f0,
+                           p11 = (unsigned long long)t1 * f1, p21 = (unsigned long long)top * f1;
+  const unsigned long long w1 = (p00 >> 32) + (unsigned)p10 + (unsigned)p01;
+  const unsigned long long w2 = (p10 >> 32) + (p01 >> 32) + (unsigned)p20 + (unsigned)p11 + (w1 >> 32);
+  const unsigned long long w3 = p21 + (p20 >> 32) + (p11 >> 32) + (w2 >> 32);
+  const unsigned lo = __funnelshift_r((unsigned)w2, (unsigned)w3, a.sh);
+  const unsigned hi = __funnelshift_r((unsigned)w3, (unsigned)(w3 >> 32), a.sh);
+  return a.off - (((unsigned long long)hi << 32) | lo);
 }
 
 // Bin of a 64-bit fixed-point phase: floor(M * Phi_hi / 2^32). It equals

@@ -266,7 +266,6 @@ extern "C" FPW_API int fpw_periodogram_batch_noalloc(void* stream, const fpw_par
   ta.peak_raw = p.peak_mode == FPW_PEAK_RAW ? 1 : 0;
   ta.K = p.K;
   ta.anchor_span = A;
-  ta.aligned = 1;
   ta.inv_alpha2 = p.inv_alpha2;
   int64_t grid = (int64_t)bps * ds->nsm;
   if (grid * warps > ta.nitems) grid = (ta.nitems + warps - 1) / warps;

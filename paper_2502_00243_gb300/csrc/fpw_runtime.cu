@@ -92,6 +92,7 @@ struct Plan {
   int nitems = 0;
   int nslots = 0;
   int max_rows = 0;  // most candidate rows (work items) of one curve
+  bool meetings = false;  // some item begins inside an anchor block
   DevBuf items;                    // work items, then the candidate rows per curve
   int32_t* cand_base = nullptr;
   void* host_stage = nullptr;  // pinned copy of items + cand_base, the source of the asynchronous upload
@@ -115,10 +116,9 @@ struct GraphEntry {
 // Status words of a context (64 bytes): 1 the status of the current call (plain,
 // shared-timestamp and drift paths), kWordLatch the latched status (kept between
 // calls), 8-9 the shared-timestamp path's max |t|. The tile path's words precede
-// its per-curve flags: 0 work-queue head, 1 status, 2-4 the grid's largest
-// deviation from a line, the largest |t| and the largest distance of an anchor
-// from the line (FP32 bits), 6-7 the grid's mean spacing (binary64).
-constexpr int kCallWords = 8, kWordGridDev = 2, kWordDf = 6;
+// its per-curve flags: 0 work-queue head, 1 status, 2-4 TileArgs::grid_dev, 5 the
+// binary places of the fixed-point times, 6-7 the grid's mean spacing (binary64).
+constexpr int kCallWords = 8, kWordGridDev = 2, kWordTimeBits = 5, kWordDf = 6;
 
 constexpr int kMaxPlans = 16;
 constexpr int kMaxGraphs = 16;
@@ -213,8 +213,9 @@ double shape_time(const fpw_ctx* ctx, int R, int w, int64_t tiles, bool wide) {
 // the context's tuned table (fpw_ctx_set_shape) > the bin count: they place the
 // phase anchors (every T R - 2 frequencies), so results don't move when the
 // launch below changes. Then what is launched, in blocks of `warps` warps with
-// `lane_R` frequencies per lane, each warp with tiles of its own: T / 32 and R
-// where the caller or the table gave them; else R as measured per bin count (a
+// `lane_R` frequencies per lane, each warp with tiles of its own that fill an
+// anchor block evenly (32 lane_R divides T R): T / 32 and R where the caller or
+// the table gave them; else R as measured per bin count (a
 // warp's bins take R*M*32*(8|16) bytes, 16 for binary64 and compensated sums) and
 // the warps that fit one block per SM, up to 8 (two per scheduler; 16-byte bins:
 // 12), N = 1000: M = 20 R = 5 2.05e12 evaluations/s (R = 10 on 4 warps 2.02), M =
@@ -224,7 +225,7 @@ double shape_time(const fpw_ctx* ctx, int R, int w, int64_t tiles, bool wide) {
 // 1.24 (R = 3 on 4 1.05), compensated M = 20 R = 2 on 10 0.90 (R = 3 on 7 0.91, R = 2 on
 // 8 0.87).
 int choose_shape(fpw_ctx* ctx, const fpw_params& p, int M, int k, int64_t C, int64_t F, int64_t max_n, int64_t n_mean,
-                 int64_t n_typ, int ngroups, const int* groups, bool dense, TileShape& out) {
+                 int64_t n_typ, int ngroups, const int* groups, TileShape& out) {
   const bool wide = p.accum != FPW_ACCUM_FP32, multi = ngroups > 0;
   int T = 128, R = 4, NC = 0, items = 8;
   if (wide)
@@ -282,13 +283,12 @@ int choose_shape(fpw_ctx* ctx, const fpw_params& p, int M, int k, int64_t C, int
     r = wide ? 2 : M <= 12 ? 8 : M <= 16 && !multi ? 6 : M <= 20 ? 5 : M <= 25 ? 4 : M <= 33 ? 3 : M <= 50 ? 2 : M <= 64 ? 3 : 1;
     if (multi && M > 50 && M <= 64) r = 2;
     w = wide ? 12 : 8;
+    const auto even = [&](int q) { return T * R % (32 * q) == 0; };
     while (r > 1 && fit(r) < 4) --r;
-    if (r == 7 || (multi && r == 6)) --r;
-    w = std::min(w, fit(r));
     // The shape that is estimated to finish first: for one curve, whose tiles all
     // take the same time, by rounds of tiles; else by the work and half a tile of
-    // the longest curve at the end (R only below the measured one). A shape that
-    // cuts an anchor block evenly, with a compiled combination if the call has one.
+    // the longest curve at the end (R only below the measured one). With a
+    // compiled combination if the call has one.
     const int spec = multi ? multi_spec_of(M, ngroups, groups) : 0;
     const auto estimate = [&](int q, int v) {
       const int64_t tiles = C * warp_tiles(F, q);
@@ -296,11 +296,17 @@ int choose_shape(fpw_ctx* ctx, const fpw_params& p, int M, int k, int64_t C, int
       const double round = shape_time(ctx, q, v, (int64_t)ctx->nsm * v, wide);
       return round * ((double)tiles / ((double)ctx->nsm * v) + 0.5 * (double)(max_n + 64) / (double)(n_mean + 64));
     };
+    if (!even(r)) {  // the next that fills a block, below or (with six warps a SM) above
+      int up = r;
+      while (up < 9 && !even(up)) ++up;
+      while (!even(r)) --r;
+      if (up < 9 && fit(up) >= 6 && estimate(up, std::min(w, fit(up))) < estimate(r, std::min(w, fit(r)))) r = up;
+    }
+    w = std::min(w, fit(r));
     double best = estimate(r, w);
     const int r0 = r;
     for (int q : {8, 6, 5, 4, 3, 2, 1}) {
-      if (q > (C == 1 ? (wide ? 4 : 8) : r0) || (q == 6 && multi) || (q == 3 && p.accum == FPW_ACCUM_FP64)) continue;
-      if ((dense && T * R % (32 * q) != 0) || (spec && q != 2 && !(spec == 3 && q == 5))) continue;
+      if (q > (C == 1 ? (wide ? 4 : 8) : r0) || !even(q) || (spec && q != 2 && !(spec == 3 && q == 4))) continue;
       for (int v : {4, 7, 8, 12}) {
         if (v > fit(q) || v > tile_max_warps(multi) || (C > 1 && v < 8)) continue;
         const double t = estimate(q, v);
@@ -329,12 +335,12 @@ int choose_shape(fpw_ctx* ctx, const fpw_params& p, int M, int k, int64_t C, int
 // the items shrink towards the end of the list and the warps finish together (a
 // fixed size left 2-10 % of the time to the last items); never less than a
 // tile, nor than 1 / (4 * items) of a warp's share. Cuts lie between anchor
-// blocks where an item holds one at least. halo: frequencies an item evaluates
-// beyond each end of its range (1 when peaks are asked for). aligned: tiles stay
-// inside anchor blocks. Candidate rows per curve in curve order. The tables are
-// uploaded from a pinned copy, ordered on `st`.
+// blocks where an item holds one at least, else between tiles of a block. halo:
+// frequencies evaluated beyond each end of a block (1 when peaks are asked for).
+// Candidate rows per curve in curve order. The tables are uploaded from a pinned
+// copy, ordered on `st`.
 Plan* build_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const TileShape& sh, int blocks_per_sm,
-                 int halo, bool aligned, uint64_t key, cudaStream_t st, int* err) {
+                 int halo, uint64_t key, cudaStream_t st, int* err) {
   *err = FPW_OK;
   const int64_t W = 32 * (int64_t)sh.lane_R, A = (int64_t)sh.threads * sh.R - 2;
   const int64_t B = (A + 2 * halo + W - 1) / W;  // tiles of an anchor block
@@ -353,6 +359,7 @@ Plan* build_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const T
   std::vector<WorkItem> sorted;  // the shares shrink as the list grows
   sorted.reserve((size_t)C + (size_t)(resident * sh.items));
   std::vector<int32_t> base((size_t)C + 1, 0);
+  bool meetings = false;
   for (const int64_t c : order) {
     const double cc = cost(c);
     int64_t lo = 0;
@@ -361,9 +368,9 @@ Plan* build_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const T
       const double share = std::max(left / (1.5 * (double)resident), least);
       const int64_t rest = (F - lo + 2 * halo + W - 1) / W;  // tiles to the end in one item
       const int64_t n = std::max<int64_t>(1, (int64_t)(share / cc));
-      int64_t hi = n >= B ? (lo / A + n / B) * A : lo + n * W - 2 * halo;
-      if (n < B && aligned) hi = std::min(hi, (lo / A + 1) * A);
-      if (n + n / 4 >= rest && (!aligned || n >= B)) hi = F;
+      const int64_t q = lo / A;
+      int64_t hi = n >= B ? (q + n / B) * A : std::min(lo - (lo == q * A ? halo : 0) + n * W, (q + 1) * A);
+      if (n + n / 4 >= rest && n >= B) hi = F;
       hi = std::min(hi, F);
       const double work = cc * (double)((hi - lo + 2 * halo + W - 1) / W);
       WorkItem w;
@@ -371,6 +378,7 @@ Plan* build_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const T
       w.f_lo = (int32_t)lo;
       w.f_hi = (int32_t)hi;
       w.slot = rows++;
+      meetings = meetings || (halo != 0 && lo != q * A);
       sorted.push_back(w);
       left = std::max(0.0, left - work);
       lo = hi;
@@ -388,6 +396,7 @@ Plan* build_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const T
   pl->key = key;
   pl->nitems = (int)sorted.size();
   pl->nslots = base[C];
+  pl->meetings = meetings;
   for (int64_t c = 0; c < C; ++c) pl->max_rows = std::max(pl->max_rows, base[c + 1] - base[c]);
   pl->grid = (int)std::max<int64_t>(1, (std::min<int64_t>(resident, pl->nitems) + sh.warps - 1) / sh.warps);
   const size_t ib = sorted.size() * sizeof(WorkItem), bb = base.size() * sizeof(int32_t);
@@ -408,7 +417,7 @@ Plan* build_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const T
 }
 
 Plan* get_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const TileShape& sh, int blocks_per_sm,
-               int halo, bool aligned, cudaStream_t st, int* err) {
+               int halo, cudaStream_t st, int* err) {
   uint64_t key = fnv1a(off, sizeof(int64_t) * (size_t)(C + 1));
   key = mix(key, C);
   key = mix(key, F);
@@ -419,7 +428,6 @@ Plan* get_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const Til
   key = mix(key, sh.items);
   key = mix(key, blocks_per_sm);
   key = mix(key, halo);
-  key = mix(key, aligned);
   key = mix(key, sh.warps);
   key = mix(key, sh.lane_R);
   for (Plan* p : ctx->plans)
@@ -428,7 +436,7 @@ Plan* get_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const Til
       *err = FPW_OK;
       return p;
     }
-  Plan* p = build_plan(ctx, off, C, F, sh, blocks_per_sm, halo, aligned, key, st, err);
+  Plan* p = build_plan(ctx, off, C, F, sh, blocks_per_sm, halo, key, st, err);
   if (!p) return nullptr;
   p->use = ++ctx->tick;
   if ((int)ctx->plans.size() >= kMaxPlans) {
@@ -480,11 +488,11 @@ void drop_graphs(fpw_ctx* ctx) {
 // (first, cleared at once), the prep kernel's output per observation and per
 // anchor block, the candidate table.
 struct Scratch {
-  size_t floors, clear, aw, rec, low, dev, delta, cand_S, cand_idx, total;  // clear: bytes to clear, from the start
+  size_t floors, meetings, clear, aw, rec, top, dev, cand_S, cand_idx, total;  // clear: bytes to clear, from the start
 };
 Scratch scratch_layout(const BatchCall& b, const TileShape& sh, const Plan* pl) {
   const size_t nobs = (size_t)b.off_h[b.C], A = (size_t)sh.threads * sh.R - 2, blocks = ((size_t)b.F + A - 1) / A;
-  const size_t rows = (size_t)(b.ngroups > 0 ? b.ngroups : 1) * (size_t)pl->nslots * (size_t)b.k;
+  const size_t slots = (size_t)(b.ngroups > 0 ? b.ngroups : 1) * (size_t)pl->nslots, rows = slots * (size_t)b.k;
   size_t o = 0;
   const auto take = [&](size_t bytes) {
     const size_t at = o;
@@ -494,12 +502,12 @@ Scratch scratch_layout(const BatchCall& b, const TileShape& sh, const Plan* pl) 
   Scratch L;
   take(kCallWords * sizeof(unsigned) + (size_t)b.C);
   L.floors = take((b.k > 0 ? (size_t)b.C * (size_t)std::max(b.ngroups, 1) : 0) * sizeof(unsigned long long));
+  L.meetings = take(pl->meetings ? slots * sizeof(ulonglong2) : 0);
   L.clear = o;
   L.aw = take((nobs + 2) * accum_bin_bytes(b.p.accum));
   L.rec = take((nobs + 2) * sizeof(ulonglong2));
-  L.low = take((nobs + 2) * sizeof(uint2));
+  L.top = take((nobs + 2) * sizeof(unsigned));
   L.dev = take(blocks * sizeof(float));
-  L.delta = take(blocks * sizeof(float));
   L.cand_S = take(rows * sizeof(double));
   L.cand_idx = take(rows * sizeof(int32_t));
   L.total = o;
@@ -530,12 +538,12 @@ int enqueue_tile_path(fpw_ctx* ctx, const BatchCall& b, const TileShape& sh, Pla
   pa.status = call + 1;
   pa.latch = static_cast<unsigned*>(ctx->words.p) + kWordLatch;
   pa.rec = reinterpret_cast<ulonglong2*>(scratch + L.rec);
-  pa.rec_low = reinterpret_cast<uint2*>(scratch + L.low);
+  pa.rec_top = reinterpret_cast<unsigned*>(scratch + L.top);
   pa.anchor_span = (int64_t)sh.threads * sh.R - 2;
   pa.block_dev = reinterpret_cast<float*>(scratch + L.dev);
-  pa.block_delta = reinterpret_cast<float*>(scratch + L.delta);
   pa.df = reinterpret_cast<double*>(call + kWordDf);
   pa.grid_dev = call + kWordGridDev;
+  pa.time_bits = reinterpret_cast<int*>(call + kWordTimeBits);
   FPW_CK(launch_prep(pa, st));
   TileArgs ta{};
   ta.t = b.t;
@@ -552,6 +560,7 @@ int enqueue_tile_path(fpw_ctx* ctx, const BatchCall& b, const TileShape& sh, Pla
   ta.floors = b.k > 0 ? reinterpret_cast<unsigned long long*>(scratch + L.floors) : nullptr;
   ta.cand_S = b.k > 0 ? reinterpret_cast<double*>(scratch + L.cand_S) : nullptr;
   ta.cand_idx = b.k > 0 ? reinterpret_cast<int32_t*>(scratch + L.cand_idx) : nullptr;
+  ta.meetings = reinterpret_cast<ulonglong2*>(scratch + L.meetings);
   ta.S_out = b.S_out;
   ta.M = b.M;
   ta.k = b.k;
@@ -559,13 +568,12 @@ int enqueue_tile_path(fpw_ctx* ctx, const BatchCall& b, const TileShape& sh, Pla
   ta.K = b.p.K;
   ta.inv_alpha2 = b.p.inv_alpha2;
   ta.rec = pa.rec;
-  ta.rec_low = pa.rec_low;
+  ta.rec_top = pa.rec_top;
   ta.anchor_span = pa.anchor_span;
-  ta.aligned = b.S_out || b.bins_out ? 1 : 0;
   ta.block_dev = pa.block_dev;
-  ta.block_delta = pa.block_delta;
   ta.df = pa.df;
   ta.grid_dev = pa.grid_dev;
+  ta.time_bits = pa.time_bits;
   ta.ngroups = b.ngroups;
   for (int q = 0; q < b.ngroups; ++q) ta.group_g[q] = b.groups[q];
   ta.group_rows = pl->nslots;
@@ -620,12 +628,12 @@ int run_tile_path(fpw_ctx* ctx, const BatchCall& b) {
   const int64_t n_typ = sn > 0.0 ? (int64_t)(sn2 / sn) : 0;  // observation-weighted mean curve size
   TileShape sh{};
   int rc = choose_shape(ctx, b.p, b.M, b.k, b.C, b.F, max_n, (int64_t)(sn / (double)b.C), n_typ, b.ngroups, b.groups,
-                        b.S_out || b.bins_out, sh);
+                        sh);
   if (rc != FPW_OK) return rc;
   const int bps = tile_max_blocks_per_sm(sh.lane_R, b.p.phase_mode, b.p.accum, 32 * sh.warps, sh.smem, b.ngroups > 0,
                                          b.bins_out != nullptr, multi_spec_of(b.M, b.ngroups, b.groups));
   if (bps < 1) return FPW_ENOTSUP;
-  Plan* pl = get_plan(ctx, b.off_h, b.C, b.F, sh, bps, b.k > 0 ? 1 : 0, b.S_out || b.bins_out, b.stream, &rc);
+  Plan* pl = get_plan(ctx, b.off_h, b.C, b.F, sh, bps, b.k > 0 ? 1 : 0, b.stream, &rc);
   if (!pl) return rc;
   ctx->last_shape = sh;
   ctx->last_grid = pl->grid;

@@ -15,20 +15,22 @@
 //   the other warps' bin updates. (A block per item, its four warps meeting at
 //   barriers around every chunk and tile, ran the same loop at 1.93e12
 //   evaluations/s where warps of their own run 2.05e12, M = 20, N = 1000.)
-//   An item computes S at f_lo - 1 .. f_hi: both neighbours of every owned
-//   frequency (the local-maximum test needs them); tiles do not overlap inside
-//   an item, the last two values of a tile are carried to the next.
+//   Phases are anchored every anchor_span frequencies, and a tile lies in one
+//   anchor block, whose frequencies with one more on either side (the
+//   local-maximum test needs both neighbours) are a whole number of tiles. Tiles
+//   do not overlap, the last two values of a tile are carried to the next; items
+//   that meet inside a block leave each other the values at their ends (Meeting).
 //
 // Per tile
 //   1. Stage (per 32 observations, lane = observation, a ring of two chunks in
 //      shared memory, the next chunk's inputs already in registers): the phase
 //      Phi_s = frac(t_i * f_s) at the tile's first frequency as a 64-bit
 //      fixed-point fraction, the step D_i = frac(t_i * df) (df = grid spacing) and
-//      the weights (a_i = x_i w_i, w_i). Where the whole grid lies on its line,
-//      Phi_s takes a few integer operations from the prep kernel's records (60
-//      operations an observation and tile for the exact product held up the hot
-//      loops for 5-10 % of the time); else it is the exact integer product of the
-//      binary64 significands.
+//      the weights (a_i = x_i w_i, w_i). Phi_s steps from the exact phase at the
+//      block's anchor frequency, the integer product of the significands, for
+//      which the prep kernel leaves the times as fixed-point numbers (about 20
+//      operations an observation and tile; 60 with both numbers taken apart held
+//      up the hot loops for 5-10 % of the time).
 //   2. Hot loop (per observation, per lane, per r): Phi = Phi_s + (l R + r) D_i
 //      (mod 2^64), bin m = floor(M * Phi_hi / 2^32), A_m += a_i, B_m += w_i in a
 //      lane-private [r][m][lane] bin array in shared memory (bank = lane, so
@@ -278,6 +280,7 @@ struct Warp {
   int lane, M, kk;
   int64_t F;
   double df;
+  int tbits;                 // binary places of the prep kernel's times
   static constexpr unsigned kBinStride = 32u * (unsigned)sizeof(typename P::Bin);  // bytes between bins of a column
 };
 
@@ -296,6 +299,7 @@ __device__ __forceinline__ Warp<P> make_warp(unsigned char* smem, const TileArgs
   w.topI = reinterpret_cast<int*>(mine + L.topI);
   w.F = args.nfreq;
   w.df = args.df ? *args.df : (w.F > 1) ? (args.freqs[w.F - 1] - args.freqs[0]) / (double)(w.F - 1) : 0.0;
+  w.tbits = args.rec ? *args.time_bits : 0;
   // bins start at zero (every reduce leaves them zero again), and so does the
   // ring (the prefetch past a curve's last observation reads slots not staged)
   for (int q = 0; q < R * w.M; ++q)
@@ -322,12 +326,12 @@ __device__ __forceinline__ int exponent_of(double v) {  // floor(log2 |v|) for n
   return (int)(((unsigned long long)__double_as_longlong(v) >> 52) & 0x7ffull) - 1023;
 }
 
-// How a tile's phases are formed: stepped from the first frequency on (the whole
-// grid on its line, no dense output); stepped from the exact phase at the anchor
-// of the tile's block (the block on a line), which kRecord derives from the prep
-// kernel's records and kAnchor from the product; products with the distance from
-// an exact phase (NlTile); the exact phase of every pair.
-enum TileMode { kLine, kRecord, kAnchor, kFixed, kExact };
+// How a tile's phases are formed: stepped from the exact phase at the anchor of
+// the tile's block (the block on a line), which kRecord takes from the prep
+// kernel's fixed-point times and kAnchor from the general product (the same
+// number, where a time or the anchor is not of that form); products with the distance from an exact phase (NlTile); the exact
+// phase of every pair.
+enum TileMode { kRecord, kAnchor, kFixed, kExact };
 
 // The frequencies of a tile off the linear grid, as FP32 pairs of f_k - f_b (f_b:
 // the tile's middle frequency). An observation's phase at f_k is its exact phase
@@ -361,43 +365,27 @@ __device__ __forceinline__ unsigned nl_phase(const ulonglong2& pd, float dh, flo
 }
 
 // Geometry of one tile: first frequency s (-1 possible), its anchor block's first
-// position sq and anchor frequency fa (index max(sq, 0)), how its phases are
-// formed, and (kRecord) the anchor's index and distance from the line through f_0.
+// position sq and anchor frequency fa (index max(sq, 0)), and how its phases are
+// formed.
 struct Tile {
   int64_t s, sq;
   double fa;
   TileMode mode;
-  unsigned a;
-  float delta;
 };
 
-// The tile at s. aligned: it lies in block q, whose block_delta is `delta`.
+// The tile at s in anchor block q.
 template <int R, class P>
-__device__ __forceinline__ Tile make_tile(const TileArgs& args, const Warp<P>& w, int64_t s, int64_t q, float delta,
-                                          double tm, bool every_lin, bool aligned, NlTile<R>& nl) {
+__device__ __forceinline__ Tile make_tile(const TileArgs& args, const Warp<P>& w, int64_t s, int64_t q, double tm,
+                                          bool every_lin, bool unfit, NlTile<R>& nl) {
   Tile g;
-  bool inside = true;  // one block's line serves the whole tile
-  if (!aligned && !every_lin) {
-    const unsigned k = s < 0 ? 0u : (unsigned)(s < w.F ? s : w.F - 1), A = (unsigned)args.anchor_span;
-    q = k / A;
-    delta = args.block_delta[q];
-    inside = s + 32 * R - 1 <= (q + 1) * (int64_t)A;
-  }
   g.s = s;
   g.sq = q * args.anchor_span - 1;
   const int64_t a = g.sq < 0 ? 0 : g.sq;
-  g.a = (unsigned)a;
-  g.delta = delta;
-  g.fa = 0.0;
-  g.mode = aligned ? kRecord : kLine;
-  if (every_lin) return g;
   g.fa = args.freqs[a];
-  bool lin, rec = false;
-  if (!inside) {
-    lin = false;
+  bool lin = every_lin;
+  if (every_lin) {
   } else if (args.block_dev) {
     lin = (double)args.block_dev[q] * tm <= kGridTolCycles;
-    rec = fabs((double)delta * 0x1p-32) * tm < 0x1p30;
   } else {
     bool off = false;
     for (int64_t j = w.lane; j < args.anchor_span + 2; j += 32) {
@@ -407,7 +395,7 @@ __device__ __forceinline__ Tile make_tile(const TileArgs& args, const Warp<P>& w
     lin = !__any_sync(0xffffffffu, off);
   }
   if (lin) {
-    g.mode = rec ? kRecord : kAnchor;
+    g.mode = args.rec && !unfit && (every_lin || fixed_anchor(g.fa, w.tbits).ok) ? kRecord : kAnchor;
     return g;
   }
   const int64_t s0 = s < 0 ? 0 : (s < w.F ? s : w.F - 1), mid = s + 16 * R;
@@ -440,8 +428,8 @@ __device__ __forceinline__ Tile make_tile(const TileArgs& args, const Warp<P>& w
 // One observation's inputs on their way from global memory to the ring.
 template <class P>
 struct Obs {
-  ulonglong2 rec;  // the prep kernel's record (kLine, kRecord), {t, 0} else
-  uint2 low;       // kRecord: what goes with it
+  ulonglong2 rec;  // the prep kernel's record (kRecord), {t, 0} else
+  unsigned top;    // kRecord: the time's top word
   typename P::In aw;
 };
 
@@ -449,12 +437,12 @@ template <class P>
 __device__ __forceinline__ Obs<P> fetch(const TileArgs& args, TileMode mode, int64_t base, int64_t n, int64_t i) {
   Obs<P> o;
   o.rec = make_ulonglong2(0ull, 0ull);  // past the curve's end: t = 0 and zero weights, which add 0 to some bin
-  o.low = make_uint2(0u, 0u);
+  o.top = 0u;
   bin_zero(o.aw);
   if (i < n) {
-    if (mode == kLine || mode == kRecord) {
+    if (mode == kRecord) {
       o.rec = args.rec[base + i];
-      if (mode == kRecord) o.low = args.rec_low[base + i];
+      o.top = args.rec_top[base + i];
     } else {
       o.rec.x = (unsigned long long)__double_as_longlong(args.t[base + i]);
     }
@@ -464,29 +452,19 @@ __device__ __forceinline__ Obs<P> fetch(const TileArgs& args, TileMode mode, int
 }
 
 // The staged phase record: {phase, step D}, {P, T} (NlTile) or {t, 0}. The phase is
-// that of frequency -1 as the prep kernel left it (kLine: the hot loop takes s + 1
-// + j steps from it), else that of the tile's first frequency: the exact phase at
-// the block's anchor, rounded up at 2^-64, plus s - sq steps. kRecord takes the
-// anchor's from P_0 + a D with 96 bits of D (the 64-bit step's rounding adds up to
-// a 2^-64 = 10^-15 cycles, and visits a round fraction of a day apart put phases
-// that close to bin edges) plus t times the anchor frequency's distance from the
-// line (FP32 of a term below 2^-33 cycles), a fifth of the operations of the
-// product. With Df = D rounded down, a + (s - sq) = s (+ the anchor's step back in
-// block 0).
+// that of the tile's first frequency: the exact phase at the block's anchor,
+// rounded up at 2^-64, plus s - sq steps (one less in block 0, which starts one
+// step before its anchor). Nothing shorter than the exact anchor will do: visits
+// a round fraction of a day apart put phases within 10^-15 cycles of bin edges at
+// round frequencies, where a step rounded once and summed over the grid, or an
+// anchor to 2^-54, moves observations to other bins.
 template <class P>
 __device__ __forceinline__ ulonglong2 record(const TileArgs& args, const Warp<P>& w, const Tile& g, TileMode mode,
-                                             const Obs<P>& o) {
-  if (mode == kLine || mode == kExact) return o.rec;
+                                             const FixedAnchor& anchor, const Obs<P>& o) {
+  if (mode == kExact) return o.rec;
+  const unsigned long long steps = (unsigned long long)(g.s - g.sq - (g.sq < 0 ? 1 : 0));
   if (mode == kRecord) {
-    const float v = __uint_as_float(o.low.y) * g.delta;  // three FP32 roundings, made up for in the next line
-    const unsigned long long low =
-        (unsigned long long)g.a * o.low.x + (unsigned long long)__float2ll_rn(__fmaf_rn(fabsf(v), 0x1p-21f, v));
-    const unsigned up = o.low.x != 0u ? 1u : 0u;  // D is rounded up
-    // the low words' carry, the rounding up, and the steps of D not of Df
-    const int more = (int)(low >> 32) + ((unsigned)low != 0u ? 1 : 0) +
-                     (up ? (int)(g.s - g.sq) - (g.sq < 0 ? 1 : 0) : 0);
-    const unsigned long long D = o.rec.y, Df = D - up;
-    return make_ulonglong2(o.rec.x + D + (unsigned long long)(long long)g.s * Df + (unsigned long long)(long long)more, D);
+    return make_ulonglong2(fixed_phase(o.rec.x, o.top, anchor) + steps * o.rec.y, o.rec.y);
   }
   const double t = __longlong_as_double((long long)o.rec.x);
   unsigned long long Pa = phase_fixed64(t, g.fa);
@@ -498,8 +476,7 @@ __device__ __forceinline__ ulonglong2 record(const TileArgs& args, const Warp<P>
                            ((unsigned long long)__float_as_uint(tt.y) << 32) | __float_as_uint(tt.x));
   }
   const unsigned long long D = phase_fixed64(t, w.df);
-  if (g.sq < 0) Pa -= D;  // block 0 starts one step before its anchor
-  return make_ulonglong2(Pa + (unsigned long long)(g.s - g.sq) * D, D);
+  return make_ulonglong2(Pa + steps * D, D);
 }
 
 // Chunk c of 32 observations into its half of the ring.
@@ -528,7 +505,7 @@ __device__ __forceinline__ void accumulate(const TileArgs& args, const Warp<P>& 
   using In = typename P::In;
   constexpr int U = 4, kChunk = 32;
   const unsigned M = (unsigned)w.M;
-  const unsigned j0 = (unsigned)w.lane * R + (MODE == kLine ? (unsigned)(g.s + 1) : 0u);
+  const unsigned j0 = (unsigned)w.lane * R;
   const unsigned col = smem_u32(w.bins), rstride = M * Warp<P>::kBinStride;
   const int64_t npad = (n + U - 1) / U * U, nchunk = (n + kChunk - 1) / kChunk;
   const auto addresses = [&](const ulonglong2& p, unsigned (&ad)[R]) {
@@ -545,9 +522,10 @@ __device__ __forceinline__ void accumulate(const TileArgs& args, const Warp<P>& 
   };
   Obs<P> o = fetch<P>(args, mode, base, n, w.lane);
   const Obs<P> o1 = fetch<P>(args, mode, base, n, 32 + w.lane);
+  const FixedAnchor anchor = fixed_anchor(g.fa, w.tbits);  // (after the loads: it waits for its own)
   __syncwarp();  // every lane is done with the previous tile's ring
-  put<P>(w, 0, record<P>(args, w, g, mode, o), o.aw);
-  put<P>(w, 1, record<P>(args, w, g, mode, o1), o1.aw);
+  put<P>(w, 0, record<P>(args, w, g, mode, anchor, o), o.aw);
+  put<P>(w, 1, record<P>(args, w, g, mode, anchor, o1), o1.aw);
   o = fetch<P>(args, mode, base, n, 64 + w.lane);
   __syncwarp();
   const unsigned pd0 = smem_u32(w.pd), aw0 = smem_u32(w.aw);
@@ -590,7 +568,7 @@ __device__ __forceinline__ void accumulate(const TileArgs& args, const Warp<P>& 
     }
     if (c + 2 < nchunk) {  // this chunk's half of the ring is free: the next but one
       __syncwarp();
-      put<P>(w, c + 2, record<P>(args, w, g, mode, o), o.aw);
+      put<P>(w, c + 2, record<P>(args, w, g, mode, anchor, o), o.aw);
       o = fetch<P>(args, mode, base, n, (c + 3) * kChunk + w.lane);
       __syncwarp();
     }
@@ -606,12 +584,12 @@ __device__ __forceinline__ void accumulate_slow(const TileArgs& args, const Warp
   using Bin = typename P::Bin;
   using In = typename P::In;
   const unsigned M = (unsigned)w.M;
-  const int64_t j0 = w.lane * R, first = g.mode == kLine ? g.s + 1 : 0;  // steps from the staged phase to the tile
+  const int64_t j0 = w.lane * R, f_hi = min((int64_t)wi.f_hi, g.sq + 1 + args.anchor_span);
   const unsigned col = smem_u32(w.bins), rstride = M * Warp<P>::kBinStride;
   for (int64_t c = 0; c * 32 < n; ++c) {
     const Obs<P> o = fetch<P>(args, g.mode, base, n, c * 32 + w.lane);
     __syncwarp();
-    put<P>(w, 0, record<P>(args, w, g, g.mode, o), o.aw);
+    put<P>(w, 0, record<P>(args, w, g, g.mode, fixed_anchor(g.fa, w.tbits), o), o.aw);
     __syncwarp();
     const int cnt = (int)((n - c * 32) < 32 ? (n - c * 32) : 32);
     for (int i = 0; i < cnt; ++i) {
@@ -628,16 +606,16 @@ __device__ __forceinline__ void accumulate_slow(const TileArgs& args, const Warp
           m[r] = __umulhi(nl_phase(pd, nl.dh[r], nl.dl[r]), M);
         } else if (PHASE == FPW_PHASE_FP32) {
           const int64_t ak = (k >= 0) ? k - (k % args.K) : 0;
-          const unsigned long long pa = pd.x + (unsigned long long)(ak - g.s + first) * pd.y;
+          const unsigned long long pa = pd.x + (unsigned long long)(ak - g.s) * pd.y;
           const float d32 = (float)(unsigned)(pd.y >> 32) * 0x1p-32f, p32 = (float)(unsigned)(pa >> 32) * 0x1p-32f;
           float p = fmaf((float)(k - ak), d32, p32);
           p = p - floorf(p);
           const unsigned mm = (unsigned)(p * (float)M);
           m[r] = mm < M ? mm : M - 1u;
         } else {
-          m[r] = bin_of_phase(pd.x + (unsigned long long)(first + j0 + r) * pd.y, M);
+          m[r] = bin_of_phase(pd.x + (unsigned long long)(j0 + r) * pd.y, M);
         }
-        if (DUMP && k >= wi.f_lo && k < wi.f_hi && k >= args.bins_k0 && k < args.bins_k1)
+        if (DUMP && k >= wi.f_lo && k < f_hi && k >= args.bins_k0 && k < args.bins_k1)
           args.bins_out[(k - args.bins_k0) * args.bins_nobs + base + c * 32 + i] = (int32_t)m[r];
       }
       Bin v[R];
@@ -654,8 +632,6 @@ __device__ __forceinline__ void accumulate_tile(const TileArgs& args, const Warp
                                                 const NlTile<R>& nl, int64_t base, int64_t n, const WorkItem& wi) {
   if (DUMP || PHASE == FPW_PHASE_FP32 || g.mode == kExact)
     accumulate_slow<R, PHASE, P, DUMP>(args, w, g, nl, base, n, wi);
-  else if (g.mode == kLine)
-    accumulate<R, P, kLine>(args, w, g, nl, base, n, kLine);
   else if (g.mode == kFixed)
     accumulate<R, P, kFixed>(args, w, g, nl, base, n, kFixed);
   else
@@ -690,16 +666,81 @@ __device__ __noinline__ void list_insert(double* topS, int* topI, int kk, double
   __syncwarp();
 }
 
+// Two values of S and, in single precision, a bin offset as 128 bits that are not zero.
+__device__ __forceinline__ ulonglong2 pack_ends(float a, float b, int off) {
+  return make_ulonglong2((unsigned long long)__float_as_uint(b) << 32 | __float_as_uint(a), (unsigned long long)off + 1ull);
+}
+__device__ __forceinline__ ulonglong2 pack_ends(double a, double b, int) {  // (no sum is the NaN of all ones)
+  return make_ulonglong2((unsigned long long)__double_as_longlong(a) + 1ull, (unsigned long long)__double_as_longlong(b) + 1ull);
+}
+__device__ __forceinline__ void unpack_ends(ulonglong2 v, float& a, float& b, int& off) {
+  a = __uint_as_float((unsigned)v.x);
+  b = __uint_as_float((unsigned)(v.x >> 32));
+  off = (int)(v.y - 1ull);
+}
+__device__ __forceinline__ void unpack_ends(ulonglong2 v, double& a, double& b, int& off) {
+  a = __longlong_as_double((long long)(v.x - 1ull));
+  b = __longlong_as_double((long long)(v.y - 1ull));
+  off = 0;
+}
+__device__ __forceinline__ ulonglong2 exchange128(ulonglong2* p, ulonglong2 v) {
+  ulonglong2 r;
+  asm volatile(
+      "{\n\t.reg .b128 a, b;\n\tmov.b128 b, {%2, %3};\n\tatom.global.exch.b128 a, [%4], b;\n\t"
+      "mov.b128 {%0, %1}, a;\n\t}"
+      : "=l"(r.x), "=l"(r.y)
+      : "l"(v.x), "l"(v.y), "l"(p)
+      : "memory");
+  return r;
+}
+
+// Where two items of a curve meet inside an anchor block, the left one's last
+// frequency k and the right one's first, k + 1, lack a neighbour. Each item
+// exchanges the S at its end (of k - 1, k or k + 1, k + 2) with what is at the
+// meeting's place: the first finds nothing there, the second the other's values,
+// and ranks k and k + 1 into its list. left: the item's beginning (S of its first
+// two frequencies, the first one's bin offset), place row; right: its end (S of its
+// last two, the last one's offset), place row + 1. Returns whether the list changed.
+template <class A>
+__device__ __noinline__ bool meet(const TileArgs& args, int64_t row, bool left, bool right, int f_lo, int f_hi, A b0,
+                                  A b1, int boff, A e0, A e1, int eoff, int key_shift, double* topS, int* topI, int kk,
+                                  int lane) {
+  ulonglong2 v = make_ulonglong2(0ull, 0ull);
+  if (lane == 0 && left) v = exchange128(args.meetings + row, pack_ends(b0, b1, boff));
+  if (lane == 1 && right) v = exchange128(args.meetings + row + 1, pack_ends(e0, e1, eoff));
+  const unsigned found = __ballot_sync(0xffffffffu, (v.x | v.y) != 0ull);
+  bool changed = false;
+  for (int side = 0; side < 2; ++side) {
+    if (!(found >> side & 1u)) continue;
+    A o0, o1;
+    int off;
+    unpack_ends(make_ulonglong2(__shfl_sync(0xffffffffu, v.x, side), __shfl_sync(0xffffffffu, v.y, side)), o0, o1, off);
+    const A S[4] = {side ? e0 : o0, side ? e1 : o1, side ? o0 : b0, side ? o1 : b1};
+    const int k = side ? f_hi - 1 : f_lo - 1;
+    const int key[2] = {k << key_shift | (side ? eoff : off), (k + 1) << key_shift | (side ? off : boff)};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const A s = S[1 + q];
+      if (!args.peak_raw && !(s > S[q] && s >= S[2 + q])) continue;
+      const A thr = topI[kk - 1] >= 0 ? (A)topS[kk - 1] : (A)-INFINITY;
+      if (!(s > thr || (s == thr && key[q] < topI[kk - 1]))) continue;
+      list_insert(topS, topI, kk, (double)s, key[q], lane);
+      changed = true;
+    }
+  }
+  return changed;
+}
+
 // Step 4: peaks among the frequencies whose right neighbour is known by now
 // (the tile's own except its last, and the previous tile's last), or every
-// owned one in raw mode, ranked into the list. c1, c2: S of the two
+// owned one in raw mode, ranked into the list: those in [f_lo, f_hi). c1, c2: S of the two
 // frequencies before the tile. The ranking key of frequency k is (k <<
 // key_shift) | extra; ce: the extra of the frequency before the tile.
 // floor: no S below it can be among the curve's k best. Returns whether the list
 // changed.
 template <int R, class P>
 __device__ __forceinline__ bool tile_peaks(const TileArgs& args, const Warp<P>& w, const typename P::S (&S)[R],
-                                           const int (&extra)[R], int key_shift, int64_t s, const WorkItem& wi,
+                                           const int (&extra)[R], int key_shift, int64_t s, int64_t f_lo, int64_t f_hi,
                                            double* topS, int* topI, typename P::S floor,
                                            typename P::S& c1, typename P::S& c2, int& ce) {
   using A = typename P::S;
@@ -727,8 +768,7 @@ __device__ __forceinline__ bool tile_peaks(const TileArgs& args, const Warp<P>& 
     const int64_t k = s + (int64_t)(lane * R + r) - 1;
     v[r] = r > 0 ? S[r > 0 ? r - 1 : 0] : l1;
     const A left = r > 1 ? S[r > 1 ? r - 2 : 0] : (r == 1 ? l1 : l2);
-    const bool owned = k >= wi.f_lo && k < wi.f_hi;
-    if (owned && (args.peak_raw || (v[r] > left && v[r] >= S[r])) && v[r] >= floor) todo |= 1u << r;
+    if (k >= f_lo && k < f_hi && (args.peak_raw || (v[r] > left && v[r] >= S[r])) && v[r] >= floor) todo |= 1u << r;
   }
   bool changed = false;
   A bs = (A)-INFINITY;  // the lane's best candidate (lowest key first where equal)
@@ -868,16 +908,30 @@ __device__ __forceinline__ int next_item(const TileArgs& args, bool first, int l
   return (int)(gridDim.x * (blockDim.x >> 5) + __shfl_sync(0xffffffffu, q, 0));
 }
 
-// Does the whole grid lie on the line through its first frequency, for every
-// curve's times (the usual case: a curve's own times are then not looked at)? A
-// frequency is off it by its block's deviation, its anchor's distance, and the
-// rounding of the step over F steps. And do all terms t delta fit record()'s 31
-// bits? Else every tile is looked at, and tiles keep to their blocks.
+// Do all blocks lie on lines for every curve's times, and are all anchors in reach
+// of the fixed-point times (the usual case: a curve's own times and the anchors
+// are then not looked at)?
 __device__ __forceinline__ bool grid_is_linear(const TileArgs& args) {
-  if (!args.rec) return false;
-  const double dev = __uint_as_float(args.grid_dev[0]), tmax = __uint_as_float(args.grid_dev[1]);
-  const double far = __uint_as_float(args.grid_dev[2]);  // units of 2^-96
-  return (dev + far * 0x1p-96) * tmax + (double)args.nfreq * 0x1p-64 <= kGridTolCycles && far * tmax < 0x1p62;
+  if (!args.rec || args.grid_dev[2] != 0u) return false;
+  return (double)__uint_as_float(args.grid_dev[0]) * (double)__uint_as_float(args.grid_dev[1]) <= kGridTolCycles;
+}
+
+// The item's frequencies in the tile's block: [wi.f_lo, f_hi); whether they begin
+// or end inside the block, where another item goes on, and whether the tile is
+// their last.
+struct Part {
+  int f_hi;
+  bool open, cut, last;
+};
+template <int W>
+__device__ __forceinline__ Part part_of(const TileArgs& args, const WorkItem& wi, int64_t s, int q, int halo) {
+  const int64_t lo = q * args.anchor_span, hi = lo + args.anchor_span;
+  Part p;
+  p.f_hi = (int)min((int64_t)wi.f_hi, hi);
+  p.open = halo && wi.f_lo != lo;
+  p.cut = halo && p.f_hi < args.nfreq && p.f_hi != hi;
+  p.last = s + W >= (int64_t)p.f_hi + (p.cut ? 0 : halo);
+  return p;
 }
 
 // At most kTileMaxThreads threads a block (wider shapes are launched as more
@@ -894,7 +948,6 @@ __global__ void __launch_bounds__(kTileMaxThreads, 1) tile_kernel(const __grid_c
   const bool grid_bad = (*(volatile unsigned*)args.status & kStatusGrid) != 0u;
   const A cal = (A)args.inv_alpha2;
   const bool every_lin = grid_is_linear(args);
-  const bool aligned = args.aligned;
   const bool plain_prior = args.inv_alpha2 == 0.0 || (args.inv_alpha2 > 0x1p-90 && args.inv_alpha2 < 0x1p+90);
   const int halo = w.kk > 0 ? 1 : 0;  // peaks need both neighbours of every owned frequency
   const int M = w.M, j0 = w.lane * R;
@@ -912,25 +965,16 @@ __global__ void __launch_bounds__(kTileMaxThreads, 1) tile_kernel(const __grid_c
     const bool plain = !(args.curve_bad[c] & kCurveWide) && plain_prior;
     A c1 = (A)-INFINITY, c2 = (A)-INFINITY;
     int ce = 0;
-    const int64_t f_end = wi.f_hi;
-    int64_t s = (int64_t)wi.f_lo - halo;
-    int64_t q = aligned ? (unsigned)wi.f_lo / (unsigned)args.anchor_span : 0;  // the range's anchor block
-    float delta = aligned && args.rec && wi.f_lo < f_end ? args.block_delta[q] : 0.f;
-    while (wi.f_lo < f_end) {
-      if (aligned) wi.f_hi = (int32_t)min(f_end, (q + 1) * args.anchor_span);
+    int q = (int)((unsigned)wi.f_lo / (unsigned)args.anchor_span);  // the anchor block of wi.f_lo and the tile
+    int64_t s = (int64_t)wi.f_lo - (wi.f_lo == q * args.anchor_span ? halo : 0);
+    while (wi.f_lo < wi.f_hi) {
       NlTile<R> nl;
-      const Tile g = make_tile<R, P>(args, w, s, q, delta, tm, every_lin, aligned, nl);
-      // the next tile: on from this one, or the start of the next block's range
-      const bool last = s + W >= (int64_t)wi.f_hi + halo;
-      const int64_t sn = last ? (int64_t)wi.f_hi - halo : s + W, lon = last ? wi.f_hi : wi.f_lo;
-      if (aligned && last) {
-        ++q;
-        if (args.rec && lon < f_end) delta = args.block_delta[q];
-      }
+      const Tile g = make_tile<R, P>(args, w, s, q, tm, every_lin, args.curve_bad[c] & kCurveUnfit, nl);
       const unsigned long long floor = w.kk > 0 ? curve_floor(args, c) : 0ull;
       accumulate_tile<R, PHASE, P, DUMP>(args, w, g, nl, base, n, wi);
 
       // S and the peak test stay in the policy's reduce type
+      const Part part = part_of<W>(args, wi, s, q, halo);
       A S[R];
       if (plain)
         reduce_bins<R, P, true>(w, cal, S);
@@ -939,19 +983,29 @@ __global__ void __launch_bounds__(kTileMaxThreads, 1) tile_kernel(const __grid_c
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int64_t k = s + (int64_t)(j0 + r);
-        if (args.S_out && k >= wi.f_lo && k < wi.f_hi) args.S_out[(int64_t)c * F + k] = (double)S[r];
+        if (args.S_out && k >= wi.f_lo && k < part.f_hi) args.S_out[(int64_t)c * F + k] = (double)S[r];
         if (k < 0 || k >= F) S[r] = (A)-INFINITY;
       }
       if (w.kk > 0) {
         int zero[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) zero[r] = 0;
-        if (tile_peaks<R, P>(args, w, S, zero, 0, s, wi, w.topS, w.topI, floor_value<A>(floor), c1, c2, ce))
-          raise_floor(args, c, w.topS, w.topI, w.kk, w.lane);
+        bool changed = tile_peaks<R, P>(args, w, S, zero, 0, s, wi.f_lo + (part.open ? 1 : 0), part.f_hi, w.topS,
+                                        w.topI, floor_value<A>(floor), c1, c2, ce);
+        const bool left = part.open && s == wi.f_lo, right = part.last && part.cut;
+        if (left || right)
+          changed |= meet<A>(args, wi.slot, left, right, wi.f_lo, part.f_hi, __shfl_sync(0xffffffffu, S[0], 0),
+                             __shfl_sync(0xffffffffu, S[R > 1 ? 1 : 0], R > 1 ? 0 : 1), 0, c2, c1, 0, 0, w.topS, w.topI,
+                             w.kk, w.lane);
+        if (changed) raise_floor(args, c, w.topS, w.topI, w.kk, w.lane);
       }
-      if (last) c1 = c2 = (A)-INFINITY;
-      s = sn;
-      wi.f_lo = (int32_t)lon;
+      s += W;
+      if (part.last) {
+        c1 = c2 = (A)-INFINITY;
+        wi.f_lo = part.f_hi;
+        s = part.f_hi - halo;
+        ++q;
+      }
     }
     item_end(args, w, wi, 1);
   }
@@ -1202,7 +1256,6 @@ __global__ void __launch_bounds__(kMultiMaxThreads, 1) tile_kernel_multi(const _
   const bool grid_bad = (*(volatile unsigned*)args.status & kStatusGrid) != 0u;
   const A cal = (A)args.inv_alpha2;
   const bool every_lin = grid_is_linear(args);
-  const bool aligned = args.aligned;
   const bool plain_prior = args.inv_alpha2 == 0.0 || (args.inv_alpha2 > 0x1p-90 && args.inv_alpha2 < 0x1p+90);
   const int halo = kk > 0 ? 1 : 0;
   const int j0 = w.lane * R;
@@ -1221,39 +1274,37 @@ __global__ void __launch_bounds__(kMultiMaxThreads, 1) tile_kernel_multi(const _
     // S and offset of the two frequencies before the tile, per group (lane g holds group g's)
     A carry1 = -INFINITY, carry2 = -INFINITY;
     int carrye = 0;
-    const int64_t f_end = wi.f_hi;
-    int64_t s = (int64_t)wi.f_lo - halo;
-    int64_t q = aligned ? (unsigned)wi.f_lo / (unsigned)args.anchor_span : 0;  // the range's anchor block
-    float delta = aligned && args.rec && wi.f_lo < f_end ? args.block_delta[q] : 0.f;
-    while (wi.f_lo < f_end) {
-      if (aligned) wi.f_hi = (int32_t)min(f_end, (q + 1) * args.anchor_span);
+    int q = (int)((unsigned)wi.f_lo / (unsigned)args.anchor_span);  // the anchor block of wi.f_lo and the tile
+    int64_t s = (int64_t)wi.f_lo - (wi.f_lo == q * args.anchor_span ? halo : 0);
+    while (wi.f_lo < wi.f_hi) {
       NlTile<R> nl;
-      const Tile g0 = make_tile<R, P>(args, w, s, q, delta, tm, every_lin, aligned, nl);
-      // the next tile: on from this one, or the start of the next block's range
-      const bool last = s + W >= (int64_t)wi.f_hi + halo;
-      const int64_t sn = last ? (int64_t)wi.f_hi - halo : s + W, lon = last ? wi.f_hi : wi.f_lo;
-      if (aligned && last) {
-        ++q;
-        if (args.rec && lon < f_end) delta = args.block_delta[q];
-      }
+      const Tile g0 = make_tile<R, P>(args, w, s, q, tm, every_lin, args.curve_bad[c] & kCurveUnfit, nl);
       accumulate_tile<R, PHASE, P, false>(args, w, g0, nl, base, n, wi);
 
       // the reported S of group g per owned frequency, and the peaks
       auto emit = [&](int g, const A (&S)[R], const int (&off)[R]) {
+        const Part part = part_of<W>(args, wi, s, q, halo);
         if (args.S_out) {
 #pragma unroll
           for (int r = 0; r < R; ++r) {
             const int64_t k = s + (int64_t)(j0 + r);
-            if (k >= wi.f_lo && k < wi.f_hi) args.S_out[((int64_t)c * ng + g) * F + k] = (double)S[r];
+            if (k >= wi.f_lo && k < part.f_hi) args.S_out[((int64_t)c * ng + g) * F + k] = (double)S[r];
           }
         }
         if (kk > 0) {
           A c1 = __shfl_sync(0xffffffffu, carry1, g), c2 = __shfl_sync(0xffffffffu, carry2, g);
           int ce = __shfl_sync(0xffffffffu, carrye, g);
           const int64_t row = (int64_t)c * ng + g;
-          if (tile_peaks<R, P>(args, w, S, off, 6, s, wi, w.topS + g * kk, w.topI + g * kk,
-                               floor_value<A>(curve_floor(args, row)), c1, c2, ce))
-            raise_floor(args, row, w.topS + g * kk, w.topI + g * kk, kk, w.lane);
+          double* const topS = w.topS + g * kk;
+          int* const topI = w.topI + g * kk;
+          bool changed = tile_peaks<R, P>(args, w, S, off, 6, s, wi.f_lo + (part.open ? 1 : 0), part.f_hi, topS, topI,
+                                          floor_value<A>(curve_floor(args, row)), c1, c2, ce);
+          const bool left = part.open && s == wi.f_lo, right = part.last && part.cut;
+          if (left || right)
+            changed |= meet<A>(args, g * args.group_rows + wi.slot, left, right, wi.f_lo, part.f_hi,
+                               __shfl_sync(0xffffffffu, S[0], 0), __shfl_sync(0xffffffffu, S[R > 1 ? 1 : 0], R > 1 ? 0 : 1),
+                               __shfl_sync(0xffffffffu, off[0], 0), c2, c1, ce, 6, topS, topI, kk, w.lane);
+          if (changed) raise_floor(args, row, topS, topI, kk, w.lane);
           if (w.lane == g) {
             carry1 = c1;
             carry2 = c2;
@@ -1318,9 +1369,14 @@ __global__ void __launch_bounds__(kMultiMaxThreads, 1) tile_kernel_multi(const _
       }
       // clear the bins for the next tile
       for (int q = 0; q < R * Mx && (SPEC == 0 || !plain); ++q) reinterpret_cast<float2*>(w.bins)[q * 32] = make_float2(0.f, 0.f);
-      if (last) carry1 = carry2 = -INFINITY;
-      s = sn;
-      wi.f_lo = (int32_t)lon;
+      const Part part = part_of<W>(args, wi, s, q, halo);
+      s += W;
+      if (part.last) {
+        carry1 = carry2 = -INFINITY;
+        wi.f_lo = part.f_hi;
+        s = part.f_hi - halo;
+        ++q;
+      }
     }
     item_end(args, w, wi, ng);
   }

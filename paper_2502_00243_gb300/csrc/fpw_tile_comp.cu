@@ -15,7 +15,6 @@ const void* tile_fn_comp(int R, int phase_mode, bool dump) {
   }
   FPW_INST(1)
   FPW_INST(2)
-  FPW_INST(3)
   FPW_INST(4)
   FPW_INST(8)
 #undef FPW_INST

@@ -12,7 +12,7 @@ const void* tile_fn_multi(int R, int phase_mode, int spec) {
   if (!fp32p) {  // at the frequencies per lane that the default shapes take
     if (spec == 1 && R == 2) return (const void*)&tile_kernel_multi<2, FPW_PHASE_FIXED64, 1>;
     if (spec == 2 && R == 2) return (const void*)&tile_kernel_multi<2, FPW_PHASE_FIXED64, 2>;
-    if (spec == 3 && R == 5) return (const void*)&tile_kernel_multi<5, FPW_PHASE_FIXED64, 3>;
+    if (spec == 3 && R == 4) return (const void*)&tile_kernel_multi<4, FPW_PHASE_FIXED64, 3>;
     if (spec == 3 && R == 2) return (const void*)&tile_kernel_multi<2, FPW_PHASE_FIXED64, 3>;
   }
 #define FPW_INST(RR)                                                                      \
@@ -21,9 +21,7 @@ const void* tile_fn_multi(int R, int phase_mode, int spec) {
                  : (const void*)&tile_kernel_multi<RR, FPW_PHASE_FIXED64, 0>;
   FPW_INST(1)
   FPW_INST(2)
-  FPW_INST(3)
   FPW_INST(4)
-  FPW_INST(5)
   FPW_INST(8)
 #undef FPW_INST
   return nullptr;
