@@ -47,9 +47,10 @@
 //
 // Grids that are not linear to within kGridTolCycles over a tile: the phase is
 // frac(t_i f_b) (exact, f_b the tile's middle frequency) plus t_i (f_k - f_b) from
-// FP32 pairs, correct to 2^-36 cycles (NlTile). A tile whose frequencies spread
-// over more than 2^7 cycles either side takes a direct exact anchor per (observation,
-// frequency).
+// FP32 pairs, correct to 2^-36 cycles (NlTile), and the exact product where that
+// leaves the bin open: the bins are those of frac(t_i f_k), whatever the tile. A
+// tile whose frequencies spread over more than 2^7 cycles either side takes a
+// direct exact anchor per (observation, frequency).
 //
 // Bin sums (policy P): FP32 pairs (A, B); binary64 pairs; or FP32 pairs with
 // compensation terms (A, B, cA, cB), where each addition is an exact two-sum
@@ -345,6 +346,13 @@ enum TileMode { kRecord, kAnchor, kFixed, kExact };
 // 30 lanes/clk/SM, fma at 110 (measured); the same sum from 61-bit integer
 // factors (three mul.hi more than the linear step) ran 1.04e12 evaluations/s at
 // M = 20.
+// The bin is that of the exact phase's leading 32 bits. The sum's are the same or
+// one more, and the bin another one only where the last one is the first of its
+// bin, the low word of M times it below M: M in 2^32 pairs, which take the exact
+// product (exact_bin). Times of 0 would all do: their phase is staged as a unit of
+// 2^-32 and a half, which is as well in bin 0. Asked per observation: 24 curves x
+// 100003 frequencies 1440 us -> 1760 (6600 with the exact product of every pair);
+// asked once a tile, which then starts over, 2100, its warps end so much later.
 template <int R>
 struct NlTile {
   float dh[R], dl[R];
@@ -363,6 +371,8 @@ __device__ __forceinline__ unsigned nl_phase(const ulonglong2& pd, float dh, flo
   const int low = (int)(__float_as_uint(e) + (unsigned)(pd.x >> 32));
   return (__float_as_uint(m) << 18) + (unsigned)pd.x + (unsigned)(low >> 4);
 }
+
+__device__ __noinline__ unsigned exact_bin(double t, double f, unsigned M) { return bin_of_phase(phase_fixed64(t, f), M); }
 
 // Geometry of one tile: first frequency s (-1 possible), its anchor block's first
 // position sq and anchor frequency fa (index max(sq, 0)), and how its phases are
@@ -470,7 +480,7 @@ __device__ __forceinline__ ulonglong2 record(const TileArgs& args, const Warp<P>
   unsigned long long Pa = phase_fixed64(t, g.fa);
   if (mode == kFixed) {
     const float2 tt = split_f32(t);
-    const unsigned long long p = ((Pa + 0xfffffffull) >> 28) + 1ull;  // units of 2^-36, rounded up, one more
+    const unsigned long long p = t == 0.0 ? 24ull : ((Pa + 0xfffffffull) >> 28) + 1ull;  // units of 2^-36, rounded up, one more
     const unsigned c = (unsigned)(p & 15ull) - kMagicLow;
     return make_ulonglong2(((unsigned long long)c << 32) | (unsigned)(p >> 4),
                            ((unsigned long long)__float_as_uint(tt.y) << 32) | __float_as_uint(tt.x));
@@ -508,11 +518,23 @@ __device__ __forceinline__ void accumulate(const TileArgs& args, const Warp<P>& 
   const unsigned j0 = (unsigned)w.lane * R;
   const unsigned col = smem_u32(w.bins), rstride = M * Warp<P>::kBinStride;
   const int64_t npad = (n + U - 1) / U * U, nchunk = (n + kChunk - 1) / kChunk;
-  const auto addresses = [&](const ulonglong2& p, unsigned (&ad)[R]) {
+  const auto addresses = [&](const ulonglong2& p, int64_t i, unsigned (&ad)[R]) {  // i: the observation
     if (MODE == kFixed) {
+      unsigned low = ~0u;
 #pragma unroll
-      for (int r = 0; r < R; ++r)
-        ad[r] = col + (unsigned)r * rstride + __umulhi(nl_phase(p, nl.dh[r], nl.dl[r]), M) * Warp<P>::kBinStride;
+      for (int r = 0; r < R; ++r) {
+        const unsigned ph = nl_phase(p, nl.dh[r], nl.dl[r]);
+        low = min(low, ph * M);
+        ad[r] = col + (unsigned)r * rstride + __umulhi(ph, M) * Warp<P>::kBinStride;
+      }
+      if (low < M && i < n) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+          if (nl_phase(p, nl.dh[r], nl.dl[r]) * M < M) {
+            const int64_t k = max((int64_t)0, min(w.F - 1, g.s + j0 + r));
+            ad[r] = col + (unsigned)r * rstride + exact_bin(args.t[base + i], args.freqs[k], M) * Warp<P>::kBinStride;
+          }
+      }
     } else {
       const unsigned long long phi = p.x + (unsigned long long)j0 * p.y;
 #pragma unroll
@@ -533,7 +555,7 @@ __device__ __forceinline__ void accumulate(const TileArgs& args, const Warp<P>& 
   In x0, x1;
   unsigned ad[R];
   lds(pd0, p1);
-  addresses(p1, ad);
+  addresses(p1, 0, ad);
   lds(aw0, x0);
   lds(pd0 + 16u, p1);
   lds(aw0 + (unsigned)sizeof(In), x1);
@@ -553,7 +575,7 @@ __device__ __forceinline__ void accumulate(const TileArgs& args, const Warp<P>& 
         lds(pa + (unsigned)u * 16u, p2);  // two records ahead: staged, a copy, or a slot whose value is not used
         lds(xa + (unsigned)u * (unsigned)sizeof(In), x2);
         unsigned an[R];
-        addresses(p1, an);
+        addresses(p1, c * kChunk + i + u + 1, an);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           sts(ad[r], bin_add(v[r], x0));
@@ -603,7 +625,9 @@ __device__ __forceinline__ void accumulate_slow(const TileArgs& args, const Warp
           const int64_t kc = k < 0 ? 0 : (k >= w.F ? w.F - 1 : k);
           m[r] = bin_of_phase(phase_fixed64(__longlong_as_double((long long)pd.x), args.freqs[kc]), M);
         } else if (g.mode == kFixed) {
-          m[r] = __umulhi(nl_phase(pd, nl.dh[r], nl.dl[r]), M);
+          const unsigned ph = nl_phase(pd, nl.dh[r], nl.dl[r]);
+          m[r] = __umulhi(ph, M);
+          if (ph * M < M) m[r] = exact_bin(args.t[base + c * 32 + i], args.freqs[k < 0 ? 0 : (k >= w.F ? w.F - 1 : k)], M);
         } else if (PHASE == FPW_PHASE_FP32) {
           const int64_t ak = (k >= 0) ? k - (k % args.K) : 0;
           const unsigned long long pa = pd.x + (unsigned long long)(ak - g.s) * pd.y;
