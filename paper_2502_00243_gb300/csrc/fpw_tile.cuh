@@ -60,8 +60,8 @@
 // hi + lo rounded once to FP32, and S is accumulated in binary64.
 //
 // DUMP instantiations additionally write the bin m of every (observation,
-// owned frequency k) with bins_k0 <= k < bins_k1 to args.bins_out, from the
-// same phase arithmetic as the sums (bin-identity checks of the product kernel).
+// owned frequency k) with bins_k0 <= k < bins_k1 to args.bins_out, in the loop that
+// forms the sums (bin-identity checks of the product kernel).
 #pragma once
 #include <math.h>
 
@@ -330,9 +330,10 @@ __device__ __forceinline__ int exponent_of(double v) {  // floor(log2 |v|) for n
 // How a tile's phases are formed: stepped from the exact phase at the anchor of
 // the tile's block (the block on a line), which kRecord takes from the prep
 // kernel's fixed-point times and kAnchor from the general product (the same
-// number, where a time or the anchor is not of that form); products with the distance from an exact phase (NlTile); the exact
-// phase of every pair.
-enum TileMode { kRecord, kAnchor, kFixed, kExact };
+// number, where a time or the anchor is not of that form); products with the
+// distance from an exact phase (NlTile); the exact phase of every pair. kStep32: the bins of kRecord or kAnchor's records by
+// FPW_PHASE_FP32's rule, an FP32 phase every K frequencies and FP32 steps.
+enum TileMode { kRecord, kAnchor, kFixed, kExact, kStep32 };
 
 // The frequencies of a tile off the linear grid, as FP32 pairs of f_k - f_b (f_b:
 // the tile's middle frequency). An observation's phase at f_k is its exact phase
@@ -507,39 +508,76 @@ __device__ __forceinline__ void put(const Warp<P>& w, int64_t c, const ulonglong
 // pipelined registers instead of moving them. Against the loop that formed and
 // used an observation's bins in the same trip (probe, loop alone): M = 20, R =
 // 5, 8 warps per SM 1.85 -> 2.08e12 evaluations/s; M = 60, R = 3, 4 warps 1.15
-// -> 1.5e12. MODE kRecord serves kAnchor too (mode).
-template <int R, class P, TileMode MODE>
+// -> 1.5e12. One loop for every way of forming the bins, with and without the
+// dump (FPW_PHASE_FP32 and the exact phase of every pair ran 0.16e12 and 0.26e12
+// evaluations/s at M = 20 in a plain loop of their own, 1.35e12 and 0.30e12 in
+// this one). MODE kRecord serves kAnchor too (mode).
+template <int R, class P, TileMode MODE, bool DUMP>
 __device__ __forceinline__ void accumulate(const TileArgs& args, const Warp<P>& w, const Tile& g, const NlTile<R>& nl,
-                                           int64_t base, int64_t n, TileMode mode) {
+                                           int64_t base, int64_t n, const WorkItem& wi, TileMode mode) {
   using Bin = typename P::Bin;
   using In = typename P::In;
-  constexpr int U = 4, kChunk = 32;
+  constexpr int U = MODE == kExact ? 1 : 4, kChunk = 32;  // (the product of a pair is long enough by itself)
   const unsigned M = (unsigned)w.M;
   const unsigned j0 = (unsigned)w.lane * R;
   const unsigned col = smem_u32(w.bins), rstride = M * Warp<P>::kBinStride;
   const int64_t npad = (n + U - 1) / U * U, nchunk = (n + kChunk - 1) / kChunk;
-  const auto addresses = [&](const ulonglong2& p, int64_t i, unsigned (&ad)[R]) {  // i: the observation
+  const auto freq = [&](int r) { return args.freqs[max((int64_t)0, min(w.F - 1, g.s + j0 + r))]; };
+  double f[MODE == kExact ? R : 1];
+  float past[MODE == kStep32 ? R : 1];  // steps past the frequency's FP32 anchor, and from the tile's first to that
+  int anchor32[MODE == kStep32 ? R : 1];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    if (MODE == kExact) f[r] = freq(r);
+    if (MODE == kStep32) {
+      const int k = (int)(g.s + j0 + r), ak = k >= 0 ? k - k % args.K : 0;
+      past[r] = (float)(k - ak);
+      anchor32[r] = ak - (int)g.s;
+    }
+  }
+  const int64_t dump_hi = min((int64_t)wi.f_hi, g.sq + 1 + args.anchor_span);
+  // the addresses of the bins of observation i, whose record is p
+  const auto addresses = [&](const ulonglong2& p, int64_t i, unsigned (&ad)[R]) {
+    unsigned m[R];
     if (MODE == kFixed) {
       unsigned low = ~0u;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const unsigned ph = nl_phase(p, nl.dh[r], nl.dl[r]);
         low = min(low, ph * M);
-        ad[r] = col + (unsigned)r * rstride + __umulhi(ph, M) * Warp<P>::kBinStride;
+        m[r] = __umulhi(ph, M);
       }
       if (low < M && i < n) {
 #pragma unroll
         for (int r = 0; r < R; ++r)
-          if (nl_phase(p, nl.dh[r], nl.dl[r]) * M < M) {
-            const int64_t k = max((int64_t)0, min(w.F - 1, g.s + j0 + r));
-            ad[r] = col + (unsigned)r * rstride + exact_bin(args.t[base + i], args.freqs[k], M) * Warp<P>::kBinStride;
-          }
+          if (nl_phase(p, nl.dh[r], nl.dl[r]) * M < M) m[r] = exact_bin(args.t[base + i], freq(r), M);
+      }
+    } else if (MODE == kExact) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) m[r] = bin_of_phase(phase_fixed64(__longlong_as_double((long long)p.x), f[r]), M);
+    } else if (MODE == kStep32) {
+      const float d32 = (float)(unsigned)(p.y >> 32) * 0x1p-32f;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const unsigned long long pa = p.x + (unsigned long long)(long long)anchor32[r] * p.y;
+        float ph = fmaf(past[r], d32, (float)(unsigned)(pa >> 32) * 0x1p-32f);
+        ph = ph - floorf(ph);
+        const unsigned b = (unsigned)(ph * (float)M);
+        m[r] = b < M ? b : M - 1u;
       }
     } else {
       const unsigned long long phi = p.x + (unsigned long long)j0 * p.y;
 #pragma unroll
-      for (int r = 0; r < R; ++r)
-        ad[r] = col + (unsigned)r * rstride + bin_of_phase(phi + (unsigned long long)r * p.y, M) * Warp<P>::kBinStride;
+      for (int r = 0; r < R; ++r) m[r] = bin_of_phase(phi + (unsigned long long)r * p.y, M);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      ad[r] = col + (unsigned)r * rstride + m[r] * Warp<P>::kBinStride;
+      if (DUMP) {
+        const int64_t k = g.s + j0 + r;
+        if (i < n && k >= wi.f_lo && k < dump_hi && k >= args.bins_k0 && k < args.bins_k1)
+          args.bins_out[(k - args.bins_k0) * args.bins_nobs + base + i] = (int32_t)m[r];
+      }
     }
   };
   Obs<P> o = fetch<P>(args, mode, base, n, w.lane);
@@ -597,69 +635,15 @@ __device__ __forceinline__ void accumulate(const TileArgs& args, const Warp<P>& 
   }
 }
 
-// The same sums one observation at a time, for what is not worth a loop of its
-// own: exact anchors per pair, the FP32 phase (an FP32 anchor every K
-// frequencies), and the bin dump.
-template <int R, int PHASE, class P, bool DUMP>
-__device__ __forceinline__ void accumulate_slow(const TileArgs& args, const Warp<P>& w, const Tile& g,
-                                             const NlTile<R>& nl, int64_t base, int64_t n, const WorkItem& wi) {
-  using Bin = typename P::Bin;
-  using In = typename P::In;
-  const unsigned M = (unsigned)w.M;
-  const int64_t j0 = w.lane * R, f_hi = min((int64_t)wi.f_hi, g.sq + 1 + args.anchor_span);
-  const unsigned col = smem_u32(w.bins), rstride = M * Warp<P>::kBinStride;
-  for (int64_t c = 0; c * 32 < n; ++c) {
-    const Obs<P> o = fetch<P>(args, g.mode, base, n, c * 32 + w.lane);
-    __syncwarp();
-    put<P>(w, 0, record<P>(args, w, g, g.mode, fixed_anchor(g.fa, w.tbits), o), o.aw);
-    __syncwarp();
-    const int cnt = (int)((n - c * 32) < 32 ? (n - c * 32) : 32);
-    for (int i = 0; i < cnt; ++i) {
-      const ulonglong2 pd = w.pd[i];
-      const In x = w.aw[i];
-      unsigned m[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int64_t k = g.s + j0 + r;
-        if (g.mode == kExact) {
-          const int64_t kc = k < 0 ? 0 : (k >= w.F ? w.F - 1 : k);
-          m[r] = bin_of_phase(phase_fixed64(__longlong_as_double((long long)pd.x), args.freqs[kc]), M);
-        } else if (g.mode == kFixed) {
-          const unsigned ph = nl_phase(pd, nl.dh[r], nl.dl[r]);
-          m[r] = __umulhi(ph, M);
-          if (ph * M < M) m[r] = exact_bin(args.t[base + c * 32 + i], args.freqs[k < 0 ? 0 : (k >= w.F ? w.F - 1 : k)], M);
-        } else if (PHASE == FPW_PHASE_FP32) {
-          const int64_t ak = (k >= 0) ? k - (k % args.K) : 0;
-          const unsigned long long pa = pd.x + (unsigned long long)(ak - g.s) * pd.y;
-          const float d32 = (float)(unsigned)(pd.y >> 32) * 0x1p-32f, p32 = (float)(unsigned)(pa >> 32) * 0x1p-32f;
-          float p = fmaf((float)(k - ak), d32, p32);
-          p = p - floorf(p);
-          const unsigned mm = (unsigned)(p * (float)M);
-          m[r] = mm < M ? mm : M - 1u;
-        } else {
-          m[r] = bin_of_phase(pd.x + (unsigned long long)(j0 + r) * pd.y, M);
-        }
-        if (DUMP && k >= wi.f_lo && k < f_hi && k >= args.bins_k0 && k < args.bins_k1)
-          args.bins_out[(k - args.bins_k0) * args.bins_nobs + base + c * 32 + i] = (int32_t)m[r];
-      }
-      Bin v[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r) lds(col + (unsigned)r * rstride + m[r] * Warp<P>::kBinStride, v[r]);
-#pragma unroll
-      for (int r = 0; r < R; ++r) sts(col + (unsigned)r * rstride + m[r] * Warp<P>::kBinStride, bin_add(v[r], x));
-    }
-  }
-}
-
 template <int R, int PHASE, class P, bool DUMP>
 __device__ __forceinline__ void accumulate_tile(const TileArgs& args, const Warp<P>& w, const Tile& g,
                                                 const NlTile<R>& nl, int64_t base, int64_t n, const WorkItem& wi) {
-  if (DUMP || PHASE == FPW_PHASE_FP32 || g.mode == kExact)
-    accumulate_slow<R, PHASE, P, DUMP>(args, w, g, nl, base, n, wi);
+  if (g.mode == kExact)
+    accumulate<R, P, kExact, DUMP>(args, w, g, nl, base, n, wi, kExact);
   else if (g.mode == kFixed)
-    accumulate<R, P, kFixed>(args, w, g, nl, base, n, kFixed);
+    accumulate<R, P, kFixed, DUMP>(args, w, g, nl, base, n, wi, kFixed);
   else
-    accumulate<R, P, kRecord>(args, w, g, nl, base, n, g.mode);
+    accumulate<R, P, PHASE == FPW_PHASE_FP32 ? kStep32 : kRecord, DUMP>(args, w, g, nl, base, n, wi, g.mode);
 }
 
 // Inserts (s, key) into the list topS/topI (kk entries sorted by S descending,
