@@ -11,6 +11,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <exception>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -356,8 +357,8 @@ Plan* build_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const T
   std::stable_sort(order.begin(), order.end(),
                    [&](int64_t x, int64_t y) { return off[x + 1] - off[x] > off[y + 1] - off[y]; });
   const double least = left / ((double)resident * 4.0 * (double)sh.items);
-  std::vector<WorkItem> sorted;  // the shares shrink as the list grows
-  sorted.reserve((size_t)C + (size_t)(resident * sh.items));
+  std::vector<WorkItem> sorted;  // (no room asked for by sh.items, which is the caller's)
+  sorted.reserve((size_t)C + (size_t)(8 * resident));
   std::vector<int32_t> base((size_t)C + 1, 0);
   bool meetings = false;
   for (const int64_t c : order) {
@@ -436,7 +437,12 @@ Plan* get_plan(fpw_ctx* ctx, const int64_t* off, int64_t C, int64_t F, const Til
       *err = FPW_OK;
       return p;
     }
-  Plan* p = build_plan(ctx, off, C, F, sh, blocks_per_sm, halo, key, st, err);
+  Plan* p = nullptr;
+  try {
+    p = build_plan(ctx, off, C, F, sh, blocks_per_sm, halo, key, st, err);
+  } catch (const std::exception&) {  // the lists' memory: no exception leaves the library
+    *err = FPW_ENOMEM;
+  }
   if (!p) return nullptr;
   p->use = ++ctx->tick;
   if ((int)ctx->plans.size() >= kMaxPlans) {
