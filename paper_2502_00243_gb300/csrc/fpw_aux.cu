@@ -468,6 +468,14 @@ cudaError_t launch_latch(unsigned* words, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+cudaError_t allow_shared_memory(const void* fn, int static_smem) {
+  int dev = 0, limit = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, limit - static_smem);
+}
+
 cudaError_t launch_fill_topk(int32_t* idx, float* S, int64_t n, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   int64_t blocks = (n + 255) / 256;

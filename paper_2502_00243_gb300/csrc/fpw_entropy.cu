@@ -226,7 +226,7 @@ cudaError_t launch_entropy_dense(const double* t, int64_t n, const double* freqs
                    : R == 2 ? reinterpret_cast<const void*>(&entropy_dense_kernel<2>)
                             : reinterpret_cast<const void*>(&entropy_dense_kernel<1>);
   const size_t smem = (size_t)(kEntChunk + 1) * 16 + kEntTable * 4 + (size_t)R * M * kEntThreads * 4;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_shared_memory(fn, 64);  // s_tm, s_df
   if (e != cudaSuccess) return e;
   const int64_t per_block = (int64_t)kEntThreads * R;
   const int64_t blocks = (nfreq + per_block - 1) / per_block;
@@ -240,7 +240,7 @@ cudaError_t launch_entropy_peaks(const int64_t* offsets, int64_t ncurves, const 
   const int64_t total = ncurves * k;
   if (total <= 0) return cudaSuccess;
   const size_t smem = (size_t)kPeakWarps * M * 4;
-  cudaError_t e = cudaFuncSetAttribute(entropy_peaks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_shared_memory(reinterpret_cast<const void*>(&entropy_peaks_kernel), 0);
   if (e != cudaSuccess) return e;
   int64_t blocks = (total + kPeakWarps - 1) / kPeakWarps;
   blocks = blocks > 65535 ? 65535 : blocks;

@@ -187,6 +187,10 @@ bool tile_has_R(int R, int accum, bool multi);     // ... of the kernel for this
 // bin-dumping instantiation when a.bins_out != NULL.
 cudaError_t launch_tile(const TileArgs& a, const TileShape& s, int phase_mode, int accum, int grid, cudaStream_t st);
 cudaError_t launch_prep(const PrepArgs& a, cudaStream_t st);
+// Lets blocks of kernel fn (static_smem bytes of its own) have all the shared
+// memory that the current device gives one. The limit is the kernel's, not the
+// call's: calls of other sizes, from other threads, share it, so it is always this.
+cudaError_t allow_shared_memory(const void* fn, int static_smem);
 cudaError_t launch_merge(const MergeArgs& a, cudaStream_t st);
 cudaError_t launch_plain(const PlainArgs& a, cudaStream_t st);
 cudaError_t launch_dense_topk(const DenseTopkArgs& a, cudaStream_t st);

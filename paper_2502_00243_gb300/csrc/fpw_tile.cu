@@ -46,8 +46,8 @@ bool tile_has_R(int R, int accum, bool multi) {
 
 int tile_max_blocks_per_sm(int R, int phase_mode, int accum, int T, size_t smem, bool multi, bool dump, int spec) {
   const void* fn = pick(R, phase_mode, accum, multi, dump, spec);
-  // the kernel's own limit of dynamic shared memory, once it is known which one runs
-  if (!fn || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+  // (here, where it is known which one runs: the others need not be loaded)
+  if (!fn || allow_shared_memory(fn, 0) != cudaSuccess) return 0;
   int nb = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, T, smem) != cudaSuccess) return 0;
   return nb;
@@ -57,8 +57,6 @@ cudaError_t launch_tile(const TileArgs& a, const TileShape& s, int phase_mode, i
   const void* fn = pick(s.lane_R, phase_mode, accum, a.ngroups > 0, a.bins_out != nullptr,
                         multi_spec_of(a.M, a.ngroups, a.group_g));
   if (!fn) return cudaErrorInvalidDeviceFunction;
-  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
-  if (e != cudaSuccess) return e;
   void* params[] = {const_cast<TileArgs*>(&a)};
   return cudaLaunchKernel(fn, dim3(grid), dim3(32 * s.warps), params, s.smem, st);
 }
