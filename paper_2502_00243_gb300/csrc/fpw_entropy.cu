@@ -38,10 +38,10 @@ __device__ __forceinline__ unsigned read_count(unsigned a) {
 // (conflict-free). Anchors lie every `span` frequencies (a multiple of the
 // block's: the phases, and with them the counts, do not depend on the launch).
 // Per staged observation the block holds the exact anchor phase P_i = frac(t_i
-// f_a) and the step D_i = frac(t_i df) as 64-bit fixed point; where the block's
-// frequencies lie on the linear grid (the tile kernels' bound on the phase
-// error) frequency j past the anchor has phase P_i + j D_i (mod 2^64), else the
-// exact anchor at its own frequency.
+// f_a) and the step D_i = frac(t_i df) as 64-bit fixed point; where all of the
+// span's frequencies lie on the linear grid (the tile kernels' bound on the
+// phase error) frequency j past the anchor has phase P_i + j D_i (mod 2^64),
+// else the exact anchor at its own frequency.
 //
 // Bound by the instructions and the shared-memory pipe together, about 2.8
 // clocks per SM and 32 counts. A count is one red.shared.add: nothing comes
@@ -74,12 +74,6 @@ __global__ void __launch_bounds__(kEntThreads) entropy_dense_kernel(const double
     const unsigned long long v = (unsigned long long)__double_as_longlong(t[i]) & 0x7fffffffffffffffull;
     if (v <= 0x7ff0000000000000ull && v > tb) tb = v;
   }
-  double dev[R];  // of frequencies f0 + tid + r T (coalesced), |f - f on the line|
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int64_t k = f0 + tid + r * T;
-    dev[r] = freqs[k < nfreq ? k : nfreq - 1];
-  }
   if (tid == 0) s_df = (nfreq > 1) ? (freqs[nfreq - 1] - freqs[0]) / (double)(nfreq - 1) : 0.0;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -94,13 +88,10 @@ __global__ void __launch_bounds__(kEntThreads) entropy_dense_kernel(const double
   tb = s_tm[0];
   for (int q = 1; q < T / 32; ++q) tb = s_tm[q] > tb ? s_tm[q] : tb;
   const double tm = __longlong_as_double((long long)tb), df = s_df;
-  bool nonlin = false;
-  double x = (double)((int)(f0 - fanchor) + tid);
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    if (f0 + tid + r * T < nfreq && fabs(dev[r] - fma(x, df, fa)) * tm > kGridTolCycles) nonlin = true;
-    x += (double)T;
-  }
+  bool nonlin = false;  // of the whole span, whichever of its blocks this is
+#pragma unroll R
+  for (int j = tid; j < span; j += T)
+    if (fanchor + j < nfreq && fabs(freqs[fanchor + j] - fma((double)j, df, fa)) * tm > kGridTolCycles) nonlin = true;
   const bool lin = !__syncthreads_or(nonlin);
   const unsigned col = (unsigned)__cvta_generic_to_shared(mine);
   constexpr unsigned step = 4u * (unsigned)(T * R);
