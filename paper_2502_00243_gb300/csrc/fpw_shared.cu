@@ -639,12 +639,13 @@ __global__ void __launch_bounds__(kShThreads, 1) shared_mma_kernel(const SharedA
       const int jo = kPaired && (p & 1) ? fpm : 0;
       const double fa = a.freqs[f0 - jo];
       if (k > 0) builders_sync(kShBuilders);  // every builder is done with the previous item's sF and stage
+      // on the line, all of them or none, whichever part of them is this pass
       bool nonlin = false;
-      for (int j = tid; j < FP; j += kShBuilders) {
-        const int64_t fi = f0 + j;
+      for (int j = tid; j < 2 * fpm; j += kShBuilders) {
+        const int64_t fi = f0 - jo + j;
         const double f = fi < F ? a.freqs[fi] : 0.0;
-        sF[j] = f;
-        if (fi < F && fabs(f - fma((double)(jo + j), df, fa)) * tmax > kGridTolCycles) nonlin = true;
+        if (j >= jo && j < jo + FP) sF[j - jo] = f;
+        if (fi < F && fabs(f - fma((double)j, df, fa)) * tmax > kGridTolCycles) nonlin = true;
       }
       const bool lin = !builders_or(nonlin, kShBuilders);
       for (int64_t ch = 0; ch < nch; ++ch, ++gc) {

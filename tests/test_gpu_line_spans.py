@@ -39,3 +39,25 @@ def test_entropy(M, span, spans):
     want = oracle.phase_entropy(t, f, M)
     assert want[5] > 0.5
     assert abs(float(H[5]) - want[5]) < 1e-5
+
+
+@pytest.mark.parametrize("M", [5, 20, 50])
+@pytest.mark.parametrize("C", [64, 128, 256])
+def test_common_times(C, M):
+    import paper_2502_00243_gb300 as G
+
+    fpm = min(64, 256 // M)
+    F = 6 * fpm - 1
+    f = grid(F, 1, 2 * fpm - 1)
+    rng = np.random.default_rng([5, C, M])
+    t = np.concatenate([np.full(3, 1024.0), rng.integers(0, 1024, 60) / 7.0])
+    x, s = rng.normal(size=(C, t.size)), rng.uniform(0.1, 0.2, (C, t.size))
+    d = [torch.from_numpy(v).cuda() for v in (t, x, s, f)]
+    S = torch.zeros(C * F, dtype=torch.float64, device="cuda")
+    G.fpw_periodogram_shared(G.Context(0), None, None, *d, M, 0, None, None, S)
+    got = S.cpu().numpy().reshape(C, F)[:, 1]
+    want = np.array([oracle.fpw(t, x[c], s[c], f[1:2], M)[0] for c in range(C)])
+    on_line = np.array([oracle.fpw(t, x[c], s[c], f[1:2] + 1e-13, M)[0] for c in range(C)])
+    tol = 1e-5 * np.sum(x * x / (s * s), axis=1)
+    assert (np.abs(want - on_line) > 10.0 * tol).sum() > C // 2
+    assert (np.abs(got - want) <= tol).all()
