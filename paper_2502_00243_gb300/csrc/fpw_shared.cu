@@ -359,7 +359,10 @@ constexpr int kShIssuers = kShThreads / 32 - kShBuilderWarps;  // one per accumu
 // those of w, of the pair's 128 curves (TMEM lane = curve) at fpm frequencies,
 // so a lane reads both sums of a bin and forms S by itself. Warp w takes lanes
 // 32 (w % 4) .. + 31 and the (w / 4)-th quarter of the frequencies; 8 columns
-// per step, the next step's loads in flight.
+// per step, the next step's loads in flight. The terms are added in the order of
+// the epilogue of one group (even and odd columns of a step apart from M = 8 on,
+// a frequency in two parts where it holds that epilogue's split column), so S does
+// not depend on how a call's groups are taken.
 __device__ __forceinline__ void pair_epilogue(const SharedArgs& a, uint32_t tmem, int64_t c, int64_t f0, bool cbad, float2 scale,
                                               int warp, int lane) {
   const int M = a.M, quarter = warp & 3, seg = warp >> 2;
@@ -375,7 +378,8 @@ __device__ __forceinline__ void pair_epilogue(const SharedArgs& a, uint32_t tmem
   double* const s64 = a.S_out ? (cvalid ? a.S_out + c * F + f0 : a.scratch64 + lane * kShMaxFpm) : nullptr;
   const float nan = __int_as_float(0x7fc00000);
   const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16), tb = ta + 256u;
-  float acc0 = 0.f, acc1 = 0.f;  // even and odd columns
+  const int split = ((a.fpm * M + 15) >> 4) << 3;
+  float acc0 = 0.f, acc1 = 0.f, part = 0.f;  // even and odd columns; the sum up to the split column
   int fend = cb + M;             // where frequency jl ends (warp-uniform)
   auto term = [&](uint32_t va, uint32_t vb) {
     const float A = __uint_as_float(va) * sa, den = __uint_as_float(vb) * sw + cal;
@@ -407,28 +411,51 @@ __device__ __forceinline__ void pair_epilogue(const SharedArgs& a, uint32_t tmem
     const uint32_t cn = (uint32_t)(c0 < clast ? c0 + 8 : clast);
     tmem_ld8_issue(ta + cn, na);
     tmem_ld8_issue(tb + cn, nb);
+    if (c0 == split) {
+      part = acc0 + acc1;
+      acc0 = acc1 = 0.f;
+    }
+    auto emit = [&]() {  // frequency jl complete
+      if (jl < jmax) {
+        const float S = cbad ? nan : acc0 + acc1 + part;
+        if (s32) s32[jl] = S;
+        if (s64) s64[jl] = (double)S;
+      }
+      acc0 = acc1 = part = 0.f;
+      ++jl;
+      fend += M;
+    };
+    // (all conditions on columns are warp-uniform)
     if (c0 >= cb && fend > c0 + 8) {
+      float lo0 = term(va[0], vb[0]), lo1 = term(va[1], vb[1]);
 #pragma unroll
-      for (int u = 0; u < 8; u += 2) {
-        acc0 += term(va[u], vb[u]);
-        acc1 += term(va[u + 1], vb[u + 1]);
+      for (int u = 2; u < 8; u += 2) {
+        lo0 += term(va[u], vb[u]);
+        lo1 += term(va[u + 1], vb[u + 1]);
+      }
+      acc0 += lo0;
+      acc1 += lo1;
+    } else if (M >= 8) {  // one frequency end at most
+      float lo0 = 0.f, lo1 = 0.f, hi0 = 0.f, hi1 = 0.f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int col = c0 + u;
+        if (col >= cb && col < ce) (u & 1 ? (col < fend ? lo1 : hi1) : (col < fend ? lo0 : hi0)) += term(va[u], vb[u]);
+      }
+      acc0 += lo0;
+      acc1 += lo1;
+      if (fend <= c0 + 8 && fend <= ce) {
+        emit();
+        acc0 = hi0;
+        acc1 = hi1;
       }
     } else {
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int col = c0 + u;
-        if (col >= cb && col < ce) {  // warp-uniform, as all conditions on columns
-          (u & 1 ? acc1 : acc0) += term(va[u], vb[u]);
-          if (col + 1 == fend) {  // frequency jl complete
-            if (jl < jmax) {
-              const float S = cbad ? nan : acc0 + acc1;
-              if (s32) s32[jl] = S;
-              if (s64) s64[jl] = (double)S;
-            }
-            acc0 = acc1 = 0.f;
-            ++jl;
-            fend += M;
-          }
+        if (col >= cb && col < ce) {
+          acc0 += term(va[u], vb[u]);
+          if (col + 1 == fend) emit();
         }
       }
     }
