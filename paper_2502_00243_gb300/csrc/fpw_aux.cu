@@ -495,7 +495,13 @@ cudaError_t launch_prep(const PrepArgs& a, cudaStream_t st) {
 cudaError_t launch_merge(const MergeArgs& a, cudaStream_t st) {
   if (a.ncurves <= 0 || a.k <= 0) return cudaSuccess;
   const unsigned groups = a.ngroups > 1 ? (unsigned)a.ngroups : 1u;
-  if ((int64_t)a.max_rows * a.k > 512) {  // long curves: a block per curve
+  // A block per curve where that is over sooner, in microseconds as measured on 152
+  // SMs: a block fills an SM and takes 5 + k; the curves' warps run at once, k
+  // rounds through the longest one's candidates. 20 curves, k = 5, 100 rows: 10
+  // against 33; 304 curves, 80 rows: 19 against 27; 608 curves, 45 rows: 35 against
+  // 18; 4000 curves, k = 20: 660 against 140; k = 64 2000 against 800.
+  const int64_t rounds = ((a.ncurves * groups) + 151) / 152, entries = (int64_t)a.max_rows * a.k;
+  if (rounds * (5 + a.k) < 5 + a.k + a.k * entries / 90) {
     const int64_t blocks = a.ncurves < 65535 ? a.ncurves : 65535;
     merge_block_kernel<<<dim3((unsigned)blocks, groups), kMergeBlock, 0, st>>>(a);
     return cudaGetLastError();

@@ -127,7 +127,7 @@ struct MergeArgs {          // ngroups groups: rows of group g at + g * group_ro
   float* topk_S;
   int out_stride;
   int32_t* topk_off;         // several-M: receives key & 63 (the bin offset); topk_idx then gets key >> 6
-  int max_rows;              // most candidate rows of one curve (0: unknown); many rows take a block per curve
+  int max_rows;              // most candidate rows of one curve: chooses a block or a warp per curve
   int ngroups;               // 0 = 1
   int64_t group_rows;
 };
