@@ -47,10 +47,14 @@ SWEEP_MS = (10, 20, 50)  # bin counts of the throughput sweep
 ENTROPY_INST_PER_EVAL = 6.94  # thread instructions per evaluation of the dense phase-entropy kernel (ncu, M = 20)
 
 
-def entropy_R(M: int) -> int:
-    """Frequencies per thread of the dense phase-entropy kernel at M bins (the
-    library's launch rule)."""
-    return 8 if M <= 12 else (4 if M <= 24 else (2 if M <= 96 else 1))
+def entropy_R(M: int, nfreq: int, nsm: int = NSM_NOMINAL) -> int:
+    """Frequencies per thread of the dense phase-entropy kernel at M bins and nfreq
+    frequencies (the library's launch rule: fewer while the grid would leave under
+    two blocks per SM, under one from two on)."""
+    R = 8 if M <= 12 else (4 if M <= 24 else (2 if M <= 96 else 1))
+    while R > 1 and -(-nfreq // (128 * R)) < (2 if R > 2 else 1) * nsm:
+        R //= 2
+    return R
 # DRAM bytes (read + write) of one tile-kernel launch at M = 20, from an ncu capture of a 1e4-curve sweep
 # batch over 2e4 frequencies (dram__bytes_read.sum + dram__bytes_write.sum). The kernel reads each curve
 # from DRAM once per launch (its phase records and weights, about 33 B per observation; per-tile
@@ -798,7 +802,7 @@ def run_configs_entropy(ctx, peak):
         # 4 B per lane (one wavefront each) plus the staged 16-byte record read
         # by every lane (two wavefronts), over 32 R evaluations; the kernel's
         # frequencies per thread R follow M
-        R = entropy_R(M)
+        R = entropy_R(M, w.nfreq)
         smem_roof = peak / SMEM_EVALS_PER_CLK_SM * (32.0 * R / (R + 2.0))
         issue_roof = peak / SMEM_EVALS_PER_CLK_SM * 128.0 / ENTROPY_INST_PER_EVAL
         terms = {"smem": smem_roof}

@@ -148,7 +148,13 @@ FPW_API int fpw_periodogram_batch(const int64_t* offsets, int64_t ncurves, const
  *   S_out:        optional device float64[ncurves * nfreq] dense periodograms (NULL: not written)
  *   topk_idx/topk_S may be NULL when k == 0.
  * With params->phase_mode == FPW_PHASE_FP64 the plain binary64 form runs:
- * one launch per curve, binary64 phases and sums (M <= 100, else FPW_ENOTSUP). */
+ * one launch per curve, binary64 phases and sums (M <= 100, else FPW_ENOTSUP).
+ * Else a curve's S and peaks at given threads and freqs_per_thread (0: chosen by M
+ * and the batch's typical curve size) do not depend on the other curves, on which
+ * outputs are asked for or on how the launch cuts the work. Device memory held by
+ * the context: 28 bytes per observation (36 for binary64 or compensated sums), 9
+ * per curve, and 32 + 12 k per work item (at most one per 32 frequencies of a
+ * curve). */
 FPW_API int fpw_periodogram_batch_ex(fpw_ctx* ctx, void* stream, const fpw_params* params, const int64_t* offsets,
                              const int64_t* offsets_host, int64_t ncurves, const double* t, const double* x,
                              const double* sigma, const double* freqs, int64_t nfreq, int M, int k,
@@ -307,8 +313,8 @@ FPW_API int fpw_periodogram_batch_noalloc(void* stream, const fpw_params* params
 
 /* Tuned kernel shapes. Adds a shape -- threads per block (multiple of 32,
  * 32..512), frequencies per thread (1, 2, 3, 4, 5, 6 or 8), observations per
- * pass (0 = largest that keeps two blocks per SM) and work items per resident
- * block (0 = 8; see fpw_params.items_per_slot) -- used for batched and single
+ * pass (0 or >= 32; see fpw_params.obs_chunk) and work items per resident
+ * warp (0 = 8; see fpw_params.items_per_slot) -- used for batched and single
  * calls whose bin count lies in [M_lo, M_hi] and whose observation-weighted
  * mean curve size lies in [n_lo, n_hi). Later entries take precedence; explicit
  * fpw_params fields override the table. An entry's 3, 5 or 6 frequencies per
@@ -324,8 +330,10 @@ FPW_API int fpw_ctx_clear_shapes(fpw_ctx* ctx);
  * call that ran the tile kernel: threads per block, frequencies per thread and
  * observations per pass of the shape that placed its phase anchors, and the
  * persistent grid (blocks). All zero
- * before the first such call. Pass the first three as fpw_params threads /
- * freqs_per_thread / obs_chunk to launch another call with the same tiles.
+ * before the first such call. Passing the first three as fpw_params threads /
+ * freqs_per_thread / obs_chunk gives another call the same phase anchors, and with
+ * them the same bins and S; it then launches that shape too, where 0 lets the
+ * library choose one by the call's size.
  * Errors: FPW_EINVAL (null pointer). */
 FPW_API int fpw_ctx_last_shape(fpw_ctx* ctx, int* threads, int* freqs_per_thread, int* obs_chunk, int* grid);
 

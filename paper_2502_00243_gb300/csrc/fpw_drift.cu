@@ -23,11 +23,12 @@
 // = beta is constant, so Q_m0 = beta Bw_m needs no sum of its own: a bin holds
 // z, Bw and Q_m1..Q_m(K-1), 1 + max(K, 1) floats; the row of H and the entry of
 // v that belong to B_0 take closed forms in the bin sums.
-// The sums accumulate in FP32 in thread-private shared-memory bins (one thread
-// per frequency, packed as float2 / float4 / float4 + float), phases are the
-// exact 64-bit anchors of the tile kernels stepped across a tile of
+// The sums accumulate in FP32 in thread-private shared-memory bins (one, two or
+// four frequencies per thread, packed as float2 / float4 / float4 + float), phases
+// are the exact 64-bit anchors of the tile kernels stepped across a span of
 // frequencies; the per-frequency reduction (one reciprocal per bin, the lower
-// triangle of the symmetric H) and the K x K Cholesky solve run in binary64.
+// triangle of the symmetric H) and the K x K Cholesky solve run in FP32 pairs, or
+// in binary64 for curves outside the pairs' range.
 #include <math.h>
 
 #include <type_traits>
@@ -258,8 +259,10 @@ __global__ void __launch_bounds__(kDrPrep) drift_prep_kernel(const DriftArgs a) 
   // bin sums are z_m = Y_m - Q_m . g itself, so a drift far above the noise
   // does not cancel inside FP32 sums of w x.
   // The pair reduction's range: H0 with a trace of at most 2^25, which bounds
-  // its condition (a pair's 2^-46 then costs S under 1e-7 where the FP32 bins
-  // leave it no digit; measured 2e-11 with beta = 1 and weights to 1e4); with
+  // its condition: a pair's 2^-46 then costs S up to 5e-7, where 2^-24 of the FP32
+  // bins leaves it no digit (against 64 bits, K = 0-4, beta = 1, 3 and 30, 20-3000
+  // observations: the largest, mean and RMS error of S are those of a binary64
+  // reduction to five digits, 1e-7 RMS with beta = 1); with
   // weights in [2^-30, 2^30], residuals at most 2^30 and not all below 2^-25,
   // beta <= 2^20, 1/alpha^2 zero or in [2^-60, 2^30] and under 2^20
   // observations, no product leaves FP32 and none that matters loses its low part.
@@ -526,8 +529,8 @@ __device__ __noinline__ double drift_reduce(const DriftArgs& a, const unsigned c
 // thread. Bins thread-private (bank = lane), [R][M][T] slots of
 // drift_bin_bytes(K): one packed read-modify-write per evaluation for K <= 3
 // (two for K = 4). The slots of the next observation are formed while this
-// one's bins are loaded. Anchors lie every a.span frequencies, a multiple of
-// the block's: phases do not depend on how the span is divided among blocks.
+// one's bins are loaded. An anchor per a.span frequencies, which one block holds
+// as T threads of R: phases do not depend on how the span is divided.
 //
 // Bound by shared memory: 8 passes per 16-byte update of a warp and 4 / R for
 // the staged record. With one frequency per thread, two observations per trip

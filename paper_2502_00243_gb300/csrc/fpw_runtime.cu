@@ -130,7 +130,6 @@ struct fpw_ctx {
   int device = 0;
   int nsm = 0;
   int smem_optin = 0;
-  int smem_per_sm = 0;
   std::mutex mu;
   cudaStream_t last_stream = nullptr;
   const unsigned* call_status = nullptr;  // device: status word of the latest call
@@ -903,7 +902,6 @@ int fpw_ctx_create(fpw_ctx** out, int device) {
   if (e == cudaSuccess) {
     ctx->nsm = prop.multiProcessorCount;
     ctx->smem_optin = (int)prop.sharedMemPerBlockOptin;
-    ctx->smem_per_sm = (int)prop.sharedMemPerMultiprocessor;
   }
   if (e == cudaSuccess) e = plain_init_attributes(ctx->smem_optin);
   if (e == cudaSuccess && (size_t)ctx->smem_optin >= shared_smem_bytes()) e = shared_init_attributes();

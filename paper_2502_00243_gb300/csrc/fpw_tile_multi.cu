@@ -1,8 +1,8 @@
 // Instantiations of the several-M tile kernel (Section 3.4; fpw_tile.cuh): the
 // generic combination for every R and phase mode, and the compiled
-// combinations (multi_spec_of) at the frequencies per thread their bin counts
-// take by default (M_max = 60: R = 1, 40: R = 2, 20: R = 4) with the fixed64
-// phase. Other (R, phase) pairs of a compiled spec run the generic kernel.
+// combinations (multi_spec_of) at the frequencies per lane their bin counts
+// take by default (M_max = 60 and 40: R = 2, 20: R = 4, or 2 in short calls) with
+// the fixed64 phase. Other (R, phase) pairs of a compiled spec run the generic one.
 #include "fpw_tile.cuh"
 
 namespace fpw {
