@@ -84,8 +84,9 @@ typedef struct fpw_params {
   int accum;            /* FPW_ACCUM_* (default FPW_ACCUM_FP32) */
   int K;                /* FPW_PHASE_FP32 only: re-anchor interval in frequencies (default 256) */
   int peak_mode;        /* FPW_PEAK_* (default FPW_PEAK_LOCALMAX) */
-  int threads;          /* 0 = tuned; else threads per block (multiple of 32, 32..512); with freqs_per_thread it also places
-                           the phase anchors, threads * freqs_per_thread - 2 frequencies apart */
+  int threads;          /* 0 = tuned; else threads per block (multiple of 32, 32..512; other blocks are launched where
+                           these leave part of an SM unused); with freqs_per_thread it also places the phase anchors,
+                           threads * freqs_per_thread - 2 frequencies apart */
   int freqs_per_thread; /* 0 = tuned; else 1, 2, 4 or 8, or 3, 5 or 6 with FPW_ACCUM_FP32 on a call of one M
                            (FPW_ENOTSUP on the other calls) */
   int obs_chunk;        /* 0 = tuned; else observations per pass (>= 32): counts towards the shape's size

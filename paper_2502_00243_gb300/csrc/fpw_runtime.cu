@@ -279,7 +279,15 @@ int choose_shape(fpw_ctx* ctx, const fpw_params& p, int M, int k, int64_t C, int
 
   const auto fit = [&](int r) { return (int)(limit / tile_smem_bytes(32, r, M, k, p.accum, ngroups)); };
   int r = R, w = T / 32;
-  if (!given) {
+  if (given) {
+    // Warps share nothing, so their blocks may have another size than T where blocks
+    // of T leave an SM's registers (tile_max_warps) or shared memory unused: 12
+    // warps an SM up to four frequencies a lane, 8 beyond (300 ragged curves x
+    // 20000 frequencies, M = 20, T = 256: R = 1 5950 us in blocks of 8 warps, 5070 in
+    // one of 12, R = 2 4060 and 3785, R = 4 on 8 3340, on 10 3240).
+    const int most = std::min(fit(r), tile_max_warps(multi)), want = std::min(most, r <= 4 ? 12 : 8);
+    if (most / w * w < want) w = want;
+  } else {
     r = wide ? 2 : M <= 12 ? 8 : M <= 16 && !multi ? 6 : M <= 20 ? 5 : M <= 25 ? 4 : M <= 33 ? 3 : M <= 50 ? 2 : M <= 64 ? 3 : 1;
     if (multi && M > 50 && M <= 64) r = 2;
     w = wide ? 12 : 8;
