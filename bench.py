@@ -55,12 +55,14 @@ def entropy_R(M: int, nfreq: int, nsm: int = NSM_NOMINAL) -> int:
     while R > 1 and -(-nfreq // (128 * R)) < (2 if R > 2 else 1) * nsm:
         R //= 2
     return R
-# DRAM bytes (read + write) of one tile-kernel launch at M = 20, from an ncu capture of a 1e4-curve sweep
-# batch over 2e4 frequencies (dram__bytes_read.sum + dram__bytes_write.sum). The kernel reads each curve
-# from DRAM once per launch (its phase records and weights, about 33 B per observation; per-tile
-# re-reads hit L2), so a full launch adds only the larger grid (8 B per extra frequency). Valid only for the
-# kernel source it was measured on (sha256 prefix of the tile-kernel sources, tile_source_hash).
-TILE_TRAFFIC = {"source_sha256_16": "9a63431f73948b4e", "bytes": 283.59e6, "nfreq": 20_000}
+
+
+# DRAM bytes (read + write) of one tile-kernel launch at M = 20, from ncu captures of a 1e4-curve sweep
+# batch over 2e4 and 6e4 frequencies (dram__bytes_read.sum + dram__bytes_write.sum: 786 and 1744 MB). A tile
+# reads its curve's records and weights again (28 B per observation); while the warps' curves are long they
+# do not all stay in L2, so a launch adds 23.9 kB per extra frequency. Valid only for the kernel source it
+# was measured on (sha256 prefix of the tile-kernel sources, tile_source_hash).
+TILE_TRAFFIC = {"source_sha256_16": "d27e02034516af6f", "bytes": 786.18e6, "nfreq": 20_000, "per_freq": 23.94e3}
 
 
 # ---------------------------------------------------------------- workload generation (spawned workers)
@@ -233,7 +235,7 @@ def tile_traffic(nfreq):
     kernel source changed since the counters were taken."""
     if TILE_TRAFFIC["bytes"] is None or tile_source_hash() != TILE_TRAFFIC["source_sha256_16"]:
         return None
-    return TILE_TRAFFIC["bytes"] + 8.0 * (nfreq - TILE_TRAFFIC["nfreq"])
+    return TILE_TRAFFIC["bytes"] + TILE_TRAFFIC["per_freq"] * (nfreq - TILE_TRAFFIC["nfreq"])
 
 
 def grid(args):
