@@ -362,7 +362,8 @@ constexpr int kShIssuers = kShThreads / 32 - kShBuilderWarps;  // one per accumu
 // per step, the next step's loads in flight. The terms are added in the order of
 // the epilogue of one group (even and odd columns of a step apart from M = 8 on,
 // a frequency in two parts where it holds that epilogue's split column), so S does
-// not depend on how a call's groups are taken.
+// not depend on how a call's groups are taken (512 curves x 1000 times x 50000
+// frequencies, M = 20: 3050 us a call, 3037 with an order of its own).
 __device__ __forceinline__ void pair_epilogue(const SharedArgs& a, uint32_t tmem, int64_t c, int64_t f0, bool cbad, float2 scale,
                                               int warp, int lane) {
   const int M = a.M, quarter = warp & 3, seg = warp >> 2;
